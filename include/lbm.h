@@ -214,6 +214,13 @@ size_t lbm_fields_bytes(const lbm_handle* h, uint32_t fields);
 int lbm_read_fields(lbm_handle* h, uint32_t fields, void* dst, size_t dst_bytes,
                     int dst_is_device);
 
+/* The same with a destination of its own for each selected field: dsts[k]
+ * takes the k-th selected field in increasing bit order (host pointers, or
+ * device pointers with dst_is_device = 1; a float or int32 field needs 4-byte
+ * alignment). RHO, UX, UY and P selected together come from one pass over the
+ * populations. Synchronises. */
+int lbm_read_fields_each(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_device);
+
 /* FP64 sum of rho over the box (of both components with two), reduced in
  * a fixed order. Synchronises. */
 int lbm_mass(lbm_handle* h, double* out);

@@ -24,6 +24,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
+inline size_t align8(size_t v) { return (v + 7) / 8 * 8; }
 
 
 
@@ -264,6 +265,77 @@ size_t field_bytes(const lbm_handle* h, uint32_t bit) {
 
 constexpr uint32_t kLastField = LBM_FIELD_RHO_GAS;
 constexpr uint32_t kAllFields = (kLastField << 1) - 1;
+constexpr int kFieldCount = 10;
+
+// The selected fields (increasing bit order) into dsts. rho, u and p come
+// from one pass over the populations; nothing is computed that was not
+// selected. Host destinations are staged in the idle population buffer
+// (18 bytes per cell at least: rho, u and p take 16).
+int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_device) {
+  int rc = select_device(h);
+  if (rc) return rc;
+  const FieldParams fp = field_params(h);
+  const size_t N = h->N();
+  char* stage = static_cast<char*>(h->pops(1 - h->cur));
+  const cudaMemcpyKind d2x = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+  void* dst[kFieldCount] = {};  // by bit index
+  int n = 0;
+  for (int b = 0; b < kFieldCount; ++b)
+    if (fields & (1u << b)) dst[b] = dsts[n++];
+  constexpr uint32_t kFloat = LBM_FIELD_RHO | LBM_FIELD_UX | LBM_FIELD_UY | LBM_FIELD_P;
+  if (fields & (kFloat | (h->comps() == 2 ? (uint32_t)LBM_FIELD_RHO_GAS : 0u))) {
+    const int bits[5] = {0, 1, 2, 3, 9};  // rho, ux, uy, p, gas density
+    float* f[5] = {};
+    for (int k = 0; k < 5; ++k)
+      if (dst[bits[k]]) f[k] = static_cast<float*>(dst_is_device ? dst[bits[k]] : static_cast<void*>(stage + 4 * N * k));
+    if (h->comps() == 2) {  // 144 bytes per cell of staging
+      CUDA_TRY(h, launch_fields2(step2_params(h), f[0], f[4], f[1], f[2], f[3], h->stream));
+    } else {
+      CUDA_TRY(h, launch_fields(fp, h->mask(), FieldOuts{f[0], f[1], f[2], f[3]}, h->stream));
+    }
+    if (!dst_is_device)
+      for (int k = 0; k < (h->comps() == 2 ? 5 : 4); ++k)
+        if (dst[bits[k]]) CUDA_TRY(h, cudaMemcpyAsync(dst[bits[k]], f[k], 4 * N, d2x, h->stream));
+  }
+  if (dst[9] && h->comps() != 2) {
+    if (dst_is_device) CUDA_TRY(h, cudaMemsetAsync(dst[9], 0, 4 * N, h->stream));
+    else memset(dst[9], 0, 4 * N);
+  }
+  if (dst[4]) {
+    // into scratch: the relabel pipeline's own labels stay those of the
+    // last relabel (the coalescence count compares the next one with them)
+    int32_t* lab = static_cast<int32_t*>(dst_is_device ? dst[4] : static_cast<void*>(stage));
+    CUDA_TRY(h, launch_diag_labels(fp, (float)h->cfg.gas_threshold, lab, stage + align8(4 * N), h->flags(), h->stream));
+    if (!dst_is_device) CUDA_TRY(h, cudaMemcpyAsync(dst[4], lab, 4 * N, d2x, h->stream));
+  }
+  const void* state[3] = {h->owner(), h->mask(), h->open()};
+  for (int b = 5; b <= 7; ++b) {
+    if (!dst[b]) continue;
+    const size_t nb = b == 5 ? 4 * N : N;
+    const int fill = b == 5 ? 0xff : 0;
+    if (state[b - 5]) CUDA_TRY(h, cudaMemcpyAsync(dst[b], state[b - 5], nb, d2x, h->stream));
+    else if (dst_is_device) CUDA_TRY(h, cudaMemsetAsync(dst[b], fill, nb, h->stream));
+    else memset(dst[b], fill, nb);
+  }
+  if (dst[8]) {
+    char* out = static_cast<char*>(dst[8]);
+    for (int k = 0; k < h->comps(); ++k, out += 4 * Q * N) {
+      FieldParams fk = fp;
+      fk.pops = component_pops(h, h->cur, k);
+      if (dst_is_device) {
+        CUDA_TRY(h, launch_pops_out(fk, 0, Q, reinterpret_cast<float*>(out), h->stream));
+        continue;
+      }
+      const int group = h->cfg.storage == LBM_F32 ? Q : 4;  // planes the staging area holds
+      for (int p0 = 0; p0 < Q; p0 += group) {
+        const int m = Q - p0 < group ? Q - p0 : group;
+        CUDA_TRY(h, launch_pops_out(fk, p0, m, reinterpret_cast<float*>(stage), h->stream));
+        CUDA_TRY(h, cudaMemcpyAsync(out + 4 * N * p0, stage, 4 * N * m, d2x, h->stream));
+      }
+    }
+  }
+  return check_flags(h);
+}
 
 }  // namespace
 
@@ -556,77 +628,24 @@ int lbm_read_fields(lbm_handle* h, uint32_t fields, void* dst, size_t dst_bytes,
   if (!h) return LBM_EINVAL;
   if (!dst || fields == 0 || (fields & ~kAllFields)) return fail(h, LBM_EINVAL, "bad field selection");
   if (dst_bytes < lbm_fields_bytes(h, fields)) return fail(h, LBM_EINVAL, "dst too small");
-  int rc = select_device(h);
-  if (rc) return rc;
-  const FieldParams fp = field_params(h);
-  const size_t N = h->N();
+  void* dsts[kFieldCount] = {};
   char* out = static_cast<char*>(dst);
-  float* stage = static_cast<float*>(h->pops(1 - h->cur));
-  const cudaMemcpyKind d2x = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  CUDA_TRY(h, launch_density(fp, h->rho(), h->stream));
-  for (uint32_t bit = 1; bit <= kLastField; bit <<= 1) {
-    if (!(fields & bit)) continue;
-    const size_t nb = field_bytes(h, bit);
-    switch (bit) {
-      case LBM_FIELD_RHO:
-      case LBM_FIELD_UX:
-      case LBM_FIELD_UY:
-      case LBM_FIELD_P:
-      case LBM_FIELD_RHO_GAS: {
-        float* target = dst_is_device ? reinterpret_cast<float*>(out) : stage;
-        if (h->comps() == 2) {
-          const Step2Params q = step2_params(h);
-          CUDA_TRY(h, launch_fields2(q, bit == LBM_FIELD_RHO ? target : nullptr,
-                                     bit == LBM_FIELD_RHO_GAS ? target : nullptr, bit == LBM_FIELD_UX ? target : nullptr,
-                                     bit == LBM_FIELD_UY ? target : nullptr, bit == LBM_FIELD_P ? target : nullptr,
-                                     h->stream));
-        } else if (bit == LBM_FIELD_RHO_GAS) {
-          CUDA_TRY(h, cudaMemsetAsync(target, 0, nb, h->stream));
-        } else {
-          CUDA_TRY(h, launch_fields(fp, h->rho(), h->mask(), bit, target, h->stream));
-        }
-        if (!dst_is_device) CUDA_TRY(h, cudaMemcpyAsync(out, stage, nb, d2x, h->stream));
-        break;
-      }
-      case LBM_FIELD_LABEL: {
-        // into scratch: the relabel pipeline's own labels stay those of the
-        // last relabel (the coalescence count compares the next one with them)
-        int32_t* lab = dst_is_device ? reinterpret_cast<int32_t*>(out) : reinterpret_cast<int32_t*>(stage);
-        CUDA_TRY(h, launch_labels(fp, h->rho(), (float)h->cfg.gas_threshold, lab, h->flags(), h->stream));
-        if (!dst_is_device) CUDA_TRY(h, cudaMemcpyAsync(out, stage, nb, d2x, h->stream));
-        break;
-      }
-      case LBM_FIELD_OWNER:
-      case LBM_FIELD_MASK:
-      case LBM_FIELD_OPEN: {
-        const void* srcp = bit == LBM_FIELD_OWNER ? (const void*)h->owner()
-                           : bit == LBM_FIELD_MASK ? (const void*)h->mask()
-                                                   : (const void*)h->open();
-        if (srcp) {
-          CUDA_TRY(h, cudaMemcpyAsync(out, srcp, nb, d2x, h->stream));
-        } else {
-          const int fill = bit == LBM_FIELD_OWNER ? 0xff : 0;
-          if (dst_is_device)
-            CUDA_TRY(h, cudaMemsetAsync(out, fill, nb, h->stream));
-          else
-            memset(out, fill, nb);
-        }
-        break;
-      }
-      case LBM_FIELD_POPS:
-        for (int pl = 0; pl < Q * h->comps(); ++pl) {
-          FieldParams fk = fp;
-          fk.pops = component_pops(h, h->cur, pl / Q);
-          float* target = dst_is_device ? reinterpret_cast<float*>(out + 4 * N * pl) : stage;
-          CUDA_TRY(h, launch_pops_out(fk, pl % Q, target, h->stream));
-          if (!dst_is_device)
-            CUDA_TRY(h, cudaMemcpyAsync(out + 4 * N * pl, stage, 4 * N, d2x, h->stream));
-        }
-        break;
+  int n = 0;
+  for (uint32_t bit = 1; bit <= kLastField; bit <<= 1)
+    if (fields & bit) {
+      dsts[n++] = out;
+      out += field_bytes(h, bit);
     }
-    out += nb;
-  }
-  return check_flags(h);
+  return read_fields(h, fields, dsts, dst_is_device);
+}
+
+int lbm_read_fields_each(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_device) {
+  if (!h) return LBM_EINVAL;
+  if (!dsts || fields == 0 || (fields & ~kAllFields)) return fail(h, LBM_EINVAL, "bad field selection");
+  int n = 0;
+  for (uint32_t bit = 1; bit <= kLastField; bit <<= 1)
+    if ((fields & bit) && !dsts[n++]) return fail(h, LBM_EINVAL, "a selected field has no destination");
+  return read_fields(h, fields, dsts, dst_is_device);
 }
 
 int lbm_nucleate(lbm_handle* h, const lbm_bubble* nuclei, int32_t n, double rho_g) {
@@ -706,15 +725,13 @@ int lbm_bubble_stats(lbm_handle* h, lbm_stats* out, double* hist, int32_t nbins,
   int rc = select_device(h);
   if (rc) return rc;
   const FieldParams fp = field_params(h);
-  // labels and areas in the idle population buffer (>= 18 bytes per cell)
+  // labels, areas and the tiles' sums in the idle population buffer (>= 18 bytes per cell)
   int32_t* lab = static_cast<int32_t*>(h->pops(1 - h->cur));
   int32_t* area = lab + h->N();
-  CUDA_TRY(h, launch_density(fp, h->rho(), h->stream));
-  CUDA_TRY(h, launch_labels(fp, h->rho(), (float)h->cfg.gas_threshold, lab, h->flags(), h->stream));
-  CUDA_TRY(h, launch_stats(h->cfg.nx, h->cfg.ny, lab, area, h->partials(), h->L.nparts, h->scalars(),
-                           h->flags() + FLAG_HIST, hist ? nbins : 0, hist ? dmin : 1.0, hist ? dmax : 2.0,
-                           h->stream));
-  double sc[3];
+  CUDA_TRY(h, launch_diag_stats(fp, (float)h->cfg.gas_threshold, lab, area, area + h->N(), h->flags(), h->partials(),
+                                h->L.nparts, h->scalars(), h->flags() + FLAG_HIST, hist ? nbins : 0, hist ? dmin : 1.0,
+                                hist ? dmax : 2.0, h->stream));
+  double sc[4];
   int hc[kMaxHistBins];
   int opened = 0, merges = 0;
   CUDA_TRY(h, cudaMemcpyAsync(sc, h->scalars(), sizeof(sc), cudaMemcpyDeviceToHost, h->stream));
@@ -724,8 +741,8 @@ int lbm_bubble_stats(lbm_handle* h, lbm_stats* out, double* hist, int32_t nbins,
   CUDA_TRY(h, cudaMemcpyAsync(&merges, h->flags() + FLAG_MERGES, sizeof(int), cudaMemcpyDeviceToHost,
                               h->stream));
   if ((rc = check_flags(h))) return rc;
-  double mass = 0.0;
-  if ((rc = lbm_mass(h, &mass))) return rc;
+  double mass = sc[3];  // of the labelled component; two lattices are summed on their own
+  if (h->comps() == 2 && (rc = lbm_mass(h, &mass))) return rc;
   memset(out, 0, sizeof(*out));
   out->step = h->t;
   out->n_bubbles = (int32_t)llround(sc[0]);
@@ -753,9 +770,8 @@ int lbm_bubble_areas(lbm_handle* h, int32_t capacity, int32_t* labels, double* a
   int32_t* area = lab + N;
   int32_t* list = area + N;
   int* count = h->flags() + FLAG_HIST;  // the histogram slots serve as scratch here
-  CUDA_TRY(h, launch_density(fp, h->rho(), h->stream));
-  CUDA_TRY(h, launch_labels(fp, h->rho(), (float)h->cfg.gas_threshold, lab, h->flags(), h->stream));
-  CUDA_TRY(h, launch_bubble_list(h->cfg.nx, h->cfg.ny, lab, area, list, count, h->stream));
+  CUDA_TRY(h, launch_diag_areas(fp, (float)h->cfg.gas_threshold, lab, area, list, count,
+                                reinterpret_cast<char*>(lab) + align8(12 * N), h->flags(), h->stream));
   int n = 0;
   CUDA_TRY(h, cudaMemcpyAsync(&n, count, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   if ((rc = check_flags(h))) return rc;

@@ -1,8 +1,7 @@
 // Film-barrier pipeline of the extended Shan-Chen model (arXiv 1708.01613,
-// Sec. 2.1.5) and the auxiliary kernels: density, gas labelling, interaction
-// zones, rupture test (Eq. 41), blocked-edge mask, the bounce-back across
-// blocked edges after each step, diagnostics fields, initialisation, FP64
-// mass and bubble statistics.
+// Sec. 2.1.5): gas labelling, interaction zones, rupture test (Eq. 41),
+// blocked-edge mask, the bounce-back across blocked edges after each step;
+// and the initialisation of a box. The diagnostics are in fields.cu.
 //
 // Readings used (the paper is silent on them):
 //  - gas cell: rho < threshold (default ln 2, the critical density of
@@ -21,13 +20,13 @@
 //    defined), neither end open.
 #include <math.h>
 
-#include "lbm_internal.cuh"
+#include "labels.cuh"
+#include "pull.cuh"
 
 namespace lbm {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kUnionIters = 1 << 20;  // bound of the union/find retry loops
 
 __device__ __forceinline__ int wrapi(int a, int n) {
   a %= n;
@@ -40,26 +39,6 @@ inline unsigned blocks_for(long long n, int threads = kThreads) {
   if (b > cap) b = cap;
   if (b < 1) b = 1;
   return (unsigned)b;
-}
-
-template <int S>
-__device__ __forceinline__ float pulled(const void* pops, const FieldParams& fp, int i, int x, int y) {
-  using T = typename Store<S>::T;
-  const T* p = static_cast<const T*>(pops);
-  const int xs = wrapi(x - cx(i), fp.nx), ys = wrapi(y - cy(i), fp.ny);
-  return Store<S>::load(p, (size_t)i * fp.N + (size_t)ys * fp.nx + xs, fp.wref[i]);
-}
-
-template <int S>
-__global__ void k_density(const FieldParams fp, float* __restrict__ rho) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < fp.N;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % fp.nx), y = (int)(c / fp.nx);
-    float f[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) f[i] = pulled<S>(fp.pops, fp, i, x, y);
-    rho[c] = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-  }
 }
 
 // --- union-find labelling (min-root hooking: the root is the min index) ---
@@ -106,35 +85,6 @@ __global__ void k_merge_count(long long N, const int32_t* __restrict__ L, int32_
     if (r >= 0 && r != c) n += merge_vote(keep, r, keep[c]);
   }
   if (n) atomicAdd(flags + FLAG_MERGES, n);
-}
-
-__device__ int find_root(const int32_t* L, int a, int* fail) {
-  for (int it = 0; it < kUnionIters; ++it) {
-    const int p = L[a];
-    if (p == a) return a;
-    a = p;
-  }
-  *fail = 1;
-  return a;
-}
-
-__device__ void unite(int32_t* L, int a, int b, int* fail) {
-  for (int it = 0; it < kUnionIters; ++it) {
-    a = find_root(L, a, fail);
-    b = find_root(L, b, fail);
-    if (a == b) return;
-    if (a < b) {
-      const int t = a;
-      a = b;
-      b = t;
-    }
-    // hook the larger root a under b; if a stopped being a root meanwhile,
-    // continue with the value it points to (links only ever decrease)
-    const int old = atomicMin(&L[a], b);
-    if (old == a) return;
-    a = old;
-  }
-  *fail = 1;
 }
 
 __global__ void k_label_union(int nx, int ny, int32_t* L, int* flags) {
@@ -323,56 +273,6 @@ __global__ void k_mask(int nx, int ny, const int32_t* __restrict__ own, const ui
   }
 }
 
-// --- diagnostics: rho, u = (j + F/2)/rho, p (Eq. 29) ---
-template <int S>
-__global__ void k_fields(const FieldParams fp, const float* __restrict__ rho,
-                         const uint8_t* __restrict__ mask, uint32_t which, float* __restrict__ out) {
-  const int nx = fp.nx, ny = fp.ny;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < fp.N;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx), y = (int)(c / nx);
-    const float r = rho[c];
-    const float psi_c = fp.rho0 * (1.0f - expf(-r * fp.inv_rho0));
-    float v = 0.f;
-    if (which == LBM_FIELD_RHO) {
-      v = r;
-    } else if (which == LBM_FIELD_P) {
-      v = r * (1.0f / 3.0f) + fp.G * psi_c * psi_c * (1.0f / 6.0f);
-    } else {
-      float f[Q];
-#pragma unroll
-      for (int i = 0; i < Q; ++i) f[i] = pulled<S>(fp.pops, fp, i, x, y);
-      const float jx = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
-      const float jy = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
-      const unsigned m = mask ? mask[c] : 0u;
-      float sx = 0.f, sy = 0.f;
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        float s = fp.rho0 * (1.0f - expf(-rho[(long long)wrapi(y + cy(i), ny) * nx + wrapi(x + cx(i), nx)] * fp.inv_rho0));
-        if ((m >> (i - 1)) & 1u) s = psi_c;
-        sx += static_cast<float>(wq(i)) * s * cx(i);
-        sy += static_cast<float>(wq(i)) * s * cy(i);
-      }
-      const float F = -fp.G * psi_c * (which == LBM_FIELD_UX ? sx : sy);
-      v = ((which == LBM_FIELD_UX ? jx : jy) + 0.5f * F) / r;
-    }
-    out[c] = v;
-  }
-}
-
-template <int S>
-__global__ void k_pops_out(const FieldParams fp, int plane, float* __restrict__ out) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < fp.N;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % fp.nx), y = (int)(c / fp.nx);
-    float v = 0.f;
-#pragma unroll
-    for (int i = 0; i < Q; ++i)
-      if (i == plane) v = pulled<S>(fp.pops, fp, i, x, y);
-    out[c] = v;
-  }
-}
-
 // The stored buffer holds f_i at the source cell of the next pull: B_i(y) = f_i(y + e_i).
 template <int S>
 __global__ void k_init_from_rho(typename Store<S>::T* __restrict__ pops, const double* __restrict__ rho,
@@ -475,110 +375,6 @@ __global__ void __launch_bounds__(kThreads) k_bubbles_rho(const lbm_bubble* __re
   }
 }
 
-// --- fixed-order FP64 reductions ---
-// A fixed number of block partials (not tied to the device's SM count), so the
-// summation order, and with it every reduced value, is the same on any GPU.
-constexpr int kRedBlocks = 608;
-
-template <int NV>
-__device__ void block_reduce_store(double (&v)[NV], double* __restrict__ out) {
-  __shared__ double sh[NV][kThreads];
-#pragma unroll
-  for (int j = 0; j < NV; ++j) sh[j][threadIdx.x] = v[j];
-  __syncthreads();
-  for (int s = kThreads / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s)
-#pragma unroll
-      for (int j = 0; j < NV; ++j) sh[j][threadIdx.x] += sh[j][threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int j = 0; j < NV; ++j) out[j * gridDim.x + blockIdx.x] = sh[j][0];
-}
-
-template <int S>
-__global__ void __launch_bounds__(kThreads) k_mass_partial(const FieldParams fp, double* partials) {
-  using T = typename Store<S>::T;
-  const T* p = static_cast<const T*>(fp.pops);
-  double acc[1] = {0.0};
-  for (int i = 0; i < Q; ++i) {
-    const float base = fp.wref[i];
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < fp.N;
-         c += (long long)gridDim.x * blockDim.x)
-      acc[0] += (double)Store<S>::load(p, (size_t)i * fp.N + c, base);
-  }
-  block_reduce_store<1>(acc, partials);
-}
-
-template <int NV>
-__global__ void __launch_bounds__(kThreads) k_sum_partials(const double* partials, int nparts, double* out) {
-  double acc[NV];
-#pragma unroll
-  for (int j = 0; j < NV; ++j) acc[j] = 0.0;
-  for (int k = threadIdx.x; k < nparts; k += blockDim.x)
-#pragma unroll
-    for (int j = 0; j < NV; ++j) acc[j] += partials[j * nparts + k];
-  block_reduce_store<NV>(acc, out);
-}
-
-__global__ void k_area(long long N, const int32_t* __restrict__ L, int32_t* __restrict__ area) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int l = L[c];
-    if (l >= 0) atomicAdd(area + l, 1);
-  }
-}
-
-// Roots with their areas appended to list (warp-aggregated slots).
-__global__ void k_bubble_list(long long N, const int32_t* __restrict__ L, const int32_t* __restrict__ area,
-                              int32_t* __restrict__ list, int* count) {
-  for (long long c0 = blockIdx.x * (long long)blockDim.x; c0 < N; c0 += (long long)gridDim.x * blockDim.x) {
-    const long long c = c0 + threadIdx.x;
-    const bool root = c < N && L[c] == c;
-    const unsigned b = __ballot_sync(0xffffffffu, root);
-    if (!b) continue;
-    const int lane = threadIdx.x & 31;
-    int base = 0;
-    if (lane == __ffs(b) - 1) base = atomicAdd(count, __popc(b));
-    base = __shfl_sync(0xffffffffu, base, __ffs(b) - 1);
-    if (root) {
-      const int k = base + __popc(b & ((1u << lane) - 1u));
-      list[2 * k] = (int32_t)c;
-      list[2 * k + 1] = area[c];
-    }
-  }
-}
-
-// partial sums: [0] bubbles, [1] gas cells, [2] sum of equivalent diameters;
-// histogram counts are integers, accumulated exactly with atomics
-constexpr int kMaxBins = 64;
-constexpr int kStatVals = 3;
-
-__global__ void __launch_bounds__(kThreads) k_stats_partial(long long N, const int32_t* __restrict__ L,
-                                                            const int32_t* __restrict__ area, int nbins,
-                                                            double ldmin, double ldspan, double* partials,
-                                                            int* hist) {
-  double v[kStatVals] = {0.0, 0.0, 0.0};
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int l = L[c];
-    if (l < 0) continue;
-    v[1] += 1.0;
-    if (l == c) {
-      const double d = 2.0 * sqrt((double)area[c] / M_PI);
-      v[0] += 1.0;
-      v[2] += d;
-      if (nbins > 0) {
-        int b = (int)floor((log(d) - ldmin) / ldspan * nbins);
-        b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
-        atomicAdd(hist + b, 1);
-      }
-    }
-  }
-  block_reduce_store<kStatVals>(v, partials);
-}
-
 // ---------------------------------------------------------------------------
 // Tiled barrier pipeline. The box is cut into 32 x 8 tiles; where nx or ny is
 // not a multiple of the tile, the last tile column or row is ragged and its
@@ -595,7 +391,6 @@ __global__ void __launch_bounds__(kThreads) k_stats_partial(long long N, const i
 // Every phase is one launch over any number of boxes (a lone box is a list
 // of one): each box's CTAs follow those of the boxes before it in the entry
 // list (RelabelEntry prefix sums), and a CTA finds its box by binary search.
-constexpr int kTX = kRelabelTileX, kTY = kRelabelTileY;
 // Mask bits of the directions 1, 2, 5, 6: each blocked edge is seen from the
 // one end where its direction is among these.
 constexpr unsigned kCanonBits = 0x33u;
@@ -626,43 +421,6 @@ __device__ __forceinline__ int find_entry(const RelabelEntry* __restrict__ e, in
 // One cell per thread. Used for two-component boxes (TWO, FP32), which also
 // get the mixture pressure; one-component boxes take the four-cell kernels
 // below, whose per-cell arithmetic is this kernel's.
-// Union-find inside one 32 x 8 tile in shared memory (local indices
-// ly * kTX + lx, -1 for liquid), hooking the larger root under the smaller,
-// so a root is the smallest local index of its piece. Bounded like the
-// global version.
-__device__ __forceinline__ int tile_find(const int* sp, int a, int* fail) {
-  for (int it = 0; it < kTX * kTY; ++it) {
-    const int p = sp[a];
-    if (p == a) return a;
-    a = p;
-  }
-  *fail = 1;
-  return a;
-}
-
-__device__ __forceinline__ void tile_unite(int* sp, int a, int b, int* fail) {
-  for (int it = 0; it < kTX * kTY; ++it) {
-    a = tile_find(sp, a, fail);
-    b = tile_find(sp, b, fail);
-    if (a == b) return;
-    if (a < b) {
-      const int t = a;
-      a = b;
-      b = t;
-    }
-    const int old = atomicMin(&sp[a], b);
-    if (old == a) return;
-    a = old;
-  }
-  *fail = 1;
-}
-
-// Global index of the tile-local root of local cell li (a gas cell).
-__device__ __forceinline__ int32_t tile_root_index(const int* sp, int li, int x0, int y0, int nx, int* fail) {
-  const int r = tile_find(sp, li, fail);
-  return (int32_t)((y0 + r / kTX) * nx + x0 + r % kTX);
-}
-
 template <int S, bool TWO>
 __global__ void __launch_bounds__(kTX * kTY) kb_density_label(const RelabelBox* __restrict__ boxes,
                                                               const RelabelEntry* __restrict__ e, int m, int parity) {
@@ -733,12 +491,6 @@ __global__ void __launch_bounds__(kTX * kTY) kb_density_label(const RelabelBox* 
   }
 }
 
-template <int S>
-__device__ __forceinline__ float dec16(unsigned short v) {
-  if constexpr (S == LBM_F16_DEV) return __half2float(__ushort_as_half(v));
-  else return __bfloat162float(__ushort_as_bfloat16(v));
-}
-
 // Four cells (x .. x + 3) of one tile row per thread, 8 x 8 threads per
 // 32 x 8 tile: the part after the densities r, shared by the vector density
 // kernels. Densities out, gas decision (rho < threshold), tile-local
@@ -763,27 +515,8 @@ __device__ __forceinline__ void density_label_tail4(const RelabelBox& B, int t, 
     for (int j = 0; j < 4; ++j)
       if (in[j]) rho[c + j] = r[j];
   }
-  __shared__ int sp[kTX * kTY];  // tile-local union-find, as in kb_density_label
-  const int la = threadIdx.y * kTX + 4 * threadIdx.x;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) sp[la + j] = gas[j] ? la + j : -1;
-  const int any = __syncthreads_or(gas[0] || gas[1] || gas[2] || gas[3]);
-  int32_t lab[4] = {-1, -1, -1, -1};
-  if (any) {
-    int fail = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (!gas[j]) continue;
-      if (j < 3 ? gas[j + 1] : (4 * threadIdx.x + 4 < kTX && sp[la + 4] >= 0)) tile_unite(sp, la + j, la + j + 1, &fail);
-      if (threadIdx.y + 1 < kTY && sp[la + j + kTX] >= 0) tile_unite(sp, la + j, la + j + kTX, &fail);
-    }
-    __syncthreads();
-    const int x0 = x - 4 * threadIdx.x, y0 = y - threadIdx.y;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (gas[j]) lab[j] = tile_root_index(sp, la + j, x0, y0, B.nx, &fail);
-    if (fail) atomicOr(B.flags + FLAG_TIMEOUT, 1);
-  }
+  int32_t lab[4];
+  const int any = tile_labels4(gas, x, y, B.nx, lab, B.flags);
 #pragma unroll
   for (int j = 0; j < 4; ++j)
     if (gas[j]) {  // the label of the previous relabel, for the coalescence count
@@ -806,138 +539,27 @@ __device__ __forceinline__ void density_label_tail4(const RelabelBox& B, int t, 
   }
 }
 
-// Sum of the nine pulled values in kb_density_label's order, for two cells
-// at once (the packed adds round per component like the scalar ones).
-__device__ __forceinline__ float2 rho_pair(const float2 (&f)[Q]) {
-  return __fadd2_rn(__fadd2_rn(__fadd2_rn(__fadd2_rn(f[0], f[1]), __fadd2_rn(f[2], f[3])),
-                               __fadd2_rn(__fadd2_rn(f[4], f[5]), __fadd2_rn(f[6], f[7]))),
-                    f[8]);
-}
-
-// One-component FP32 storage, four cells per thread. Where the box's rows
-// start on 16-byte boundaries (nx % 4 == 0) and the cells and the columns
-// they pull from lie inside the row, a plane arrives in one 16-byte load, a
-// plane the pull shifts by one column adds the value beside it; other cells
-// (the box's first and last columns, ragged tiles, other widths) load one by
-// one with the periodic wrap.
-__global__ void __launch_bounds__(kTX / 4 * kTY, 16) kb_density_label32(const RelabelBox* __restrict__ boxes,
-                                                                        const RelabelEntry* __restrict__ e, int m,
-                                                                        int parity) {
+// One component, four cells per thread (pull4): each cell's arithmetic is
+// kb_density_label's, so densities, labels and tile flags are bitwise the same.
+template <int S>
+__global__ void __launch_bounds__(kTX / 4 * kTY, 16) kb_density_label4(const RelabelBox* __restrict__ boxes,
+                                                                       const RelabelEntry* __restrict__ e, int m,
+                                                                       int parity) {
+  using T = typename Store<S>::T;
   const int k = find_entry<kOffTiles>(e, m, blockIdx.x);
   const RelabelBox& B = boxes[e[k].box];
   const int t = blockIdx.x - e[k].off_tiles;
-  const float* p = static_cast<const float*>(B.pops[B.cur ^ parity]);
+  const T* p = static_cast<const T*>(B.pops[B.cur ^ parity]);
   const int nx = B.nx, ny = B.ny;
-  const size_t N = (size_t)nx * ny;
   const int x = (t % B.ntx) * kTX + 4 * threadIdx.x, y = (t / B.ntx) * kTY + threadIdx.y;
-  const bool rowin = y < ny;
-  const int yi = rowin ? y : 0;
-  const size_t r0 = (size_t)yi * nx, rm = (size_t)wrap1(yi - 1, ny) * nx, rp = (size_t)wrap1(yi + 1, ny) * nx;
   const bool aligned = ((reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(B.rho) |
                          reinterpret_cast<uintptr_t>(B.label)) & 15u) == 0;
-  const bool vec = rowin && aligned && (nx & 3) == 0 && x >= 1 && x + 5 <= nx;  // columns x - 1 .. x + 4
   float2 fa[Q], fb[Q];  // cells (x, x + 1) and (x + 2, x + 3)
-  if (vec) {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      const float* q = p + (size_t)i * N + row + x;
-      const float4 w = __ldg(reinterpret_cast<const float4*>(q));  // columns x .. x + 3
-      if (cx(i) > 0) {  // columns x - 1 .. x + 2
-        fa[i] = make_float2(__ldg(q - 1), w.x);
-        fb[i] = make_float2(w.y, w.z);
-      } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
-        fa[i] = make_float2(w.y, w.z);
-        fb[i] = make_float2(w.w, __ldg(q + 4));
-      } else {
-        fa[i] = make_float2(w.x, w.y);
-        fb[i] = make_float2(w.z, w.w);
-      }
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      const float* q = p + (size_t)i * N + row;
-      float v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = rowin && x + j < nx ? __ldg(q + wrap1(x + j - cx(i), nx)) : 0.f;
-      fa[i] = make_float2(v[0], v[1]);
-      fb[i] = make_float2(v[2], v[3]);
-    }
-  }
+  pull4<S>(p, B.wref, nx, ny, x, y, aligned, fa, fb);
   const float2 ra = rho_pair(fa), rb = rho_pair(fb);
   const float r[4] = {ra.x, ra.y, rb.x, rb.y};
-  density_label_tail4(B, t, x, y, r0 + x, r, rowin, vec);
-}
-
-// 16-bit storage, four cells per thread. Where the box's rows start on
-// 8-byte boundaries (nx % 4 == 0) and the four cells and the columns they
-// pull from lie inside the row, a plane arrives in one 8-byte load; a plane
-// the pull shifts by one column adds the 4-byte word beside it, and its
-// pairs (source columns s, s + 1 with s odd) are the high half of one word
-// and the low half of the next. Other cells load element by element with
-// the periodic wrap. Each cell's arithmetic is kb_density_label's, so
-// densities, labels and tile flags are bitwise the same.
-template <int S>
-__device__ __forceinline__ float2 dec16x2(uint32_t bits) {
-  return make_float2(dec16<S>((unsigned short)(bits & 0xffffu)), dec16<S>((unsigned short)(bits >> 16)));
-}
-
-template <int S>
-__global__ void __launch_bounds__(kTX / 4 * kTY, 16) kb_density_label16(const RelabelBox* __restrict__ boxes,
-                                                                        const RelabelEntry* __restrict__ e, int m,
-                                                                        int parity) {
-  const int k = find_entry<kOffTiles>(e, m, blockIdx.x);
-  const RelabelBox& B = boxes[e[k].box];
-  const int t = blockIdx.x - e[k].off_tiles;
-  const unsigned short* p = static_cast<const unsigned short*>(B.pops[B.cur ^ parity]);
-  const int nx = B.nx, ny = B.ny;
-  const size_t N = (size_t)nx * ny;
-  const int x = (t % B.ntx) * kTX + 4 * threadIdx.x, y = (t / B.ntx) * kTY + threadIdx.y;
-  const bool rowin = y < ny;
-  const int yi = rowin ? y : 0;
-  const size_t r0 = (size_t)yi * nx, rm = (size_t)wrap1(yi - 1, ny) * nx, rp = (size_t)wrap1(yi + 1, ny) * nx;
-  const bool aligned = ((reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(B.rho) |
-                         reinterpret_cast<uintptr_t>(B.label)) & 15u) == 0;
-  const bool vec = rowin && aligned && (nx & 3) == 0 && x >= 2 && x + 6 <= nx;  // columns x - 2 .. x + 5
-  float2 fa[Q], fb[Q];  // cells (x, x + 1) and (x + 2, x + 3)
-  if (vec) {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      const unsigned short* q = p + (size_t)i * N + row + x;
-      const uint2 w = __ldg(reinterpret_cast<const uint2*>(q));  // columns x .. x + 3
-      uint32_t lo = w.x, hi = w.y;
-      if (cx(i) > 0) {  // columns x - 1 .. x + 2
-        const uint32_t wm = __ldg(reinterpret_cast<const uint32_t*>(q - 2));
-        lo = __byte_perm(wm, w.x, 0x5432);
-        hi = __byte_perm(w.x, w.y, 0x5432);
-      } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
-        const uint32_t wp = __ldg(reinterpret_cast<const uint32_t*>(q + 4));
-        lo = __byte_perm(w.x, w.y, 0x5432);
-        hi = __byte_perm(w.y, wp, 0x5432);
-      }
-      const float2 wr = make_float2(B.wref[i], B.wref[i]);
-      fa[i] = __fadd2_rn(wr, dec16x2<S>(lo));
-      fb[i] = __fadd2_rn(wr, dec16x2<S>(hi));
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      const unsigned short* q = p + (size_t)i * N + row;
-      unsigned v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = rowin && x + j < nx ? __ldg(q + wrap1(x + j - cx(i), nx)) : 0u;
-      const float2 wr = make_float2(B.wref[i], B.wref[i]);
-      fa[i] = __fadd2_rn(wr, dec16x2<S>(v[0] | (v[1] << 16)));
-      fb[i] = __fadd2_rn(wr, dec16x2<S>(v[2] | (v[3] << 16)));
-    }
-  }
-  const float2 ra = rho_pair(fa), rb = rho_pair(fb);
-  const float r[4] = {ra.x, ra.y, rb.x, rb.y};
-  density_label_tail4(B, t, x, y, r0 + x, r, rowin, vec);
+  density_label_tail4(B, t, x, y, (size_t)(y < ny ? y : 0) * nx + x, r, y < ny,
+                      y < ny && aligned && (nx & 3) == 0 && x + 4 <= nx);
 }
 
 // Also appends every tile that needs a visit (active now or at the previous
@@ -1269,27 +891,6 @@ __global__ void __launch_bounds__(kTX * kTY) kb_bounce(const RelabelBox* __restr
 
 }  // namespace
 
-int mass_partials_needed() { return kRedBlocks * kStatVals; }
-
-#define LBM_DISPATCH(storage, KERNEL, ...)                                  \
-  switch (storage) {                                                        \
-    case LBM_F32: KERNEL<LBM_F32><<<__VA_ARGS__>>>; break;                  \
-    case LBM_F16_DEV: KERNEL<LBM_F16_DEV><<<__VA_ARGS__>>>; break;          \
-    case LBM_BF16_DEV: KERNEL<LBM_BF16_DEV><<<__VA_ARGS__>>>; break;        \
-    default: return cudaErrorInvalidValue;                                  \
-  }
-
-cudaError_t launch_density(const FieldParams& fp, float* rho, cudaStream_t s) {
-  const unsigned b = blocks_for(fp.N);
-  switch (fp.storage) {
-    case LBM_F32: k_density<LBM_F32><<<b, kThreads, 0, s>>>(fp, rho); break;
-    case LBM_F16_DEV: k_density<LBM_F16_DEV><<<b, kThreads, 0, s>>>(fp, rho); break;
-    case LBM_BF16_DEV: k_density<LBM_BF16_DEV><<<b, kThreads, 0, s>>>(fp, rho); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
-}
-
 cudaError_t launch_labels(const FieldParams& fp, const float* rho, float threshold, int32_t* label,
                           int* flags, cudaStream_t s, int32_t* keep) {
   const unsigned b = blocks_for(fp.N);
@@ -1322,29 +923,6 @@ cudaError_t launch_rupture(int nx, int ny, float G, float rho0, float eps, const
 cudaError_t launch_mask(int nx, int ny, const int32_t* owner, const uint8_t* open, uint8_t* mask,
                         cudaStream_t s) {
   k_mask<<<blocks_for((long long)nx * ny), kThreads, 0, s>>>(nx, ny, owner, open, mask);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fields(const FieldParams& fp, const float* rho, const uint8_t* mask, uint32_t which,
-                          float* out, cudaStream_t s) {
-  const unsigned b = blocks_for(fp.N);
-  switch (fp.storage) {
-    case LBM_F32: k_fields<LBM_F32><<<b, kThreads, 0, s>>>(fp, rho, mask, which, out); break;
-    case LBM_F16_DEV: k_fields<LBM_F16_DEV><<<b, kThreads, 0, s>>>(fp, rho, mask, which, out); break;
-    case LBM_BF16_DEV: k_fields<LBM_BF16_DEV><<<b, kThreads, 0, s>>>(fp, rho, mask, which, out); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pops_out(const FieldParams& fp, int plane, float* out, cudaStream_t s) {
-  const unsigned b = blocks_for(fp.N);
-  switch (fp.storage) {
-    case LBM_F32: k_pops_out<LBM_F32><<<b, kThreads, 0, s>>>(fp, plane, out); break;
-    case LBM_F16_DEV: k_pops_out<LBM_F16_DEV><<<b, kThreads, 0, s>>>(fp, plane, out); break;
-    case LBM_BF16_DEV: k_pops_out<LBM_BF16_DEV><<<b, kThreads, 0, s>>>(fp, plane, out); break;
-    default: return cudaErrorInvalidValue;
-  }
   return cudaGetLastError();
 }
 
@@ -1397,45 +975,6 @@ cudaError_t launch_bubbles_rho(const lbm_bubble* d_bubbles, int n, double rho_l,
   return cudaGetLastError();
 }
 
-cudaError_t launch_mass(const FieldParams& fp, double* partials, int nparts, double* out_dev,
-                        cudaStream_t s) {
-  if (nparts < kRedBlocks) return cudaErrorInvalidValue;
-  switch (fp.storage) {
-    case LBM_F32: k_mass_partial<LBM_F32><<<kRedBlocks, kThreads, 0, s>>>(fp, partials); break;
-    case LBM_F16_DEV: k_mass_partial<LBM_F16_DEV><<<kRedBlocks, kThreads, 0, s>>>(fp, partials); break;
-    case LBM_BF16_DEV: k_mass_partial<LBM_BF16_DEV><<<kRedBlocks, kThreads, 0, s>>>(fp, partials); break;
-    default: return cudaErrorInvalidValue;
-  }
-  k_sum_partials<1><<<1, kThreads, 0, s>>>(partials, kRedBlocks, out_dev);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_stats(int nx, int ny, const int32_t* label, int32_t* area, double* partials, int nparts,
-                         double* out_dev, int* hist, int nbins, double dmin, double dmax, cudaStream_t s) {
-  if (nparts < kRedBlocks * kStatVals || nbins > kMaxBins) return cudaErrorInvalidValue;
-  const long long N = (long long)nx * ny;
-  cudaError_t e = cudaMemsetAsync(area, 0, sizeof(int32_t) * N, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, sizeof(int) * kMaxBins, s);
-  if (e != cudaSuccess) return e;
-  k_area<<<blocks_for(N), kThreads, 0, s>>>(N, label, area);
-  const double ldmin = log(dmin > 0 ? dmin : 1.0);
-  const double ldspan = log(dmax > dmin && dmin > 0 ? dmax : 2.0 * (dmin > 0 ? dmin : 1.0)) - ldmin;
-  k_stats_partial<<<kRedBlocks, kThreads, 0, s>>>(N, label, area, nbins, ldmin, ldspan, partials, hist);
-  k_sum_partials<kStatVals><<<1, kThreads, 0, s>>>(partials, kRedBlocks, out_dev);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_bubble_list(int nx, int ny, const int32_t* label, int32_t* area, int32_t* list, int* count,
-                               cudaStream_t s) {
-  const long long N = (long long)nx * ny;
-  cudaError_t e = cudaMemsetAsync(area, 0, sizeof(int32_t) * N, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  k_area<<<blocks_for(N), kThreads, 0, s>>>(N, label, area);
-  k_bubble_list<<<blocks_for(N), kThreads, 0, s>>>(N, label, area, list, count);
-  return cudaGetLastError();
-}
-
 bool relabel_tiled_ok(int nx, int ny, int R) { return nx > 2 * R && ny > 2 * R && R <= kOMaxR; }
 
 int relabel_tile_count(int nx, int ny) { return ((nx + kTX - 1) / kTX) * ((ny + kTY - 1) / kTY); }
@@ -1457,12 +996,14 @@ cudaError_t launch_relabel_boxes(int storage, const RelabelBox* boxes, const Rel
     kb_density_label<LBM_F32, true><<<totals[0], block, 0, s>>>(boxes, entries, m, parity);
   } else {
     switch (storage) {
-      case LBM_F32: kb_density_label32<<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity); break;
+      case LBM_F32: 
+        kb_density_label4<LBM_F32><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
+        break;
       case LBM_F16_DEV:
-        kb_density_label16<LBM_F16_DEV><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
+        kb_density_label4<LBM_F16_DEV><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
         break;
       case LBM_BF16_DEV:
-        kb_density_label16<LBM_BF16_DEV><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
+        kb_density_label4<LBM_BF16_DEV><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
         break;
       default: return cudaErrorInvalidValue;
     }

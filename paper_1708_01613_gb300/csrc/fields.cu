@@ -1,0 +1,543 @@
+// Diagnostics of a state: fields, populations, FP64 mass, gas labels, bubble
+// statistics and areas (arXiv 1708.01613, Eqs. 11, 29; Sec. 5 statistics).
+//
+// Every one of these is bound by memory, so each reads the populations once
+// and keeps what it needs on the chip:
+//  - the fields rho, u and p come from one pass that forms the densities of a
+//    tile with its halo in shared memory (a pass per field after a density
+//    pass read the populations up to eight times);
+//  - all population planes are written by one launch, rows by grid
+//    coordinates (a launch per plane with a 64-bit modulo per cell ran at a
+//    third of the bandwidth);
+//  - labels, areas, statistics and the mass come from one density pass over
+//    32 x 8 tiles that joins the gas cells of each tile in shared memory and
+//    flags the tiles holding gas; the passes after it visit only those.
+#include <math.h>
+
+#include "labels.cuh"
+#include "pull.cuh"
+
+namespace lbm {
+namespace {
+
+constexpr int kThreads = 256;
+
+// --- densities (untiled relabel, growth census without the barrier) ---
+constexpr int kRows = 4;  // rows per thread of the row kernels: four cells' loads in flight
+
+template <int S>
+__global__ void __launch_bounds__(kThreads) k_density(const FieldParams fp, float* __restrict__ rho) {
+  using T = typename Store<S>::T;
+  const T* p = static_cast<const T*>(fp.pops);
+  const int nx = fp.nx, ny = fp.ny;
+  const int x = blockIdx.x * kThreads + threadIdx.x;
+  if (x >= nx) return;
+  const int xm = pull_wrap(x - 1, nx), xp = pull_wrap(x + 1, nx);
+  for (int yb = blockIdx.y * kRows; yb < ny; yb += gridDim.y * kRows) {
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const int y = yb + r;
+      if (y >= ny) break;
+      float f[Q];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const int ys = cy(i) > 0 ? pull_wrap(y - 1, ny) : (cy(i) < 0 ? pull_wrap(y + 1, ny) : y);
+        const int xs = cx(i) > 0 ? xm : (cx(i) < 0 ? xp : x);
+        f[i] = Store<S>::load(p, (size_t)i * fp.N + (size_t)ys * nx + xs, fp.wref[i]);
+      }
+      rho[(size_t)y * nx + x] = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
+    }
+  }
+}
+
+// --- populations: plane i of the incoming state, f_i(x) = B_i(x - e_i) ---
+// 8192^2, all nine planes: FP32 2452 -> 822 us, FP16 2330 -> 1707 us (a launch
+// per plane before, with a 64-bit division per cell).
+template <int S>
+__global__ void __launch_bounds__(kThreads) k_pops_out(const FieldParams fp, int plane0, float* __restrict__ out) {
+  using T = typename Store<S>::T;
+  const int nx = fp.nx, ny = fp.ny;
+  const int x = blockIdx.x * kThreads + threadIdx.x;
+  if (x >= nx) return;
+  const int i = plane0 + blockIdx.z;
+  const int ex = (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
+  const int ey = (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0);
+  const T* p = static_cast<const T*>(fp.pops) + (size_t)i * fp.N + pull_wrap(x - ex, nx);
+  float* o = out + (size_t)blockIdx.z * fp.N + x;
+  const float base = fp.wref[i];
+  for (int yb = blockIdx.y * kRows; yb < ny; yb += gridDim.y * kRows) {
+    float v[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+      if (yb + r < ny) v[r] = Store<S>::load(p, (size_t)pull_wrap(yb + r - ey, ny) * nx, base);
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+      if (yb + r < ny) o[(size_t)(yb + r) * nx] = v[r];
+  }
+}
+
+// --- rho, u = (j + F/2)/rho, p (Eq. 29): any of the four in one pass ---
+// A 64 x 8 tile per CTA, two cells per thread. With a velocity asked for, the
+// CTA also forms the densities of the tile's one-cell halo (148 cells beside
+// 512) and shares psi; without one, nothing is shared.
+constexpr int kFX = 64, kFY = 8;
+
+template <int S>
+__device__ __forceinline__ float pulled9(const FieldParams& fp, int x, int y, float (&f)[Q]) {
+  using T = typename Store<S>::T;
+  const T* p = static_cast<const T*>(fp.pops);
+  const int nx = fp.nx, ny = fp.ny;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int xs = pull_wrap(x - cx(i), nx), ys = pull_wrap(y - cy(i), ny);
+    f[i] = Store<S>::load(p, (size_t)i * fp.N + (size_t)ys * nx + xs, fp.wref[i]);
+  }
+  return ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
+}
+
+template <int S, bool VEL>
+__global__ void __launch_bounds__(kThreads) k_fields(const FieldParams fp, const uint8_t* __restrict__ mask,
+                                                     const FieldOuts out) {
+  __shared__ float psi[VEL ? kFY + 2 : 1][VEL ? kFX + 2 : 1];
+  const int nx = fp.nx, ny = fp.ny;
+  const int ntx = (nx + kFX - 1) / kFX;
+  const int x0 = (int)(blockIdx.x % ntx) * kFX, y0 = (int)(blockIdx.x / ntx) * kFY;
+  const int lx = threadIdx.x % kFX, ly = threadIdx.x / kFX;  // cells (lx, ly) and (lx, ly + 4)
+  float rho[2], jx[2], jy[2], ps[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int x = x0 + lx, y = y0 + ly + 4 * q;
+    if (x >= nx || y >= ny) continue;
+    float f[Q];
+    const float r = pulled9<S>(fp, x, y, f);
+    rho[q] = r;
+    jx[q] = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
+    jy[q] = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
+    ps[q] = fp.rho0 * (1.0f - expf(-r * fp.inv_rho0));
+    if (VEL) psi[ly + 4 * q + 1][lx + 1] = ps[q];
+  }
+  if (VEL) {
+    // the halo of the cells inside the box: rows -1 and h, columns -1 and w
+    const int w = min(kFX, nx - x0), h = min(kFY, ny - y0);
+    const int n = 2 * (w + 2) + 2 * h;
+    for (int k = threadIdx.x; k < n; k += kThreads) {
+      int hx, hy;
+      if (k < 2 * (w + 2)) {
+        hy = k < w + 2 ? -1 : h;
+        hx = (k < w + 2 ? k : k - (w + 2)) - 1;
+      } else {
+        const int m = k - 2 * (w + 2);
+        hx = m < h ? -1 : w;
+        hy = m < h ? m : m - h;
+      }
+      float f[Q];
+      const float r = pulled9<S>(fp, pull_wrap(x0 + hx, nx), pull_wrap(y0 + hy, ny), f);
+      psi[hy + 1][hx + 1] = fp.rho0 * (1.0f - expf(-r * fp.inv_rho0));
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int x = x0 + lx, y = y0 + ly + 4 * q;
+    if (x >= nx || y >= ny) continue;
+    const size_t c = (size_t)y * nx + x;
+    const float r = rho[q], psi_c = ps[q];
+    if (out.rho) out.rho[c] = r;
+    if (out.p) out.p[c] = r * (1.0f / 3.0f) + fp.G * psi_c * psi_c * (1.0f / 6.0f);
+    if (VEL) {
+      const unsigned m = mask ? mask[c] : 0u;
+      float sx = 0.f, sy = 0.f;
+#pragma unroll
+      for (int i = 1; i < Q; ++i) {
+        float s = psi[ly + 4 * q + 1 + cy(i)][lx + 1 + cx(i)];
+        if ((m >> (i - 1)) & 1u) s = psi_c;
+        sx += static_cast<float>(wq(i)) * s * cx(i);
+        sy += static_cast<float>(wq(i)) * s * cy(i);
+      }
+      const float g = -fp.G * psi_c;
+      if (out.ux) out.ux[c] = (jx[q] + 0.5f * (g * sx)) / r;
+      if (out.uy) out.uy[c] = (jy[q] + 0.5f * (g * sy)) / r;
+    }
+  }
+}
+
+// --- FP64 sums of FP32 values ---
+// A running sum as an unevaluated pair s + e of FP32 values (Knuth's TwoSum:
+// s and the rounding error of every addition, exactly), handed to FP64 after a
+// few dozen values. FP64 adds run at 1/64 of the FP32 rate here: one per value
+// took 0.61 ms at 4096^2 (FP32 storage) where the bytes take 0.09 ms.
+struct Sum2 {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float b) {
+    const float t = __fadd_rn(s, b), z = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(b, z)));
+    s = t;
+  }
+  __device__ __forceinline__ void add(const Sum2& o) {
+    add(o.s);
+    e = __fadd_rn(e, o.e);
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+
+// Sum of a Sum2 over the warp, in a fixed order (valid in lane 0).
+__device__ __forceinline__ double warp_sum(Sum2 a) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    Sum2 b;
+    b.s = __shfl_down_sync(0xffffffffu, a.s, d);
+    b.e = __shfl_down_sync(0xffffffffu, a.e, d);
+    a.add(b);
+  }
+  return a.value();
+}
+
+// --- fixed-order FP64 reductions ---
+// A fixed number of block partials (not tied to the device's SM count), so the
+// summation order, and with it every reduced value, is the same on any GPU.
+constexpr int kRedBlocks = 608;
+
+template <int NV>
+__device__ void block_reduce_store(double (&v)[NV], double* __restrict__ out) {
+  __shared__ double sh[NV][kThreads];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) sh[j][threadIdx.x] = v[j];
+  __syncthreads();
+  for (int s = kThreads / 2; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s)
+#pragma unroll
+      for (int j = 0; j < NV; ++j) sh[j][threadIdx.x] += sh[j][threadIdx.x + s];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int j = 0; j < NV; ++j) out[j * gridDim.x + blockIdx.x] = sh[j][0];
+}
+
+// Sum of all stored populations: rows of one plane after another, four rows'
+// values in flight per thread.
+template <int S>
+__global__ void __launch_bounds__(kThreads) k_mass_partial(const FieldParams fp, double* partials) {
+  using T = typename Store<S>::T;
+  const T* p = static_cast<const T*>(fp.pops);
+  const long long rows = (long long)Q * fp.ny;
+  double acc[1] = {0.0};
+  for (long long r0 = (long long)blockIdx.x * kRows; r0 < rows; r0 += (long long)gridDim.x * kRows) {
+    for (int xb = 0; xb < fp.nx; xb += 8 * kThreads) {
+      Sum2 a;
+#pragma unroll
+      for (int r = 0; r < kRows; ++r) {
+        const long long row = r0 + r;
+        if (row >= rows) break;
+        const int i = (int)(row / fp.ny);
+        const T* q = p + (size_t)i * fp.N + (size_t)(row - (long long)i * fp.ny) * fp.nx;
+        const float base = fp.wref[i];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int x = xb + k * kThreads + threadIdx.x;
+          if (x < fp.nx) a.add(Store<S>::load(q, (size_t)x, base));
+        }
+      }
+      acc[0] += a.value();
+    }
+  }
+  block_reduce_store<1>(acc, partials);
+}
+
+template <int NV>
+__global__ void __launch_bounds__(kThreads) k_sum_partials(const double* partials, int nparts, double* out) {
+  double acc[NV];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) acc[j] = 0.0;
+  for (int k = threadIdx.x; k < nparts; k += blockDim.x)
+#pragma unroll
+    for (int j = 0; j < NV; ++j) acc[j] += partials[j * nparts + k];
+  block_reduce_store<NV>(acc, out);
+}
+
+// --- labels, areas, statistics ---
+// Density pass over 32 x 8 tiles (8 x 8 threads, four cells each): the labels
+// of each tile's own gas pieces (the smallest index of the piece), one gas
+// flag per tile; with AREA the area slots of its gas cells cleared; with MASS
+// the FP64 sum of the tile's populations.
+template <int S, bool AREA, bool MASS>
+__global__ void __launch_bounds__(kTX / 4 * kTY) kd_label(const FieldParams fp, float threshold, bool base,
+                                                          int32_t* __restrict__ label, int32_t* __restrict__ area,
+                                                          uint8_t* __restrict__ tile_gas, double* __restrict__ tile_mass,
+                                                          int* __restrict__ flags) {
+  using T = typename Store<S>::T;
+  const int nx = fp.nx, ny = fp.ny;
+  const int ntx = (nx + kTX - 1) / kTX, t = blockIdx.x;
+  const int x = (t % ntx) * kTX + 4 * threadIdx.x, y = (t / ntx) * kTY + threadIdx.y;
+  float2 fa[Q], fb[Q];
+  pull4<S>(static_cast<const T*>(fp.pops), fp.wref, nx, ny, x, y, base, fa, fb);
+  const float2 ra = rho_pair(fa), rb = rho_pair(fb);
+  const float r[4] = {ra.x, ra.y, rb.x, rb.y};
+  const bool rowin = y < ny;
+  bool in[4], gas[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    in[j] = rowin && x + j < nx;
+    gas[j] = in[j] && r[j] < threshold;
+  }
+  if (MASS) {
+    Sum2 a;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      if (in[0]) a.add(fa[i].x);
+      if (in[1]) a.add(fa[i].y);
+      if (in[2]) a.add(fb[i].x);
+      if (in[3]) a.add(fb[i].y);
+    }
+    __shared__ double wm[2];
+    const double v = warp_sum(a);
+    const int tid = threadIdx.y * (kTX / 4) + threadIdx.x;
+    if ((tid & 31) == 0) wm[tid >> 5] = v;
+    __syncthreads();
+    if (tid == 0) tile_mass[t] = wm[0] + wm[1];
+  }
+  int32_t lab[4];
+  const int any = tile_labels4(gas, x, y, nx, lab, flags);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (!in[j]) continue;
+    label[(size_t)y * nx + x + j] = lab[j];
+    if (AREA && gas[j]) area[(size_t)y * nx + x + j] = 0;
+  }
+  if (threadIdx.x == 0 && threadIdx.y == 0) tile_gas[t] = (uint8_t)(any != 0);
+}
+
+// One warp per tile with gas: its right and bottom borders joined to the
+// neighbouring tiles (periodic wrap included).
+constexpr int kTileWarps = 8;
+
+__global__ void __launch_bounds__(32 * kTileWarps) kd_union(int nx, int ny, int ntx, int ntiles,
+                                                            const uint8_t* __restrict__ tile_gas, int32_t* L,
+                                                            int* __restrict__ flags) {
+  int fail = 0;
+  for (int t = blockIdx.x * kTileWarps + (threadIdx.x >> 5); t < ntiles; t += gridDim.x * kTileWarps)
+    if (tile_gas[t]) tile_union_borders(L, (t % ntx) * kTX, (t / ntx) * kTY, nx, ny, threadIdx.x & 31, &fail);
+  if (fail) atomicOr(flags + FLAG_TIMEOUT, 1);
+}
+
+// Final labels of the gas tiles; with AREA the cells counted per root, one
+// atomic for the cells of a warp's row that share a root.
+template <bool AREA>
+__global__ void __launch_bounds__(32 * kTileWarps) kd_flatten(int nx, int ny, int ntx, int ntiles,
+                                                              const uint8_t* __restrict__ tile_gas, int32_t* L,
+                                                              int32_t* __restrict__ area, int* __restrict__ flags) {
+  int fail = 0;
+  const int lane = threadIdx.x & 31;
+  for (int t = blockIdx.x * kTileWarps + (threadIdx.x >> 5); t < ntiles; t += gridDim.x * kTileWarps) {
+    if (!tile_gas[t]) continue;
+    const int x = (t % ntx) * kTX + lane, y0 = (t / ntx) * kTY;
+    int run = -1, n = 0;  // cells of this column so far that share the root `run`
+    for (int j = 0; j < kTY; ++j) {
+      const int y = y0 + j;
+      const int c = y * nx + x;
+      int r = -1;
+      if (x < nx && y < ny && L[c] >= 0) {
+        r = find_root(L, c, &fail);
+        L[c] = r;
+      }
+      if (AREA && r >= 0) {
+        if (r != run) {
+          if (n) atomicAdd(area + run, n);
+          run = r;
+          n = 0;
+        }
+        ++n;
+      }
+    }
+    if (AREA) {  // one addition per root and warp
+      const unsigned peers = __match_any_sync(0xffffffffu, run);
+      const int total = __reduce_add_sync(peers, n);
+      if (run >= 0 && lane == __ffs(peers) - 1) atomicAdd(area + run, total);
+    }
+  }
+  if (fail) atomicOr(flags + FLAG_TIMEOUT, 1);
+}
+
+// partial sums: [0] bubbles, [1] gas cells, [2] sum of equivalent diameters;
+// histogram counts are integers, accumulated exactly with atomics
+constexpr int kMaxBins = 64;
+constexpr int kStatVals = 4;  // and [3] the mass (the tiles' partial sums)
+
+__global__ void __launch_bounds__(kThreads) kd_stats(int nx, int ny, int ntx, int ntiles,
+                                                     const uint8_t* __restrict__ tile_gas,
+                                                     const int32_t* __restrict__ L, const int32_t* __restrict__ area,
+                                                     const double* __restrict__ tile_mass, int nbins, double ldmin,
+                                                     double ldspan, double* partials, int* hist) {
+  double v[kStatVals] = {0.0, 0.0, 0.0, 0.0};
+  const int lane = threadIdx.x & 31;
+  int gas = 0;
+  for (int t = blockIdx.x * kTileWarps + (threadIdx.x >> 5); t < ntiles; t += gridDim.x * kTileWarps) {
+    if (!tile_gas[t]) continue;
+    const int x = (t % ntx) * kTX + lane, y0 = (t / ntx) * kTY;
+    for (int j = 0; j < kTY; ++j) {
+      const int y = y0 + j;
+      if (x >= nx || y >= ny) break;
+      const int c = y * nx + x, l = L[c];
+      if (l < 0) continue;
+      ++gas;
+      if (l == c) {
+        const double d = 2.0 * sqrt((double)area[c] / M_PI);
+        v[0] += 1.0;
+        v[2] += d;
+        if (nbins > 0) {
+          int b = (int)floor((log(d) - ldmin) / ldspan * nbins);
+          b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
+          atomicAdd(hist + b, 1);
+        }
+      }
+    }
+  }
+  v[1] = (double)gas;
+  for (int t = blockIdx.x * kThreads + threadIdx.x; t < ntiles; t += gridDim.x * kThreads) v[3] += tile_mass[t];
+  block_reduce_store<kStatVals>(v, partials);
+}
+
+// Roots with their areas appended to list (warp-aggregated slots).
+__global__ void __launch_bounds__(32 * kTileWarps) kd_list(int nx, int ny, int ntx, int ntiles,
+                                                           const uint8_t* __restrict__ tile_gas,
+                                                           const int32_t* __restrict__ L,
+                                                           const int32_t* __restrict__ area, int32_t* __restrict__ list,
+                                                           int* count) {
+  const int lane = threadIdx.x & 31;
+  for (int t = blockIdx.x * kTileWarps + (threadIdx.x >> 5); t < ntiles; t += gridDim.x * kTileWarps) {
+    if (!tile_gas[t]) continue;
+    const int x = (t % ntx) * kTX + lane, y0 = (t / ntx) * kTY;
+    for (int j = 0; j < kTY; ++j) {
+      const int y = y0 + j, c = y * nx + x;
+      const bool root = x < nx && y < ny && L[c] == c;
+      const unsigned b = __ballot_sync(0xffffffffu, root);
+      if (!b) continue;
+      int base = 0;
+      if (lane == __ffs(b) - 1) base = atomicAdd(count, __popc(b));
+      base = __shfl_sync(0xffffffffu, base, __ffs(b) - 1);
+      if (root) {
+        const int k = base + __popc(b & ((1u << lane) - 1u));
+        list[2 * k] = c;
+        list[2 * k + 1] = area[c];
+      }
+    }
+  }
+}
+
+inline dim3 row_grid(int nx, int ny, int planes) {
+  const int gy = (ny + kRows - 1) / kRows;
+  return dim3((nx + kThreads - 1) / kThreads, gy < 65535 ? gy : 65535, planes);
+}
+
+inline int tile_grid(int ntiles) {
+  const int n = (ntiles + kTileWarps - 1) / kTileWarps, cap = device_sm_count() * 8;
+  return n < cap ? n : cap;
+}
+
+inline bool base16(const void* a) { return (reinterpret_cast<uintptr_t>(a) & 15u) == 0; }
+
+}  // namespace
+
+#define LBM_BY_STORAGE(storage, CALL)              \
+  switch (storage) {                               \
+    case LBM_F32: CALL(LBM_F32); break;            \
+    case LBM_F16_DEV: CALL(LBM_F16_DEV); break;    \
+    case LBM_BF16_DEV: CALL(LBM_BF16_DEV); break;  \
+    default: return cudaErrorInvalidValue;         \
+  }
+
+int mass_partials_needed() { return kRedBlocks * kStatVals; }
+
+cudaError_t launch_density(const FieldParams& fp, float* rho, cudaStream_t s) {
+#define CALL(S) k_density<S><<<row_grid(fp.nx, fp.ny, 1), kThreads, 0, s>>>(fp, rho)
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pops_out(const FieldParams& fp, int plane0, int planes, float* out, cudaStream_t s) {
+#define CALL(S) k_pops_out<S><<<row_grid(fp.nx, fp.ny, planes), kThreads, 0, s>>>(fp, plane0, out)
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fields(const FieldParams& fp, const uint8_t* mask, const FieldOuts& out, cudaStream_t s) {
+  const unsigned tiles = (unsigned)((fp.nx + kFX - 1) / kFX) * (unsigned)((fp.ny + kFY - 1) / kFY);
+  if (out.ux || out.uy) {
+#define CALL(S) k_fields<S, true><<<tiles, kThreads, 0, s>>>(fp, mask, out)
+    LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
+  } else {
+#define CALL(S) k_fields<S, false><<<tiles, kThreads, 0, s>>>(fp, mask, out)
+    LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_mass(const FieldParams& fp, double* partials, int nparts, double* out_dev, cudaStream_t s) {
+  if (nparts < kRedBlocks) return cudaErrorInvalidValue;
+#define CALL(S) k_mass_partial<S><<<kRedBlocks, kThreads, 0, s>>>(fp, partials)
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
+  k_sum_partials<1><<<1, kThreads, 0, s>>>(partials, kRedBlocks, out_dev);
+  return cudaGetLastError();
+}
+
+size_t diag_scratch_bytes(int nx, int ny) {
+  const size_t nt = (size_t)relabel_tile_count(nx, ny);
+  return nt * sizeof(double) + nt;
+}
+
+// Tile sums first (8-byte aligned scratch), then the flags.
+static uint8_t* diag_flags(void* scratch, int nt) { return static_cast<uint8_t*>(scratch) + (size_t)nt * sizeof(double); }
+
+template <bool AREA, bool MASS>
+static cudaError_t labels_pass(const FieldParams& fp, float threshold, int32_t* label, int32_t* area, void* scratch,
+                               int* flags, cudaStream_t s) {
+  const int nt = relabel_tile_count(fp.nx, fp.ny), ntx = (fp.nx + kTX - 1) / kTX;
+  uint8_t* tg = diag_flags(scratch, nt);
+  double* tm = static_cast<double*>(scratch);
+#define CALL(S) \
+  kd_label<S, AREA, MASS><<<nt, dim3(kTX / 4, kTY), 0, s>>>(fp, threshold, base16(fp.pops), label, area, tg, tm, flags)
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
+  kd_union<<<tile_grid(nt), 32 * kTileWarps, 0, s>>>(fp.nx, fp.ny, ntx, nt, tg, label, flags);
+  kd_flatten<AREA><<<tile_grid(nt), 32 * kTileWarps, 0, s>>>(fp.nx, fp.ny, ntx, nt, tg, label, area, flags);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_diag_labels(const FieldParams& fp, float threshold, int32_t* label, void* scratch, int* flags,
+                               cudaStream_t s) {
+  return labels_pass<false, false>(fp, threshold, label, nullptr, scratch, flags, s);
+}
+
+cudaError_t launch_diag_stats(const FieldParams& fp, float threshold, int32_t* label, int32_t* area, void* scratch,
+                              int* flags, double* partials, int nparts, double* out_dev, int* hist, int nbins,
+                              double dmin, double dmax, cudaStream_t s) {
+  if (nparts < kRedBlocks * kStatVals || nbins > kMaxBins) return cudaErrorInvalidValue;
+  const int nt = relabel_tile_count(fp.nx, fp.ny), ntx = (fp.nx + kTX - 1) / kTX;
+  cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int) * kMaxBins, s);
+  if (e != cudaSuccess) return e;
+  if ((e = labels_pass<true, true>(fp, threshold, label, area, scratch, flags, s)) != cudaSuccess) return e;
+  const double ldmin = log(dmin > 0 ? dmin : 1.0);
+  const double ldspan = log(dmax > dmin && dmin > 0 ? dmax : 2.0 * (dmin > 0 ? dmin : 1.0)) - ldmin;
+  kd_stats<<<kRedBlocks, kThreads, 0, s>>>(fp.nx, fp.ny, ntx, nt, diag_flags(scratch, nt), label, area,
+                                           static_cast<const double*>(scratch), nbins, ldmin, ldspan, partials, hist);
+  k_sum_partials<kStatVals><<<1, kThreads, 0, s>>>(partials, kRedBlocks, out_dev);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_diag_areas(const FieldParams& fp, float threshold, int32_t* label, int32_t* area, int32_t* list,
+                              int* count, void* scratch, int* flags, cudaStream_t s) {
+  const int nt = relabel_tile_count(fp.nx, fp.ny), ntx = (fp.nx + kTX - 1) / kTX;
+  cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  if ((e = labels_pass<true, false>(fp, threshold, label, area, scratch, flags, s)) != cudaSuccess) return e;
+  kd_list<<<tile_grid(nt), 32 * kTileWarps, 0, s>>>(fp.nx, fp.ny, ntx, nt, diag_flags(scratch, nt), label, area, list,
+                                                    count);
+  return cudaGetLastError();
+}
+
+}  // namespace lbm

@@ -224,26 +224,38 @@ struct FieldParams {
 };
 
 cudaError_t launch_density(const FieldParams& fp, float* rho, cudaStream_t s);
-// Gas labels (4-connected, smallest index) of rho into label. With keep (the
-// relabel pipeline: the owner array), each new gas cell first parks its
-// label of the previous relabel there and the coalescence events are added
-// to flags[FLAG_MERGES]; keep = nullptr for diagnostics.
+// Relabel of a box that does not use the tiled pipeline: gas labels
+// (4-connected, smallest index) of rho into label. Each new gas cell first
+// parks its label of the previous relabel in keep (the owner array) and the
+// coalescence events are added to flags[FLAG_MERGES].
 cudaError_t launch_labels(const FieldParams& fp, const float* rho, float threshold, int32_t* label,
-                          int* flags, cudaStream_t s, int32_t* keep = nullptr);
-// Per-bubble areas of a label array: roots (label[c] == c) with their cell
-// counts appended to list (pairs root, area) in any order; the count goes to
-// *count (device). area: N int32 scratch.
-cudaError_t launch_bubble_list(int nx, int ny, const int32_t* label, int32_t* area, int32_t* list, int* count,
-                               cudaStream_t s);
+                          int* flags, cudaStream_t s, int32_t* keep);
 cudaError_t launch_owner(int nx, int ny, int R, const int32_t* label, int32_t* owner, cudaStream_t s);
 cudaError_t launch_rupture(int nx, int ny, float G, float rho0, float eps, const float* rho,
                            const int32_t* owner, int8_t* sgn, uint8_t* open, int* flags,
                            cudaStream_t s);
 cudaError_t launch_mask(int nx, int ny, const int32_t* owner, const uint8_t* open, uint8_t* mask,
                         cudaStream_t s);
-cudaError_t launch_fields(const FieldParams& fp, const float* rho, const uint8_t* mask,
-                          uint32_t which, float* out, cudaStream_t s);
-cudaError_t launch_pops_out(const FieldParams& fp, int plane, float* out, cudaStream_t s);
+// Diagnostics (fields.cu). Any of rho, u and p in one pass (nullptr: not asked for).
+struct FieldOuts {
+  float *rho, *ux, *uy, *p;
+};
+cudaError_t launch_fields(const FieldParams& fp, const uint8_t* mask, const FieldOuts& out, cudaStream_t s);
+// Planes plane0 .. plane0 + planes of the incoming state, back to back.
+cudaError_t launch_pops_out(const FieldParams& fp, int plane0, int planes, float* out, cudaStream_t s);
+// Scratch the three label passes need beside their arrays (8-byte aligned).
+size_t diag_scratch_bytes(int nx, int ny);
+// Gas labels of the current state.
+cudaError_t launch_diag_labels(const FieldParams& fp, float threshold, int32_t* label, void* scratch, int* flags,
+                               cudaStream_t s);
+// Labels, areas (at their roots), then [0] bubbles [1] gas cells [2] sum of
+// equivalent diameters [3] mass into out_dev and the histogram into hist.
+cudaError_t launch_diag_stats(const FieldParams& fp, float threshold, int32_t* label, int32_t* area, void* scratch,
+                              int* flags, double* partials, int nparts, double* out_dev, int* hist, int nbins,
+                              double dmin, double dmax, cudaStream_t s);
+// Labels, areas, and the (root, area) pairs in any order with their count.
+cudaError_t launch_diag_areas(const FieldParams& fp, float threshold, int32_t* label, int32_t* area, int32_t* list,
+                              int* count, void* scratch, int* flags, cudaStream_t s);
 cudaError_t launch_init_from_rho(int storage, void* pops, const double* rho, int nx, int ny,
                                  const float* wref, cudaStream_t s);
 cudaError_t launch_load_plane(int storage, void* pops, const float* f_plane, int plane, int nx,
@@ -252,9 +264,6 @@ cudaError_t launch_bubbles_rho(const lbm_bubble* d_bubbles, int n, double rho_l,
                                double width, int nx, int ny, double* rho, cudaStream_t s);
 cudaError_t launch_mass(const FieldParams& fp, double* partials, int nparts, double* out_dev,
                         cudaStream_t s);
-cudaError_t launch_stats(int nx, int ny, const int32_t* label, int32_t* area, double* partials,
-                         int nparts, double* out_dev, int* hist, int nbins, double dmin, double dmax,
-                         cudaStream_t s);
 constexpr int kMaxHistBins = 64;
 // Tiled barrier pipeline (barrier.cu): density + labels + tile flags, then
 // union, flatten, owner, rupture and mask restricted to tiles near gas.

@@ -72,6 +72,7 @@ SIGNATURES = {
     "lbm_halted": (C.c_int, [_vp]),
     "lbm_fields_bytes": (C.c_size_t, [_vp, C.c_uint32]),
     "lbm_read_fields": (C.c_int, [_vp, C.c_uint32, _vp, C.c_size_t, C.c_int]),
+    "lbm_read_fields_each": (C.c_int, [_vp, C.c_uint32, C.POINTER(_vp), C.c_int]),
     "lbm_mass": (C.c_int, [_vp, C.POINTER(C.c_double)]),
     "lbm_nucleate": (C.c_int, [_vp, _vp, C.c_int32, C.c_double]),
     "lbm_set_growth": (C.c_int, [_vp, C.c_double, C.c_double]),
@@ -290,20 +291,20 @@ class Simulation:
         written directly by the library."""
         import torch
 
-        out = {}
-        lib = load_library()
+        out, ptrs, bits = {}, {}, 0
         for name in names:
             bit, dt = FIELDS[name]
-            nb = int(lib.lbm_fields_bytes(self.handle, bit))
             shape = (9 * self.components, self.ny, self.nx) if name == "pops" else (self.ny, self.nx)
             if device:
-                t = torch.empty(shape, dtype=getattr(torch, np.dtype(dt).name), device=self.device)
-                self._call("lbm_read_fields", C.c_uint32(bit), C.c_void_p(t.data_ptr()), nb, 1)
-                out[name] = t
+                out[name] = torch.empty(shape, dtype=getattr(torch, np.dtype(dt).name), device=self.device)
+                ptrs[bit] = out[name].data_ptr()
             else:
-                a = np.empty(shape, dtype=dt)
-                self._call("lbm_read_fields", C.c_uint32(bit), C.c_void_p(a.ctypes.data), nb, 0)
-                out[name] = a
+                out[name] = np.empty(shape, dtype=dt)
+                ptrs[bit] = out[name].ctypes.data
+            bits |= bit
+        if bits:
+            dsts = (C.c_void_p * len(ptrs))(*[ptrs[b] for b in sorted(ptrs)])
+            self._call("lbm_read_fields_each", C.c_uint32(bits), dsts, 1 if device else 0)
         return out
 
     def mass(self) -> float:
@@ -338,18 +339,19 @@ class Simulation:
     def bubble_areas(self):
         """(labels, areas) of the bubbles of the current density, in
         increasing label order (labels int32, areas float64 cell counts)."""
-        n = C.c_int32(0)
-        lib = load_library()
         import torch
 
-        with torch.cuda.device(self.device):
-            rc = lib.lbm_bubble_areas(self.handle, 0, None, None, C.byref(n))
-        if rc not in (LBM_OK, LBM_EINVAL):
-            _check(rc, self.handle)
-        labels = np.zeros(max(n.value, 1), np.int32)
-        areas = np.zeros(max(n.value, 1), np.float64)
-        self._call("lbm_bubble_areas", int(len(labels)), C.c_void_p(labels.ctypes.data),
-                   C.c_void_p(areas.ctypes.data), C.byref(n))
+        lib = load_library()
+        n = C.c_int32(1024)  # a list with more bubbles is asked for again, with room
+        while True:
+            room = n.value
+            labels, areas = np.zeros(room, np.int32), np.zeros(room, np.float64)
+            with torch.cuda.device(self.device):
+                rc = lib.lbm_bubble_areas(self.handle, room, C.c_void_p(labels.ctypes.data),
+                                          C.c_void_p(areas.ctypes.data), C.byref(n))
+            if rc != LBM_EINVAL or n.value <= room:
+                break
+        _check(rc, self.handle)
         return labels[:n.value].copy(), areas[:n.value].copy()
 
     def sync(self) -> None:
