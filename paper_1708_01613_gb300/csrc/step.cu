@@ -29,7 +29,7 @@
 //    device counter (the automatic choice where nx % 16 == 0).
 //  - k_step_batch: march2 over work items (box, strip, row chunk) of many
 //    boxes in one launch (batch.cu).
-#include "lbm_internal.cuh"
+#include "cellmath.cuh"
 #include "tma.cuh"
 
 namespace lbm {
@@ -37,137 +37,15 @@ namespace {
 
 constexpr int kBX = 256;           // columns per strip (= compute threads)
 constexpr int kTmaThreads = kBX + 32;
-constexpr float kW1 = 1.0f / 9.0f, kW5 = 1.0f / 36.0f, kW0 = 4.0f / 9.0f;
 
 __device__ __forceinline__ int wrapi(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
-
-// ---------------------------------------------------------------- cell math
-// The per-cell arithmetic is written once for V = float (one cell) and
-// V = float2 (two neighbouring cells, packed FP32 instructions), with every
-// operation an explicitly rounded add, multiply or fused multiply-add, so all
-// kernels produce bitwise the same populations.
-template <typename V>
-struct VOps;
-
-template <>
-struct VOps<float> {
-  static __device__ __forceinline__ float set(float a) { return a; }
-  static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-  static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-  static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-  static __device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-  static __device__ __forceinline__ float rcp(float a) { return __frcp_rn(a); }
-  static __device__ __forceinline__ float ex(float a) { return __expf(a); }
-  static __device__ __forceinline__ int bad(float rho) { return !(rho > 0.f && rho < 1e30f); }
-};
-
-// The pair type uses the packed two-wide FP32 instructions of sm_100 and
-// later, whose rounding per component is that of the scalar intrinsics; a
-// difference is the fused b * (-1) + a, which rounds once, exactly as a - b.
-template <>
-struct VOps<float2> {
-  static __device__ __forceinline__ float2 set(float a) { return make_float2(a, a); }
-  static __device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-  static __device__ __forceinline__ float2 sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-  static __device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-  static __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-  static __device__ __forceinline__ float2 rcp(float2 a) { return make_float2(__frcp_rn(a.x), __frcp_rn(a.y)); }
-  static __device__ __forceinline__ float2 ex(float2 a) { return make_float2(__expf(a.x), __expf(a.y)); }
-  static __device__ __forceinline__ int bad(float2 rho) { return VOps<float>::bad(rho.x) | VOps<float>::bad(rho.y); }
-};
-
-// Eq. 11: rho and j from the nine incoming populations.
-template <typename V>
-__device__ __forceinline__ void moments9(const V f[Q], V& rho, V& jx, V& jy) {
-  using O = VOps<V>;
-  rho = O::add(O::add(O::add(f[0], f[1]), O::add(f[2], f[3])), O::add(O::add(f[4], f[5]), O::add(f[6], f[7])));
-  rho = O::add(rho, f[8]);
-  jx = O::add(O::sub(f[1], f[3]), O::add(O::sub(f[5], f[7]), O::sub(f[8], f[6])));
-  jy = O::add(O::sub(f[2], f[4]), O::add(O::sub(f[5], f[7]), O::sub(f[6], f[8])));
-}
-
-// Full density from the summed stored values: for 16-bit storage (DEV) the
-// stored values are deviations g_i = f_i - w_i rho_ref, whose sum is
-// rho - rho_ref (the weights sum to one).
-template <bool DEV, typename V>
-__device__ __forceinline__ V full_rho(V rho_raw, const StepParams& p) {
-  return DEV ? VOps<V>::add(VOps<V>::set(p.rho_ref), rho_raw) : rho_raw;
-}
-
-// Eq. 30.
-template <typename V>
-__device__ __forceinline__ V psi_of(V rho, const StepParams& p) {
-  using O = VOps<V>;
-  return O::mul(O::set(p.rho0), O::sub(O::set(1.0f), O::ex(O::mul(rho, O::set(-p.inv_rho0)))));
-}
-
-// Eq. 22 with the barrier substitution: s[i] holds psi(x + e_i), or psi(x)
-// where the edge is blocked.
-template <typename V>
-__device__ __forceinline__ void force_of(const V s[Q], V psi_c, float G, V& Fx, V& Fy) {
-  using O = VOps<V>;
-  const V w1 = O::set(kW1), w5 = O::set(kW5);
-  const V d57 = O::sub(s[5], s[7]);
-  const V sx = O::fma(w1, O::sub(s[1], s[3]), O::mul(w5, O::add(d57, O::sub(s[8], s[6]))));
-  const V sy = O::fma(w1, O::sub(s[2], s[4]), O::mul(w5, O::add(d57, O::sub(s[6], s[8]))));
-  const V gp = O::mul(O::set(-G), psi_c);
-  Fx = O::mul(gp, sx);
-  Fy = O::mul(gp, sy);
-}
-
-// Eqs. 39-40 (u_eq = (j + tau F)/rho), Eq. 14 evaluated by opposite pairs,
-// Eq. 18 (BGK). f holds the incoming stored values and receives the outgoing
-// ones. With DEV the values are deviations from w_i rho_ref: j is unchanged
-// (sum e_i w_i = 0) and the equilibrium deviation is
-// w_i (rho - rho_ref - 1.5 rho u^2 + rho (3 e.u + 4.5 (e.u)^2)).
-template <bool TAU_ONE, bool DEV, typename V>
-__device__ __forceinline__ void collide(V f[Q], V rho_raw, V jx, V jy, V Fx, V Fy, const StepParams& p, int& bad) {
-  using O = VOps<V>;
-  const V rho = full_rho<DEV>(rho_raw, p);
-  const V ir = O::rcp(rho);
-  const V tau = O::set(p.tau);
-  const V ux = O::mul(O::fma(tau, Fx, jx), ir);
-  const V uy = O::mul(O::fma(tau, Fy, jy), ir);
-  bad |= O::bad(rho);
-  const V uu = O::fma(ux, ux, O::mul(uy, uy));
-  const V a = DEV ? O::fma(O::mul(O::set(-1.5f), rho), uu, rho_raw) : O::mul(rho, O::fma(O::set(-1.5f), uu, O::set(1.0f)));
-  const V r3 = O::mul(O::set(3.0f), rho), r45 = O::mul(O::set(4.5f), rho);
-  const V w1 = O::set(kW1), w5 = O::set(kW5);
-  V feq[Q];
-  feq[0] = O::mul(O::set(kW0), a);
-  {
-    const V s = O::fma(O::mul(r45, ux), ux, a), t = O::mul(r3, ux);
-    feq[1] = O::mul(w1, O::add(s, t));
-    feq[3] = O::mul(w1, O::sub(s, t));
-  }
-  {
-    const V s = O::fma(O::mul(r45, uy), uy, a), t = O::mul(r3, uy);
-    feq[2] = O::mul(w1, O::add(s, t));
-    feq[4] = O::mul(w1, O::sub(s, t));
-  }
-  {
-    const V e = O::add(ux, uy);
-    const V s = O::fma(O::mul(r45, e), e, a), t = O::mul(r3, e);
-    feq[5] = O::mul(w5, O::add(s, t));
-    feq[7] = O::mul(w5, O::sub(s, t));
-  }
-  {
-    const V e = O::sub(uy, ux);
-    const V s = O::fma(O::mul(r45, e), e, a), t = O::mul(r3, e);
-    feq[6] = O::mul(w5, O::add(s, t));
-    feq[8] = O::mul(w5, O::sub(s, t));
-  }
-  const V om = O::set(p.inv_tau);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) f[i] = TAU_ONE ? feq[i] : O::fma(O::sub(feq[i], f[i]), om, f[i]);
-}
 
 // Force + collision + store of one cell from the psi ring.
 template <int S, bool MASKED, bool TAU_ONE>
 __device__ __forceinline__ void finish_cell(float f[Q], float rho, float jx, float jy, unsigned m,
                                             const float (*ring)[kBX + 2], int sm, int s0, int sp, int jc,
                                             const StepParams& p, typename Store<S>::T* __restrict__ dst,
-                                            size_t base, int& bad) {
+                                            size_t base, uint32_t& worst) {
   const float psi_c = ring[s0][jc];
   float s[Q];
 #pragma unroll
@@ -179,7 +57,7 @@ __device__ __forceinline__ void finish_cell(float f[Q], float rho, float jx, flo
   }
   float Fx, Fy;
   force_of(s, psi_c, p.G, Fx, Fy);
-  collide<TAU_ONE, S != LBM_F32>(f, rho, jx, jy, Fx, Fy, p, bad);
+  collide<TAU_ONE, S != LBM_F32>(f, rho, jx, jy, Fx, Fy, p, worst);
 #pragma unroll
   for (int i = 0; i < Q; ++i) Store<S>::store_raw(dst, (size_t)i * p.N + base, f[i]);
 }
@@ -223,7 +101,7 @@ __global__ void __launch_bounds__(kBX) k_step_strip(const StepParams p) {
 
   float fprev[Q];
   float rho_prev = 1.f, jx_prev = 0.f, jy_prev = 0.f;
-  int bad = 0;
+  uint32_t worst = 0;
   for (int r = y0 - 1, k = 0; r <= y1; ++r, ++k) {
     const int rr = wrapi(r, ny);
     const long long row0 = (long long)rr * nx;
@@ -253,7 +131,7 @@ __global__ void __launch_bounds__(kBX) k_step_strip(const StepParams p) {
       const int rc = r - 1;
       const unsigned m = MASKED ? p.mask[(size_t)rc * nx + x] : 0u;
       finish_cell<S, MASKED, TAU_ONE>(fprev, rho_prev, jx_prev, jy_prev, m, ring, (k - 2) & 3, (k - 1) & 3,
-                                      k & 3, jc, p, dst, (size_t)rc * nx + x, bad);
+                                      k & 3, jc, p, dst, (size_t)rc * nx + x, worst);
     }
 #pragma unroll
     for (int i = 0; i < Q; ++i) fprev[i] = f[i];
@@ -261,7 +139,7 @@ __global__ void __launch_bounds__(kBX) k_step_strip(const StepParams p) {
     jx_prev = jx;
     jy_prev = jy;
   }
-  if (bad) atomicOr(p.flags + FLAG_NUMERIC, 1);
+  report_faults(worst, p.flags);
 }
 
 // ---------------------------------------------------------------- TMA-staged kernel
@@ -356,7 +234,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_tma(const StepParams
   float fprev[Q];
   float rho_prev = 1.f, jx_prev = 0.f, jy_prev = 0.f;
   unsigned m_prev = 0;
-  int bad = 0;
+  uint32_t worst = 0;
   int k_abort = 0;
   for (int k = 0; k < nst; ++k) {
     const int slot = k % NSTAGE;
@@ -392,7 +270,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_tma(const StepParams
     } else if (k >= 2 && active) {
       const int rc = y0 + k - 2;  // row collided now
       finish_cell<S, MASKED, TAU_ONE>(fprev, rho_prev, jx_prev, jy_prev, m_prev, ring, (k - 2) & 3, (k - 1) & 3,
-                                      k & 3, jc, p, dst, (size_t)rc * nx + x0 + tid, bad);
+                                      k & 3, jc, p, dst, (size_t)rc * nx + x0 + tid, worst);
     }
 #pragma unroll
     for (int i = 0; i < Q; ++i) fprev[i] = f[i];
@@ -412,7 +290,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_tma(const StepParams
     __syncthreads();
     return;
   }
-  if (bad) atomicOr(p.flags + FLAG_NUMERIC, 1);
+  report_faults(worst, p.flags);
 }
 
 // ---------------------------------------------------------------- two-cell staged kernel
@@ -650,7 +528,7 @@ struct Tma2Smem {
 // Returns false if a stage wait timed out (the CTA must then leave).
 template <int S, bool MASKED, bool TAU_ONE, int NSTAGE, bool FULL = false, bool UNAL = false>
 __device__ __forceinline__ bool march2(const StepParams& p, const Tma2Smem<S, MASKED, NSTAGE, UNAL>& sm, int x0,
-                                       int width_, int y0, int y1, unsigned& gstage, int& bad) {
+                                       int width_, int y0, int y1, unsigned& gstage, uint32_t& worst) {
   const int width = FULL ? kBX2 : width_;  // FULL: a whole strip (known at compile time)
   using G = TmaGeom2<S>;
   using T = typename G::T;
@@ -787,7 +665,7 @@ __device__ __forceinline__ bool march2(const StepParams& p, const Tma2Smem<S, MA
       }
       float2 Fx, Fy;
       force_of(sv, psi_c, p.G, Fx, Fy);
-      collide<TAU_ONE, S != LBM_F32>(fprev, rho_prev, jx_prev, jy_prev, Fx, Fy, p, bad);
+      collide<TAU_ONE, S != LBM_F32>(fprev, rho_prev, jx_prev, jy_prev, Fx, Fy, p, worst);
       const size_t base = (size_t)rc * nx + x0 + 2 * tid;
       if (UNAL) {
         // a pair at an odd buffer index (odd row start, or odd i N) cannot
@@ -854,13 +732,13 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_tma2(const StepParam
   if (y0 >= y1) return;
   march2_init(sm);
   unsigned gstage = 0;
-  int bad = 0;
+  uint32_t worst = 0;
   const int width = min(kBX2, p.nx - x0);
   const bool ok = width == kBX2
-                      ? march2<S, MASKED, TAU_ONE, NSTAGE, true, UNAL>(p, sm, x0, width, y0, y1, gstage, bad)
-                      : march2<S, MASKED, TAU_ONE, NSTAGE, false, UNAL>(p, sm, x0, width, y0, y1, gstage, bad);
+                      ? march2<S, MASKED, TAU_ONE, NSTAGE, true, UNAL>(p, sm, x0, width, y0, y1, gstage, worst)
+                      : march2<S, MASKED, TAU_ONE, NSTAGE, false, UNAL>(p, sm, x0, width, y0, y1, gstage, worst);
   if (!ok) return;
-  if (bad) atomicOr(p.flags + FLAG_NUMERIC, 1);
+  report_faults(worst, p.flags);
 }
 
 // One box, dynamically scheduled: as many CTAs as fit take row chunks (of
@@ -878,7 +756,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_dyn(const StepParams
   march2_init(sm);
   int* counter = p.flags + FLAG_ITEM;
   unsigned gstage = 0;
-  int bad = 0;
+  uint32_t worst = 0;
   for (int guard = 0; guard < nitems + 1; ++guard) {
     __syncthreads();  // the previous chunk's ring and item index are no longer read
     if (threadIdx.x == 0) item_sh = atomicAdd(counter, 1);
@@ -895,11 +773,11 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_dyn(const StepParams
     // full strips take the compile-time-width march (with tau != 1 the two
     // inlined copies would spill at this kernel's register budget)
     const bool ok = TAU_ONE && width == kBX2
-                        ? march2<S, MASKED, TAU_ONE, NSTAGE, TAU_ONE, UNAL>(p, sm, x0, width, y0, y1, gstage, bad)
-                        : march2<S, MASKED, TAU_ONE, NSTAGE, false, UNAL>(p, sm, x0, width, y0, y1, gstage, bad);
+                        ? march2<S, MASKED, TAU_ONE, NSTAGE, TAU_ONE, UNAL>(p, sm, x0, width, y0, y1, gstage, worst)
+                        : march2<S, MASKED, TAU_ONE, NSTAGE, false, UNAL>(p, sm, x0, width, y0, y1, gstage, worst);
     if (!ok) break;  // a stage wait timed out (recorded); no further chunks
   }
-  if (bad) atomicOr(p.flags + FLAG_NUMERIC, 1);
+  report_faults(worst, p.flags);
   __syncthreads();
   if (threadIdx.x == 0) {
     // every CTA arrives here after its last draw from the counter
@@ -950,16 +828,16 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     p.rho0 = in.rho0;
     p.inv_rho0 = in.inv_rho0;
     p.rho_ref = in.rho_ref;
-    int bad = 0;
+    uint32_t worst = 0;
     // full strips take the compile-time-width march (with tau != 1 the two
     // inlined copies would spill at this kernel's register budget)
     const bool ok = TAU_ONE && it.width == kBX2
                         ? march2<S, MASKED, TAU_ONE, NSTAGE, TAU_ONE, UNAL>(p, sm, it.x0, it.width, it.y0, it.y1,
-                                                                             gstage, bad)
+                                                                             gstage, worst)
                         : march2<S, MASKED, TAU_ONE, NSTAGE, false, UNAL>(p, sm, it.x0, it.width, it.y0, it.y1,
-                                                                         gstage, bad);
+                                                                         gstage, worst);
     if (!ok) return;
-    if (bad) atomicOr(p.flags + FLAG_NUMERIC, 1);
+    report_faults(worst, p.flags);
   }
 }
 
