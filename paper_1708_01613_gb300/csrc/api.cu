@@ -69,15 +69,15 @@ Layout layout_for(const lbm_config& c) {
     off = align_up(off + bytes);
     return o;
   };
-  const size_t eb = (size_t)storage_bytes(c.storage);
   const size_t comps = c.components == 2 ? 2 : 1;
-  L.pops[0] = take(comps * Q * N * eb);
-  L.pops[1] = take(comps * Q * N * eb);
+  const size_t pops = comps * Q * (size_t)pop_shape(c.storage, c.nx, c.ny).plane * storage_bytes(c.storage);
+  L.pops[0] = take(pops);
+  L.pops[1] = take(pops);
   L.rho = take(4 * N);
   L.label = take(4 * N);
   if (c.barrier) {
     L.owner = take(4 * N);
-    L.mask = take(N);
+    L.mask = take((size_t)mask_pitch(c.nx) * c.ny);
     L.open = take(N);
     L.sgn = take(N);
     L.ntiles = relabel_tile_count(c.nx, c.ny);
@@ -118,21 +118,18 @@ int fail(lbm_handle* h, int code, const char* fmt, ...) {
       return fail((h), LBM_ECUDA, "%s: %s", #expr, cudaGetErrorString(e_));             \
   } while (0)
 
-// Buffer `buf`'s planes of component k (two-component boxes are FP32).
-void* component_pops(lbm_handle* h, int buf, int k) {
-  return static_cast<char*>(h->pops(buf)) + (size_t)k * Q * h->N() * storage_bytes(h->cfg.storage);
-}
-
 Step2Params step2_params(lbm_handle* h) {
   const lbm_config& c = h->cfg;
   Step2Params q{};
-  q.src = h->pops(h->cur);
-  q.dst = h->pops(1 - h->cur);
+  q.src = h->col0(h->cur);
+  q.dst = h->col0(1 - h->cur);
   q.mask = c.barrier ? h->mask() : nullptr;
   q.flags = h->flags();
   q.nx = c.nx;
   q.ny = c.ny;
-  q.N = (long long)h->N();
+  q.pitch = h->shape.pitch;
+  q.plane = h->shape.plane;
+  q.mpitch = mask_pitch(c.nx);
   q.tau_m = (float)c.tau;
   q.tau_g = (float)c.tau_g;
   q.inv_tau_m = (float)(1.0 / c.tau);
@@ -147,16 +144,26 @@ Step2Params step2_params(lbm_handle* h) {
 
 FieldParams field_params(lbm_handle* h) {
   FieldParams fp{};
-  fp.pops = h->pops(h->cur);
+  fp.pops = h->col0(h->cur);
   fp.storage = h->cfg.storage;
   fp.nx = h->cfg.nx;
   fp.ny = h->cfg.ny;
   fp.N = (long long)h->N();
+  fp.pitch = h->shape.pitch;
+  fp.plane = h->shape.plane;
+  fp.mpitch = mask_pitch(h->cfg.nx);
   fp.G = (float)h->cfg.G;
   fp.rho0 = (float)h->cfg.rho0;
   fp.inv_rho0 = (float)(1.0 / h->cfg.rho0);
   fp.tau = (float)h->cfg.tau;
   for (int i = 0; i < Q; ++i) fp.wref[i] = h->wref[i];
+  return fp;
+}
+
+// The same for component k's planes.
+FieldParams component_params(lbm_handle* h, int k) {
+  FieldParams fp = field_params(h);
+  fp.pops = h->col0(h->cur, k);
   return fp;
 }
 
@@ -177,7 +184,7 @@ int check_flags(lbm_handle* h) {
 int reset_state(lbm_handle* h) {
   CUDA_TRY(h, cudaMemsetAsync(h->flags(), 0, sizeof(int) * FLAG_COUNT, h->stream));
   if (h->cfg.barrier) {
-    CUDA_TRY(h, cudaMemsetAsync(h->mask(), 0, h->N(), h->stream));
+    CUDA_TRY(h, cudaMemsetAsync(h->mask() - kMaskPad, 0, h->mask_bytes(), h->stream));
     CUDA_TRY(h, cudaMemsetAsync(h->open(), 0, h->N(), h->stream));
     CUDA_TRY(h, cudaMemsetAsync(h->sgn(), 0, h->N(), h->stream));
     CUDA_TRY(h, cudaMemsetAsync(h->owner(), 0xff, 4 * h->N(), h->stream));
@@ -220,7 +227,7 @@ int relabel(lbm_handle* h) {
   CUDA_TRY(h, launch_owner(c.nx, c.ny, c.zone_radius, h->label(), h->owner(), h->stream));
   CUDA_TRY(h, launch_rupture(c.nx, c.ny, (float)c.G, (float)c.rho0, (float)c.rupture_eps, h->rho(),
                              h->owner(), h->sgn(), h->open(), h->flags(), h->stream));
-  CUDA_TRY(h, launch_mask(c.nx, c.ny, h->owner(), h->open(), h->mask(), h->stream));
+  CUDA_TRY(h, launch_mask(c.nx, c.ny, mask_pitch(c.nx), h->owner(), h->open(), h->mask(), h->stream));
   h->launches += kRelabelLaunches;
   return LBM_OK;
 }
@@ -236,7 +243,7 @@ cudaError_t bounce_after_step(lbm_handle* h) {
     relabel_entry_sizes(c.nx, c.ny, &totals[0], &totals[1], &totals[2]);
     return launch_bounce_boxes(c.storage, two, h->rbox(), h->rentries(), 1, totals[2], h->cur ^ 1, h->stream);
   }
-  return launch_bounce(c.storage, two, h->pops(1 - h->cur), h->mask(), c.nx, c.ny, h->stream);
+  return launch_bounce(field_params(h), two, h->col0(1 - h->cur), h->mask(), h->stream);
 }
 
 int read_opened(lbm_handle* h, int* out) {
@@ -313,15 +320,17 @@ int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_de
     if (!dst[b]) continue;
     const size_t nb = b == 5 ? 4 * N : N;
     const int fill = b == 5 ? 0xff : 0;
-    if (state[b - 5]) CUDA_TRY(h, cudaMemcpyAsync(dst[b], state[b - 5], nb, d2x, h->stream));
+    if (state[b - 5] && b == 6)  // rows without their padding
+      CUDA_TRY(h, cudaMemcpy2DAsync(dst[b], h->cfg.nx, state[b - 5], mask_pitch(h->cfg.nx), h->cfg.nx, h->cfg.ny, d2x,
+                                    h->stream));
+    else if (state[b - 5]) CUDA_TRY(h, cudaMemcpyAsync(dst[b], state[b - 5], nb, d2x, h->stream));
     else if (dst_is_device) CUDA_TRY(h, cudaMemsetAsync(dst[b], fill, nb, h->stream));
     else memset(dst[b], fill, nb);
   }
   if (dst[8]) {
     char* out = static_cast<char*>(dst[8]);
     for (int k = 0; k < h->comps(); ++k, out += 4 * Q * N) {
-      FieldParams fk = fp;
-      fk.pops = component_pops(h, h->cur, k);
+      const FieldParams fk = component_params(h, k);
       if (dst_is_device) {
         CUDA_TRY(h, launch_pops_out(fk, 0, Q, reinterpret_cast<float*>(out), h->stream));
         continue;
@@ -353,6 +362,8 @@ int handle_fail(lbm_handle* h, int code, const char* fmt, ...) {
 
 int handle_relabel(lbm_handle* h) { return relabel(h); }
 
+FieldParams handle_field_params(lbm_handle* h) { return field_params(h); }
+
 bool handle_relabel_tiled(const lbm_handle* h) {
   return h->cfg.barrier && relabel_tiled_ok(h->cfg.nx, h->cfg.ny, h->cfg.zone_radius);
 }
@@ -361,8 +372,11 @@ RelabelBox handle_relabel_box(lbm_handle* h) {
   const lbm_config& c = h->cfg;
   RelabelBox b;
   memset(&b, 0, sizeof(b));
-  b.pops[0] = h->pops(0);
-  b.pops[1] = h->pops(1);
+  b.pops[0] = h->col0(0);
+  b.pops[1] = h->col0(1);
+  b.pitch = h->shape.pitch;
+  b.plane = h->shape.plane;
+  b.mpitch = mask_pitch(c.nx);
   b.rho = h->rho();
   b.label = h->label();
   b.owner = h->owner();
@@ -402,14 +416,15 @@ StepParams handle_step_params(lbm_handle* h) {
   p.flags = h->flags();
   p.nx = c.nx;
   p.ny = c.ny;
-  p.N = (long long)h->N();
+  p.pitch = h->shape.pitch;
+  p.plane = h->shape.plane;
+  p.mpitch = mask_pitch(c.nx);
   p.tau = (float)c.tau;
   p.inv_tau = (float)(1.0 / c.tau);
   p.G = (float)c.G;
   p.rho0 = (float)c.rho0;
   p.inv_rho0 = (float)(1.0 / c.rho0);
   p.rho_ref = (float)c.rho_ref;
-  for (int i = 0; i < Q; ++i) p.wref[i] = h->wref[i];
   return p;
 }
 
@@ -456,6 +471,7 @@ int lbm_create(const lbm_config* cfg, void* d_workspace, size_t bytes, void* cud
   if (!h) return LBM_ENOMEM;
   h->cfg = *cfg;
   h->L = L;
+  h->shape = pop_shape(cfg->storage, cfg->nx, cfg->ny);
   h->ws = static_cast<char*>(d_workspace);
   h->stream = static_cast<cudaStream_t>(cuda_stream);
   h->cur = 0;
@@ -492,8 +508,7 @@ int lbm_init_density(lbm_handle* h, const double* rho, int src_is_device) {
     src = static_cast<const double*>(stage);
   }
   for (int k = 0; k < comps; ++k)  // component k's planes follow the previous component's nine
-    CUDA_TRY(h, launch_init_from_rho(h->cfg.storage, component_pops(h, h->cur, k), src + (size_t)k * h->N(),
-                                     h->cfg.nx, h->cfg.ny, h->wref, h->stream));
+    CUDA_TRY(h, launch_init_from_rho(component_params(h, k), src + (size_t)k * h->N(), h->stream));
   return reset_state(h);
 }
 
@@ -518,8 +533,7 @@ int lbm_init_bubbles(lbm_handle* h, const lbm_bubble* b, int32_t n, double rho_l
   if (n > 0)
     CUDA_TRY(h, cudaMemcpyAsync(d_b, b, sizeof(lbm_bubble) * n, cudaMemcpyHostToDevice, h->stream));
   CUDA_TRY(h, launch_bubbles_rho(d_b, n, rho_l, rho_g, width, h->cfg.nx, h->cfg.ny, d_rho, h->stream));
-  CUDA_TRY(h, launch_init_from_rho(h->cfg.storage, h->pops(h->cur), d_rho, h->cfg.nx, h->cfg.ny, h->wref,
-                                   h->stream));
+  CUDA_TRY(h, launch_init_from_rho(field_params(h), d_rho, h->stream));
   // the bubble list is read from pageable memory by an async copy: keep it valid
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   return reset_state(h);
@@ -538,8 +552,7 @@ int lbm_load_populations(lbm_handle* h, const float* f, int src_is_device) {
       CUDA_TRY(h, cudaMemcpyAsync(stage, plane, 4 * N, cudaMemcpyHostToDevice, h->stream));
       plane = stage;
     }
-    CUDA_TRY(h, launch_load_plane(h->cfg.storage, component_pops(h, h->cur, pl / Q), plane, pl % Q, h->cfg.nx,
-                                  h->cfg.ny, h->wref, h->stream));
+    CUDA_TRY(h, launch_load_plane(component_params(h, pl / Q), plane, pl % Q, h->stream));
   }
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->halted = 0;
@@ -573,8 +586,8 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
                                     h->flags() + FLAG_GAS, h->stream));
       h->launches += c.barrier ? 1 : 2;
     }
-    p.src = h->pops(h->cur);
-    p.dst = h->pops(1 - h->cur);
+    p.src = h->col0(h->cur);
+    p.dst = h->col0(1 - h->cur);
     if (c.components == 2) {
       const Step2Params q = step2_params(h);
       CUDA_TRY(h, launch_step2(q, h->stream));
@@ -583,8 +596,8 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     }
     h->launches += 1;
     if (growing) {
-      CUDA_TRY(h, launch_growth(c.storage, p.dst, h->gas_list(), h->flags() + FLAG_GAS, (long long)h->N(),
-                                h->growth_rate, h->growth_budget, h->released(), (int)(h->t & 1), h->stream));
+      CUDA_TRY(h, launch_growth(field_params(h), p.dst, h->gas_list(), h->flags() + FLAG_GAS, h->growth_rate,
+                                h->growth_budget, h->released(), (int)(h->t & 1), h->stream));
       h->launches += 1;
     }
     if (c.barrier) {  // populations that would cross a blocked edge bounce back
@@ -607,8 +620,7 @@ int lbm_set_step_variant(lbm_handle* h, int variant) {
   if (variant < 0 || variant > 4) return fail(h, LBM_EINVAL, "variant must be 0, 1, 2, 3 or 4");
   if (variant == 2 && !step_tma_allowed(h->cfg.storage, h->cfg.nx))
     return fail(h, LBM_ENOTSUP, "TMA-staged step needs nx %% 16 == 0 and nx >= 272");
-  if ((variant == 3 || variant == 4) && !step_tma2_allowed(h->cfg.storage, h->cfg.nx) &&
-      !step_tma2_unaligned_allowed(h->cfg.nx))
+  if ((variant == 3 || variant == 4) && !step_tma2_allowed(h->cfg.nx))
     return fail(h, LBM_ENOTSUP, "two-cell staged step needs nx >= 16");
   h->variant = variant;
   return LBM_OK;
@@ -662,8 +674,7 @@ int lbm_nucleate(lbm_handle* h, const lbm_bubble* nuclei, int32_t n, double rho_
   if (rc) return rc;
   lbm_bubble* d_n = static_cast<lbm_bubble*>(h->pops(1 - h->cur));  // the idle buffer stages the list
   CUDA_TRY(h, cudaMemcpyAsync(d_n, nuclei, sizeof(lbm_bubble) * n, cudaMemcpyHostToDevice, h->stream));
-  CUDA_TRY(h, launch_nucleate(h->cfg.storage, h->pops(h->cur), d_n, n, rho_g, h->cfg.nx, h->cfg.ny, h->wref,
-                              h->stream));
+  CUDA_TRY(h, launch_nucleate(field_params(h), h->col0(h->cur), d_n, n, rho_g, h->stream));
   h->launches += 1;
   // the list is read from pageable memory by an async copy: keep it valid
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
@@ -707,8 +718,7 @@ int lbm_mass(lbm_handle* h, double* out) {
   if (rc) return rc;
   double part[2] = {0.0, 0.0};
   for (int k = 0; k < h->comps(); ++k) {
-    FieldParams fk = field_params(h);
-    fk.pops = component_pops(h, h->cur, k);
+    const FieldParams fk = component_params(h, k);
     CUDA_TRY(h, launch_mass(fk, h->partials(), h->L.nparts, h->scalars(), h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(&part[k], h->scalars(), sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));  // the scalar slot is reused by the next component

@@ -253,8 +253,8 @@ __global__ void k_rupture(int nx, int ny, float G, float rho0, float eps,
   if (opened) atomicAdd(flags + FLAG_OPENED, opened);
 }
 
-__global__ void k_mask(int nx, int ny, const int32_t* __restrict__ own, const uint8_t* __restrict__ open,
-                       uint8_t* __restrict__ mask) {
+__global__ void k_mask(int nx, int ny, int mpitch, const int32_t* __restrict__ own,
+                       const uint8_t* __restrict__ open, uint8_t* __restrict__ mask) {
   const long long N = (long long)nx * ny;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
        c += (long long)gridDim.x * blockDim.x) {
@@ -269,44 +269,38 @@ __global__ void k_mask(int nx, int ny, const int32_t* __restrict__ own, const ui
         if (on != -1 && on != o && !open[nb]) m |= 1u << (i - 1);
       }
     }
-    mask[c] = (uint8_t)m;
+    put_cell(mask + (size_t)y * mpitch, x, nx, (uint8_t)m);
   }
 }
 
-// The stored buffer holds f_i at the source cell of the next pull: B_i(y) = f_i(y + e_i).
+// --- initialisation: rows by grid coordinates, one column per thread ---
+// The stored buffer holds f_i at the source cell of the next pull:
+// B_i(y) = f_i(y + e_i).
 template <int S>
-__global__ void k_init_from_rho(typename Store<S>::T* __restrict__ pops, const double* __restrict__ rho,
-                                int nx, int ny, FieldParams fp) {
-  const long long N = (long long)nx * ny;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx), y = (int)(c / nx);
+__global__ void __launch_bounds__(kThreads) k_init_from_rho(const FieldParams fp, typename Store<S>::T* __restrict__ pops,
+                                                            const double* __restrict__ rho) {
+  const int nx = fp.nx, ny = fp.ny, x = blockIdx.x * kThreads + threadIdx.x;
+  if (x >= nx) return;
+  const int xm = pull_wrap(x - 1, nx), xp = pull_wrap(x + 1, nx);
+  for (int y = blockIdx.y; y < ny; y += gridDim.y) {
+    const size_t r0 = (size_t)y * nx, rm = (size_t)pull_wrap(y - 1, ny) * nx, rp = (size_t)pull_wrap(y + 1, ny) * nx;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const long long src = (long long)wrapi(y + cy(i), ny) * nx + wrapi(x + cx(i), nx);
-      const float f = (float)(wq(i) * rho[src]);
-      Store<S>::store(pops, (size_t)i * N + c, f, fp.wref[i]);
+      const double r = rho[(cy(i) > 0 ? rp : (cy(i) < 0 ? rm : r0)) + (cx(i) > 0 ? xp : (cx(i) < 0 ? xm : x))];
+      put_cell(pops + (size_t)i * fp.plane + (size_t)y * fp.pitch, x, nx, Store<S>::of((float)(wq(i) * r), fp.wref[i]));
     }
   }
 }
 
 template <int S>
-__global__ void k_load_plane(typename Store<S>::T* __restrict__ pops, const float* __restrict__ fpl,
-                             int plane, int nx, int ny, float base) {
-  const long long N = (long long)nx * ny;
-  int ex = 0, ey = 0;
-#pragma unroll
-  for (int i = 0; i < Q; ++i)
-    if (i == plane) {
-      ex = cx(i);
-      ey = cy(i);
-    }
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx), y = (int)(c / nx);
-    const long long src = (long long)wrapi(y + ey, ny) * nx + wrapi(x + ex, nx);
-    Store<S>::store(pops, (size_t)plane * N + c, fpl[src], base);
-  }
+__global__ void __launch_bounds__(kThreads) k_load_plane(const FieldParams fp, typename Store<S>::T* __restrict__ pops,
+                                                         const float* __restrict__ f, int plane, int ex, int ey) {
+  const int nx = fp.nx, ny = fp.ny, x = blockIdx.x * kThreads + threadIdx.x;
+  if (x >= nx) return;
+  const int xs = pull_wrap(x + ex, nx);
+  for (int y = blockIdx.y; y < ny; y += gridDim.y)
+    put_cell(pops + (size_t)plane * fp.plane + (size_t)y * fp.pitch, x, nx,
+             Store<S>::of(f[(size_t)pull_wrap(y + ey, ny) * nx + xs], fp.wref[plane]));
 }
 
 // Initial density of a bubble set (tanh profile of the signed distance to the
@@ -430,30 +424,27 @@ __global__ void __launch_bounds__(kTX * kTY) kb_density_label(const RelabelBox* 
   const int t = blockIdx.x - e[k].off_tiles;
   const T* p = static_cast<const T*>(B.pops[B.cur ^ parity]);
   const int nx = B.nx, ny = B.ny;
-  const size_t N = (size_t)nx * ny;
   const int x = (t % B.ntx) * kTX + threadIdx.x, y = (t / B.ntx) * kTY + threadIdx.y;
   const bool in = x < nx && y < ny;  // a ragged tile's threads outside the box only join the barriers
   const int xi = in ? x : 0, yi = in ? y : 0;
-  const int xm = wrap1(xi - 1, nx), xp = wrap1(xi + 1, nx);
-  const size_t r0 = (size_t)yi * nx, rm = (size_t)wrap1(yi - 1, ny) * nx, rp = (size_t)wrap1(yi + 1, ny) * nx;
+  const size_t P = (size_t)B.plane;
+  const size_t r0 = (size_t)yi * B.pitch, rm = (size_t)wrap1(yi - 1, ny) * B.pitch, rp = (size_t)wrap1(yi + 1, ny) * B.pitch;
   float f[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-    const int xs = cx(i) > 0 ? xm : (cx(i) < 0 ? xp : xi);
-    f[i] = Store<S>::load(p, (size_t)i * N + row + xs, B.wref[i]);
+    f[i] = Store<S>::load(p + (xi - cx(i)), (size_t)i * P + row, B.wref[i]);
   }
   const float r = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-  const size_t c = r0 + xi;
+  const size_t c = (size_t)yi * nx + xi;
   if (in) B.rho[c] = r;
   if (TWO && in) {  // two components (FP32): the gas lattice follows the melt's nine planes
-    const float* pg = reinterpret_cast<const float*>(p) + (size_t)Q * N;
+    const float* pg = reinterpret_cast<const float*>(p) + (size_t)Q * P;
     float g = 0.f;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      const int xs = cx(i) > 0 ? xm : (cx(i) < 0 ? xp : x);
-      g += __ldg(pg + (size_t)i * N + row + xs);
+      g += __ldg(pg + (size_t)i * P + row + (x - cx(i)));
     }
     const float a = B.rho0 * (1.0f - expf(-r / B.rho0)), b = B.rho0 * (1.0f - expf(-g / B.rho0));
     B.pr[c] = (r + g) * (1.0f / 3.0f) + (B.G * a * a + 2.0f * B.G_mg * a * b + B.G_gg * b * b) * (1.0f / 6.0f);
@@ -552,14 +543,12 @@ __global__ void __launch_bounds__(kTX / 4 * kTY, 16) kb_density_label4(const Rel
   const T* p = static_cast<const T*>(B.pops[B.cur ^ parity]);
   const int nx = B.nx, ny = B.ny;
   const int x = (t % B.ntx) * kTX + 4 * threadIdx.x, y = (t / B.ntx) * kTY + threadIdx.y;
-  const bool aligned = ((reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(B.rho) |
-                         reinterpret_cast<uintptr_t>(B.label)) & 15u) == 0;
   float2 fa[Q], fb[Q];  // cells (x, x + 1) and (x + 2, x + 3)
-  pull4<S>(p, B.wref, nx, ny, x, y, aligned, fa, fb);
+  pull4<S>(p, B.plane, B.pitch, B.wref, ny, x < nx ? x : 0, y < ny ? y : 0, fa, fb);
   const float2 ra = rho_pair(fa), rb = rho_pair(fb);
   const float r[4] = {ra.x, ra.y, rb.x, rb.y};
   density_label_tail4(B, t, x, y, (size_t)(y < ny ? y : 0) * nx + x, r, y < ny,
-                      y < ny && aligned && (nx & 3) == 0 && x + 4 <= nx);
+                      y < ny && (nx & 3) == 0 && x + 4 <= nx);
 }
 
 // Also appends every tile that needs a visit (active now or at the previous
@@ -812,7 +801,7 @@ __global__ void __launch_bounds__(kTX * kTY) kb_mask(const RelabelBox* __restric
         if (on != -1 && on != o && !B.open[nb]) msk |= 1u << (i - 1);
       }
     }
-    if (in) B.mask[c] = (uint8_t)msk;
+    if (in) put_cell(B.mask + (size_t)y * B.mpitch, x, nx, (uint8_t)msk);
     // tiles holding a blocked edge go to the bounce-back's list
     const int film = __syncthreads_or((msk & kCanonBits) != 0);
     if (threadIdx.x == 0 && threadIdx.y == 0) {
@@ -836,36 +825,35 @@ __global__ void __launch_bounds__(kTX * kTY) kb_mask(const RelabelBox* __restric
 // (4 or 2 bytes: the values move bit for bit); TWO: a second lattice follows
 // the first nine planes.
 template <typename T, bool TWO>
-__device__ __forceinline__ void bounce_cell(T* __restrict__ pops, size_t N, int x, int y, int nx, int ny,
+__device__ __forceinline__ void bounce_cell(T* __restrict__ pops, size_t plane, int pitch, int x, int y, int nx, int ny,
                                             unsigned m) {
   m &= kCanonBits;
   if (!m) return;
-  const size_t c = (size_t)y * nx + x;
 #pragma unroll
   for (int i = 1; i <= 6; ++i) {
     if (i == 3 || i == 4 || !((m >> (i - 1)) & 1u)) continue;
-    const size_t a = (size_t)i * N + c;
-    const size_t b = (size_t)opp(i) * N + (size_t)wrap1(y + cy(i), ny) * nx + wrap1(x + cx(i), nx);
-    const T va = pops[a], vb = pops[b];
-    pops[a] = vb;
-    pops[b] = va;
-    if (TWO) {
-      const size_t a2 = a + Q * N, b2 = b + Q * N;
-      const T wa = pops[a2], wb = pops[b2];
-      pops[a2] = wb;
-      pops[b2] = wa;
+    const int xb = wrap1(x + cx(i), nx);
+    T* ra = pops + (size_t)i * plane + (size_t)y * pitch;
+    T* rb = pops + (size_t)opp(i) * plane + (size_t)wrap1(y + cy(i), ny) * pitch;
+#pragma unroll
+    for (int k = 0; k < (TWO ? 2 : 1); ++k, ra += Q * plane, rb += Q * plane) {
+      const T va = ra[x], vb = rb[xb];
+      put_cell(ra, x, nx, vb);
+      put_cell(rb, xb, nx, va);
     }
   }
 }
 
 // Every cell of a box (boxes that do not use the tiled pipeline).
 template <typename T, bool TWO>
-__global__ void k_bounce(T* __restrict__ pops, const uint8_t* __restrict__ mask, int nx, int ny) {
+__global__ void k_bounce(T* __restrict__ pops, const uint8_t* __restrict__ mask, int nx, int ny, int pitch,
+                         long long plane, int mpitch) {
   const long long N = (long long)nx * ny;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
        c += (long long)gridDim.x * blockDim.x) {
-    const unsigned m = mask[c];
-    if (m & kCanonBits) bounce_cell<T, TWO>(pops, (size_t)N, (int)(c % nx), (int)(c / nx), nx, ny, m);
+    const int x = (int)(c % nx), y = (int)(c / nx);
+    const unsigned m = mask[(size_t)y * mpitch + x];
+    if (m & kCanonBits) bounce_cell<T, TWO>(pops, (size_t)plane, pitch, x, y, nx, ny, m);
   }
 }
 
@@ -878,14 +866,13 @@ __global__ void __launch_bounds__(kTX * kTY) kb_bounce(const RelabelBox* __restr
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
   T* pops = static_cast<T*>(const_cast<void*>(B.pops[B.cur ^ q]));
-  const size_t N = (size_t)B.nx * B.ny;
   const int nfilm = B.flags[FLAG_FILM];
   for (int w = lw.first; w < nfilm; w += lw.stride) {
     const int t = B.film_list[w];
     const int x = (t % B.ntx) * kTX + threadIdx.x, y = (t / B.ntx) * kTY + threadIdx.y;
     if (x >= B.nx || y >= B.ny) continue;
-    const unsigned msk = B.mask[(size_t)y * B.nx + x];
-    if (msk & kCanonBits) bounce_cell<T, TWO>(pops, N, x, y, B.nx, B.ny, msk);
+    const unsigned msk = B.mask[(size_t)y * B.mpitch + x];
+    if (msk & kCanonBits) bounce_cell<T, TWO>(pops, (size_t)B.plane, B.pitch, x, y, B.nx, B.ny, msk);
   }
 }
 
@@ -920,51 +907,37 @@ cudaError_t launch_rupture(int nx, int ny, float G, float rho0, float eps, const
   return cudaGetLastError();
 }
 
-cudaError_t launch_mask(int nx, int ny, const int32_t* owner, const uint8_t* open, uint8_t* mask,
+cudaError_t launch_mask(int nx, int ny, int mpitch, const int32_t* owner, const uint8_t* open, uint8_t* mask,
                         cudaStream_t s) {
-  k_mask<<<blocks_for((long long)nx * ny), kThreads, 0, s>>>(nx, ny, owner, open, mask);
+  k_mask<<<blocks_for((long long)nx * ny), kThreads, 0, s>>>(nx, ny, mpitch, owner, open, mask);
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_from_rho(int storage, void* pops, const double* rho, int nx, int ny,
-                                 const float* wref, cudaStream_t s) {
-  FieldParams fp{};
-  for (int i = 0; i < Q; ++i) fp.wref[i] = wref[i];
-  const unsigned b = blocks_for((long long)nx * ny);
-  switch (storage) {
-    case LBM_F32:
-      k_init_from_rho<LBM_F32><<<b, kThreads, 0, s>>>(static_cast<float*>(pops), rho, nx, ny, fp);
-      break;
-    case LBM_F16_DEV:
-      k_init_from_rho<LBM_F16_DEV><<<b, kThreads, 0, s>>>(static_cast<__half*>(pops), rho, nx, ny, fp);
-      break;
-    case LBM_BF16_DEV:
-      k_init_from_rho<LBM_BF16_DEV><<<b, kThreads, 0, s>>>(static_cast<__nv_bfloat16*>(pops), rho, nx,
-                                                            ny, fp);
-      break;
-    default: return cudaErrorInvalidValue;
+static dim3 init_grid(const FieldParams& fp) {
+  return dim3((fp.nx + kThreads - 1) / kThreads, fp.ny < 65535 ? fp.ny : 65535);
+}
+
+#define LBM_BY_STORAGE(storage, CALL)                           \
+  switch (storage) {                                            \
+    case LBM_F32: CALL(LBM_F32, float); break;                  \
+    case LBM_F16_DEV: CALL(LBM_F16_DEV, __half); break;         \
+    case LBM_BF16_DEV: CALL(LBM_BF16_DEV, __nv_bfloat16); break; \
+    default: return cudaErrorInvalidValue;                      \
   }
+
+cudaError_t launch_init_from_rho(const FieldParams& fp, const double* rho, cudaStream_t s) {
+#define CALL(S, T) k_init_from_rho<S><<<init_grid(fp), kThreads, 0, s>>>(fp, static_cast<T*>(const_cast<void*>(fp.pops)), rho)
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
   return cudaGetLastError();
 }
 
-cudaError_t launch_load_plane(int storage, void* pops, const float* f_plane, int plane, int nx, int ny,
-                              const float* wref, cudaStream_t s) {
-  const unsigned b = blocks_for((long long)nx * ny);
-  switch (storage) {
-    case LBM_F32:
-      k_load_plane<LBM_F32><<<b, kThreads, 0, s>>>(static_cast<float*>(pops), f_plane, plane, nx, ny,
-                                                    wref[plane]);
-      break;
-    case LBM_F16_DEV:
-      k_load_plane<LBM_F16_DEV><<<b, kThreads, 0, s>>>(static_cast<__half*>(pops), f_plane, plane, nx, ny,
-                                                        wref[plane]);
-      break;
-    case LBM_BF16_DEV:
-      k_load_plane<LBM_BF16_DEV><<<b, kThreads, 0, s>>>(static_cast<__nv_bfloat16*>(pops), f_plane,
-                                                         plane, nx, ny, wref[plane]);
-      break;
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t launch_load_plane(const FieldParams& fp, const float* f, int plane, cudaStream_t s) {
+#define CALL(S, T)                                                                                                   \
+  k_load_plane<S><<<init_grid(fp), kThreads, 0, s>>>(fp, static_cast<T*>(const_cast<void*>(fp.pops)), f, plane, cx(plane), \
+                                                     cy(plane))
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
   return cudaGetLastError();
 }
 
@@ -1019,16 +992,15 @@ cudaError_t launch_relabel_boxes(int storage, const RelabelBox* boxes, const Rel
   return cudaGetLastError();
 }
 
-cudaError_t launch_bounce(int storage, bool two, void* pops, const uint8_t* mask, int nx, int ny, cudaStream_t s) {
-  const unsigned b = blocks_for((long long)nx * ny);
-  if (two) {
-    if (storage != LBM_F32) return cudaErrorInvalidValue;
-    k_bounce<uint32_t, true><<<b, kThreads, 0, s>>>(static_cast<uint32_t*>(pops), mask, nx, ny);
-  } else if (storage == LBM_F32) {
-    k_bounce<uint32_t, false><<<b, kThreads, 0, s>>>(static_cast<uint32_t*>(pops), mask, nx, ny);
-  } else {
-    k_bounce<uint16_t, false><<<b, kThreads, 0, s>>>(static_cast<uint16_t*>(pops), mask, nx, ny);
-  }
+cudaError_t launch_bounce(const FieldParams& fp, bool two, void* pops, const uint8_t* mask, cudaStream_t s) {
+  const unsigned b = blocks_for(fp.N);
+  if (two && fp.storage != LBM_F32) return cudaErrorInvalidValue;
+#define CALL(T, TWO) \
+  k_bounce<T, TWO><<<b, kThreads, 0, s>>>(static_cast<T*>(pops), mask, fp.nx, fp.ny, fp.pitch, fp.plane, fp.mpitch)
+  if (two) CALL(uint32_t, true);
+  else if (fp.storage == LBM_F32) CALL(uint32_t, false);
+  else CALL(uint16_t, false);
+#undef CALL
   return cudaGetLastError();
 }
 

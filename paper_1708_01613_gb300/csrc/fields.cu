@@ -32,7 +32,6 @@ __global__ void __launch_bounds__(kThreads) k_density(const FieldParams fp, floa
   const int nx = fp.nx, ny = fp.ny;
   const int x = blockIdx.x * kThreads + threadIdx.x;
   if (x >= nx) return;
-  const int xm = pull_wrap(x - 1, nx), xp = pull_wrap(x + 1, nx);
   for (int yb = blockIdx.y * kRows; yb < ny; yb += gridDim.y * kRows) {
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
@@ -42,8 +41,7 @@ __global__ void __launch_bounds__(kThreads) k_density(const FieldParams fp, floa
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         const int ys = cy(i) > 0 ? pull_wrap(y - 1, ny) : (cy(i) < 0 ? pull_wrap(y + 1, ny) : y);
-        const int xs = cx(i) > 0 ? xm : (cx(i) < 0 ? xp : x);
-        f[i] = Store<S>::load(p, (size_t)i * fp.N + (size_t)ys * nx + xs, fp.wref[i]);
+        f[i] = Store<S>::load(p + (x - cx(i)), (size_t)i * fp.plane + (size_t)ys * fp.pitch, fp.wref[i]);
       }
       rho[(size_t)y * nx + x] = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
     }
@@ -51,28 +49,65 @@ __global__ void __launch_bounds__(kThreads) k_density(const FieldParams fp, floa
 }
 
 // --- populations: plane i of the incoming state, f_i(x) = B_i(x - e_i) ---
-// 8192^2, all nine planes: FP32 2452 -> 822 us, FP16 2330 -> 1707 us (a launch
-// per plane before, with a 64-bit division per cell).
+// Four columns of kRows rows per thread. The source row's four columns start
+// at x - e_x: an aligned vector load, and the word beside it for a shifted
+// plane. Dense output rows of a width that is not a multiple of four are
+// written one value at a time. 8192^2, all planes: see the launcher's users;
+// a launch per plane with a division per cell took 2452 us (FP32) and 2330 us
+// (FP16), one value per thread in one launch 822 and 1707 us.
 template <int S>
-__global__ void __launch_bounds__(kThreads) k_pops_out(const FieldParams fp, int plane0, float* __restrict__ out) {
+__device__ __forceinline__ float4 load4(const typename Store<S>::T* q, int ex, float base) {
+  if constexpr (S == LBM_F32) {
+    const float4 w = __ldg(reinterpret_cast<const float4*>(q));
+    if (ex > 0) return make_float4(__ldg(q - 1), w.x, w.y, w.z);
+    if (ex < 0) return make_float4(w.y, w.z, w.w, __ldg(q + 4));
+    return w;
+  } else {
+    const uint2 w = __ldg(reinterpret_cast<const uint2*>(q));
+    uint32_t lo = w.x, hi = w.y;
+    if (ex > 0) {
+      lo = __byte_perm(__ldg(reinterpret_cast<const uint32_t*>(q - 2)), w.x, 0x5432);
+      hi = __byte_perm(w.x, w.y, 0x5432);
+    } else if (ex < 0) {
+      lo = __byte_perm(w.x, w.y, 0x5432);
+      hi = __byte_perm(w.y, __ldg(reinterpret_cast<const uint32_t*>(q + 4)), 0x5432);
+    }
+    const float2 wr = make_float2(base, base), a = __fadd2_rn(wr, dec16x2<S>(lo)), b = __fadd2_rn(wr, dec16x2<S>(hi));
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+}
+
+template <int S>
+__global__ void __launch_bounds__(kThreads) k_pops_out(const FieldParams fp, int plane0, bool vec,
+                                                       float* __restrict__ out) {
   using T = typename Store<S>::T;
   const int nx = fp.nx, ny = fp.ny;
-  const int x = blockIdx.x * kThreads + threadIdx.x;
+  const int x = 4 * (blockIdx.x * kThreads + threadIdx.x);
   if (x >= nx) return;
   const int i = plane0 + blockIdx.z;
   const int ex = (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
   const int ey = (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0);
-  const T* p = static_cast<const T*>(fp.pops) + (size_t)i * fp.N + pull_wrap(x - ex, nx);
+  const T* p = static_cast<const T*>(fp.pops) + (size_t)i * fp.plane + x;
   float* o = out + (size_t)blockIdx.z * fp.N + x;
   const float base = fp.wref[i];
   for (int yb = blockIdx.y * kRows; yb < ny; yb += gridDim.y * kRows) {
-    float v[kRows];
+    float4 v[kRows];
 #pragma unroll
     for (int r = 0; r < kRows; ++r)
-      if (yb + r < ny) v[r] = Store<S>::load(p, (size_t)pull_wrap(yb + r - ey, ny) * nx, base);
+      if (yb + r < ny) v[r] = load4<S>(p + (size_t)pull_wrap(yb + r - ey, ny) * fp.pitch, ex, base);
 #pragma unroll
-    for (int r = 0; r < kRows; ++r)
-      if (yb + r < ny) o[(size_t)(yb + r) * nx] = v[r];
+    for (int r = 0; r < kRows; ++r) {
+      if (yb + r >= ny) continue;
+      float* q = o + (size_t)(yb + r) * nx;
+      if (vec) {
+        *reinterpret_cast<float4*>(q) = v[r];
+      } else {
+        q[0] = v[r].x;
+        if (x + 1 < nx) q[1] = v[r].y;
+        if (x + 2 < nx) q[2] = v[r].z;
+        if (x + 3 < nx) q[3] = v[r].w;
+      }
+    }
   }
 }
 
@@ -86,11 +121,11 @@ template <int S>
 __device__ __forceinline__ float pulled9(const FieldParams& fp, int x, int y, float (&f)[Q]) {
   using T = typename Store<S>::T;
   const T* p = static_cast<const T*>(fp.pops);
-  const int nx = fp.nx, ny = fp.ny;
+  const int ny = fp.ny;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
-    const int xs = pull_wrap(x - cx(i), nx), ys = pull_wrap(y - cy(i), ny);
-    f[i] = Store<S>::load(p, (size_t)i * fp.N + (size_t)ys * nx + xs, fp.wref[i]);
+    const int ys = pull_wrap(y - cy(i), ny);
+    f[i] = Store<S>::load(p + (x - cx(i)), (size_t)i * fp.plane + (size_t)ys * fp.pitch, fp.wref[i]);
   }
   return ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
 }
@@ -145,7 +180,7 @@ __global__ void __launch_bounds__(kThreads) k_fields(const FieldParams fp, const
     if (out.rho) out.rho[c] = r;
     if (out.p) out.p[c] = r * (1.0f / 3.0f) + fp.G * psi_c * psi_c * (1.0f / 6.0f);
     if (VEL) {
-      const unsigned m = mask ? mask[c] : 0u;
+      const unsigned m = mask ? mask[(size_t)y * fp.mpitch + x] : 0u;
       float sx = 0.f, sy = 0.f;
 #pragma unroll
       for (int i = 1; i < Q; ++i) {
@@ -230,7 +265,7 @@ __global__ void __launch_bounds__(kThreads) k_mass_partial(const FieldParams fp,
         const long long row = r0 + r;
         if (row >= rows) break;
         const int i = (int)(row / fp.ny);
-        const T* q = p + (size_t)i * fp.N + (size_t)(row - (long long)i * fp.ny) * fp.nx;
+        const T* q = p + (size_t)i * fp.plane + (size_t)(row - (long long)i * fp.ny) * fp.pitch;
         const float base = fp.wref[i];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -261,7 +296,7 @@ __global__ void __launch_bounds__(kThreads) k_sum_partials(const double* partial
 // flag per tile; with AREA the area slots of its gas cells cleared; with MASS
 // the FP64 sum of the tile's populations.
 template <int S, bool AREA, bool MASS>
-__global__ void __launch_bounds__(kTX / 4 * kTY) kd_label(const FieldParams fp, float threshold, bool base,
+__global__ void __launch_bounds__(kTX / 4 * kTY) kd_label(const FieldParams fp, float threshold, bool vec4,
                                                           int32_t* __restrict__ label, int32_t* __restrict__ area,
                                                           uint8_t* __restrict__ tile_gas, double* __restrict__ tile_mass,
                                                           int* __restrict__ flags) {
@@ -270,7 +305,7 @@ __global__ void __launch_bounds__(kTX / 4 * kTY) kd_label(const FieldParams fp, 
   const int ntx = (nx + kTX - 1) / kTX, t = blockIdx.x;
   const int x = (t % ntx) * kTX + 4 * threadIdx.x, y = (t / ntx) * kTY + threadIdx.y;
   float2 fa[Q], fb[Q];
-  pull4<S>(static_cast<const T*>(fp.pops), fp.wref, nx, ny, x, y, base, fa, fb);
+  pull4<S>(static_cast<const T*>(fp.pops), fp.plane, fp.pitch, fp.wref, ny, x < nx ? x : 0, y < ny ? y : 0, fa, fb);
   const float2 ra = rho_pair(fa), rb = rho_pair(fb);
   const float r[4] = {ra.x, ra.y, rb.x, rb.y};
   const bool rowin = y < ny;
@@ -298,12 +333,18 @@ __global__ void __launch_bounds__(kTX / 4 * kTY) kd_label(const FieldParams fp, 
   }
   int32_t lab[4];
   const int any = tile_labels4(gas, x, y, nx, lab, flags);
+  const size_t c = (size_t)y * nx + x;
+  if (vec4 && in[3]) {
+    *reinterpret_cast<int4*>(label + c) = make_int4(lab[0], lab[1], lab[2], lab[3]);
+  } else {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (!in[j]) continue;
-    label[(size_t)y * nx + x + j] = lab[j];
-    if (AREA && gas[j]) area[(size_t)y * nx + x + j] = 0;
+    for (int j = 0; j < 4; ++j)
+      if (in[j]) label[c + j] = lab[j];
   }
+  if (AREA)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (gas[j]) area[c + j] = 0;
   if (threadIdx.x == 0 && threadIdx.y == 0) tile_gas[t] = (uint8_t)(any != 0);
 }
 
@@ -456,7 +497,9 @@ cudaError_t launch_density(const FieldParams& fp, float* rho, cudaStream_t s) {
 }
 
 cudaError_t launch_pops_out(const FieldParams& fp, int plane0, int planes, float* out, cudaStream_t s) {
-#define CALL(S) k_pops_out<S><<<row_grid(fp.nx, fp.ny, planes), kThreads, 0, s>>>(fp, plane0, out)
+  const bool vec = fp.nx % 4 == 0 && base16(out) && fp.N % 4 == 0;
+  const dim3 grid = row_grid((fp.nx + 3) / 4, fp.ny, planes);
+#define CALL(S) k_pops_out<S><<<grid, kThreads, 0, s>>>(fp, plane0, vec, out)
   LBM_BY_STORAGE(fp.storage, CALL)
 #undef CALL
   return cudaGetLastError();
@@ -500,7 +543,7 @@ static cudaError_t labels_pass(const FieldParams& fp, float threshold, int32_t* 
   uint8_t* tg = diag_flags(scratch, nt);
   double* tm = static_cast<double*>(scratch);
 #define CALL(S) \
-  kd_label<S, AREA, MASS><<<nt, dim3(kTX / 4, kTY), 0, s>>>(fp, threshold, base16(fp.pops), label, area, tg, tm, flags)
+  kd_label<S, AREA, MASS><<<nt, dim3(kTX / 4, kTY), 0, s>>>(fp, threshold, fp.nx % 4 == 0 && base16(label), label, area, tg, tm, flags)
   LBM_BY_STORAGE(fp.storage, CALL)
 #undef CALL
   kd_union<<<tile_grid(nt), 32 * kTileWarps, 0, s>>>(fp.nx, fp.ny, ntx, nt, tg, label, flags);

@@ -43,8 +43,8 @@ __global__ void k_gas_census(const float* __restrict__ rho, long long N, float t
 
 template <int S>
 __global__ void k_growth(typename Store<S>::T* __restrict__ pops, const int32_t* __restrict__ list,
-                         const int* __restrict__ count, long long N, double rate, double budget,
-                         double* __restrict__ released, int parity) {
+                         const int* __restrict__ count, int nx, int pitch, long long plane, double rate,
+                         double budget, double* __restrict__ released, int parity) {
   const int n = *count;
   const double before = released[parity];
   double release = 0.0;
@@ -60,11 +60,11 @@ __global__ void k_growth(typename Store<S>::T* __restrict__ pops, const int32_t*
 #pragma unroll
   for (int i = 0; i < Q; ++i) add[i] = (float)(wq(i) * drho);
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const size_t c = (size_t)list[k];
+    const int c = list[k], y = c / nx, x = c - y * nx;
+    typename Store<S>::T* row = pops + (size_t)y * pitch;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const size_t idx = (size_t)i * N + c;
-      Store<S>::store_raw(pops, idx, __fadd_rn(Store<S>::raw(pops, idx), add[i]));
+    for (int i = 0; i < Q; ++i, row += plane) {
+      put_cell(row, x, nx, Store<S>::enc(__fadd_rn(Store<S>::raw(row, x), add[i])));
     }
   }
 }
@@ -84,7 +84,7 @@ __device__ __forceinline__ bool in_nucleus(const lbm_bubble* __restrict__ nu, in
 
 template <int S>
 __global__ void k_nucleate(typename Store<S>::T* __restrict__ pops, const lbm_bubble* __restrict__ nu, int n,
-                           double rho_g, int nx, int ny, FieldWref wr) {
+                           double rho_g, int nx, int ny, int pitch, long long plane, FieldWref wr) {
   const long long N = (long long)nx * ny;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
        c += (long long)gridDim.x * blockDim.x) {
@@ -93,8 +93,9 @@ __global__ void k_nucleate(typename Store<S>::T* __restrict__ pops, const lbm_bu
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       // incoming f_i(x) lives at B_i(x - e_i)
-      const long long src = (long long)wrap1(y - cy(i), ny) * nx + wrap1(x - cx(i), nx);
-      Store<S>::store(pops, (size_t)i * N + src, (float)(wq(i) * rho_g), wr.w[i]);
+      const int xs = wrap1(x - cx(i), nx);
+      typename Store<S>::T* row = pops + (size_t)i * plane + (size_t)wrap1(y - cy(i), ny) * pitch;
+      put_cell(row, xs, nx, Store<S>::of((float)(wq(i) * rho_g), wr.w[i]));
     }
   }
 }
@@ -115,46 +116,36 @@ cudaError_t launch_gas_census(const float* rho, long long N, float threshold, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_growth(int storage, void* pops, const int32_t* list, const int* count, long long N,
-                          double rate, double budget, double* released, int parity, cudaStream_t s) {
-  const unsigned g = (unsigned)device_sm_count() * 4;
-  switch (storage) {
-    case LBM_F32:
-      k_growth<LBM_F32><<<g, kThreadsG, 0, s>>>(static_cast<float*>(pops), list, count, N, rate, budget, released,
-                                                parity);
-      break;
-    case LBM_F16_DEV:
-      k_growth<LBM_F16_DEV><<<g, kThreadsG, 0, s>>>(static_cast<__half*>(pops), list, count, N, rate, budget,
-                                                    released, parity);
-      break;
-    case LBM_BF16_DEV:
-      k_growth<LBM_BF16_DEV><<<g, kThreadsG, 0, s>>>(static_cast<__nv_bfloat16*>(pops), list, count, N, rate,
-                                                     budget, released, parity);
-      break;
-    default: return cudaErrorInvalidValue;
+#define LBM_BY_STORAGE(storage, CALL)                    \
+  switch (storage) {                                     \
+    case LBM_F32: CALL(LBM_F32, float); break;           \
+    case LBM_F16_DEV: CALL(LBM_F16_DEV, __half); break;  \
+    case LBM_BF16_DEV: CALL(LBM_BF16_DEV, __nv_bfloat16); break; \
+    default: return cudaErrorInvalidValue;               \
   }
+
+cudaError_t launch_growth(const FieldParams& fp, void* pops, const int32_t* list, const int* count, double rate,
+                          double budget, double* released, int parity, cudaStream_t s) {
+  const unsigned g = (unsigned)device_sm_count() * 4;
+#define CALL(S, T)                                                                                                   \
+  k_growth<S><<<g, kThreadsG, 0, s>>>(static_cast<T*>(pops), list, count, fp.nx, fp.pitch, fp.plane, rate, budget, \
+                                      released, parity)
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
   return cudaGetLastError();
 }
 
-cudaError_t launch_nucleate(int storage, void* pops, const lbm_bubble* nuclei, int n, double rho_g, int nx,
-                            int ny, const float* wref, cudaStream_t s) {
+cudaError_t launch_nucleate(const FieldParams& fp, void* pops, const lbm_bubble* nuclei, int n, double rho_g,
+                            cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   FieldWref wr;
-  for (int i = 0; i < Q; ++i) wr.w[i] = wref[i];
-  const unsigned g = grid_for((long long)nx * ny);
-  switch (storage) {
-    case LBM_F32:
-      k_nucleate<LBM_F32><<<g, kThreadsG, 0, s>>>(static_cast<float*>(pops), nuclei, n, rho_g, nx, ny, wr);
-      break;
-    case LBM_F16_DEV:
-      k_nucleate<LBM_F16_DEV><<<g, kThreadsG, 0, s>>>(static_cast<__half*>(pops), nuclei, n, rho_g, nx, ny, wr);
-      break;
-    case LBM_BF16_DEV:
-      k_nucleate<LBM_BF16_DEV><<<g, kThreadsG, 0, s>>>(static_cast<__nv_bfloat16*>(pops), nuclei, n, rho_g, nx,
-                                                       ny, wr);
-      break;
-    default: return cudaErrorInvalidValue;
-  }
+  for (int i = 0; i < Q; ++i) wr.w[i] = fp.wref[i];
+  const unsigned g = grid_for(fp.N);
+#define CALL(S, T)                                                                                              \
+  k_nucleate<S><<<g, kThreadsG, 0, s>>>(static_cast<T*>(pops), nuclei, n, rho_g, fp.nx, fp.ny, fp.pitch, fp.plane, \
+                                        wr)
+  LBM_BY_STORAGE(fp.storage, CALL)
+#undef CALL
   return cudaGetLastError();
 }
 

@@ -56,11 +56,12 @@ struct Store<LBM_F32> {
   static constexpr int bytes = 4;
   __device__ static __forceinline__ float load(const T* p, size_t i, float) { return __ldg(p + i); }
   __device__ static __forceinline__ float load_smem(const T* p, int i, float) { return p[i]; }
-  __device__ static __forceinline__ void store(T* p, size_t i, float v, float) { p[i] = v; }
+  __device__ static __forceinline__ T of(float v, float) { return v; }
   // raw stored value (FP32: the population itself)
   __device__ static __forceinline__ float raw(const T* p, size_t i) { return __ldg(p + i); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return p[i]; }
   __device__ static __forceinline__ void store_raw(T* p, size_t i, float v) { p[i] = v; }
+  __device__ static __forceinline__ T enc(float v) { return v; }
 };
 
 template <>
@@ -73,13 +74,13 @@ struct Store<LBM_F16_DEV> {
   __device__ static __forceinline__ float load_smem(const T* p, int i, float base) {
     return __fadd_rn(base, __half2float(p[i]));
   }
-  __device__ static __forceinline__ void store(T* p, size_t i, float v, float base) {
-    p[i] = __float2half_rn(__fsub_rn(v, base));
-  }
+  // the stored word of a full population value
+  __device__ static __forceinline__ T of(float v, float base) { return __float2half_rn(__fsub_rn(v, base)); }
   // raw stored value: the deviation g = f - w_i rho_ref
   __device__ static __forceinline__ float raw(const T* p, size_t i) { return __half2float(__ldg(p + i)); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return __half2float(p[i]); }
   __device__ static __forceinline__ void store_raw(T* p, size_t i, float g) { p[i] = __float2half_rn(g); }
+  __device__ static __forceinline__ T enc(float g) { return __float2half_rn(g); }
 };
 
 template <>
@@ -92,15 +93,50 @@ struct Store<LBM_BF16_DEV> {
   __device__ static __forceinline__ float load_smem(const T* p, int i, float base) {
     return __fadd_rn(base, __bfloat162float(p[i]));
   }
-  __device__ static __forceinline__ void store(T* p, size_t i, float v, float base) {
-    p[i] = __float2bfloat16_rn(__fsub_rn(v, base));
-  }
+  __device__ static __forceinline__ T of(float v, float base) { return __float2bfloat16_rn(__fsub_rn(v, base)); }
   __device__ static __forceinline__ float raw(const T* p, size_t i) { return __bfloat162float(__ldg(p + i)); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return __bfloat162float(p[i]); }
   __device__ static __forceinline__ void store_raw(T* p, size_t i, float g) { p[i] = __float2bfloat16_rn(g); }
+  __device__ static __forceinline__ T enc(float g) { return __float2bfloat16_rn(g); }
 };
 
 inline int storage_bytes(int s) { return s == LBM_F32 ? 4 : 2; }
+
+// Population planes in HBM. A plane is ny rows of `pitch` values; a row's
+// column 0 starts on a 128-byte boundary, kRowPad bytes into the row, and two
+// ghost columns on either side repeat the other end of the periodic row
+// (columns -2, -1 hold nx - 2, nx - 1; columns nx, nx + 1 hold 0, 1), so a
+// kernel that reads up to two columns beyond its own never wraps, and every
+// row of every width takes aligned vector loads and bulk copies. Each kernel
+// that writes a slot of the outer two columns writes its ghost too. What lies
+// beyond the ghosts is never used, but may be read (vector loads, bulk copies).
+// The mask has rows of `mask_pitch` bytes with the same ghosts.
+constexpr int kRowPad = 128, kMaskPad = 16;
+
+struct PopShape {
+  int pitch;        // values between rows
+  long long plane;  // values between planes
+};
+
+inline PopShape pop_shape(int storage, int nx, int ny) {
+  const int e = storage_bytes(storage);
+  // 16 bytes at least after the last column
+  const long long row = ((long long)kRowPad + (long long)nx * e + 16 + 127) / 128 * 128;
+  PopShape s;
+  s.pitch = (int)(row / e);
+  s.plane = (long long)s.pitch * ny;
+  return s;
+}
+inline int mask_pitch(int nx) { return (2 * kMaskPad + nx + 15) / 16 * 16; }
+
+// One value in its slot and, in the outer two columns, in its ghost. `row`
+// points at column 0.
+template <typename T>
+__device__ __forceinline__ void put_cell(T* row, int x, int nx, T v) {
+  row[x] = v;
+  if (x < 2) row[nx + x] = v;
+  if (x >= nx - 2) row[x - nx] = v;
+}
 
 // Row-chunk height of a launch whose `resident` CTAs draw chunks (gx strips
 // by ny rows) from a counter. Chunks of max_rows rows give `items48` chunks;
@@ -130,13 +166,13 @@ struct StepParams {
   const uint8_t* mask;   // blocked-edge mask (nullptr: plain Shan-Chen)
   int* flags;            // device flag slots
   int nx, ny;
-  long long N;           // nx * ny (plane stride)
+  int pitch, mpitch;     // row strides: population values, mask bytes (src, dst and mask point at column 0)
+  long long plane;       // plane stride
   int rows_per_chunk;    // rows marched by one CTA
   int force_generic;     // kernel variant: 0 automatic, 1 plain loads, 2 one-cell staged, 3 two-cell staged,
                          // 4 two-cell staged with dynamically scheduled row chunks
   float tau, inv_tau, G, rho0, inv_rho0;
   float rho_ref;         // reference density of 16-bit deviations
-  float wref[Q];         // w_i * rho_ref (16-bit deviation base)
 };
 
 // Two-component step (step2.cu): 18 FP32 planes per buffer, melt then gas.
@@ -146,7 +182,8 @@ struct Step2Params {
   const uint8_t* mask;  // nullptr: no barrier
   int* flags;
   int nx, ny;
-  long long N;
+  int pitch, mpitch;    // as in StepParams
+  long long plane;
   int rows_per_chunk;
   float tau_m, tau_g, inv_tau_m, inv_tau_g;
   float G_mm, G_mg, G_gg, rho0, inv_rho0;
@@ -164,6 +201,8 @@ struct BatchInst {
   const uint8_t* mask;  // nullptr: plain Shan-Chen
   int* flags;
   int nx, ny;
+  int pitch, mpitch;
+  long long plane;
   float tau, inv_tau, G, rho0, inv_rho0, rho_ref;
   int cur;              // buffer holding the state when parity == 0
   int pad;
@@ -182,43 +221,28 @@ int device_sm_count();
 cudaError_t launch_step(int storage, const StepParams& p, cudaStream_t s);
 // Launch geometry the fused step uses for a box (for tests/benchmarks).
 void step_geometry(int nx, int ny, int* grid_x, int* grid_y, int* rows_per_chunk, int* block);
-// Whether the TMA-staged step kernel can run on a box of width nx.
+// Widths the staged variants accept (lbm_set_step_variant): 2 takes widths
+// that are multiples of 16 and of at least one strip and its halo, 3 and 4
+// any width of 16 or more.
 bool step_tma_allowed(int storage, int nx);
+bool step_tma2_allowed(int nx);
 // Batched fused step (two-cell staged march over a list of work items of
 // many boxes); one persistent grid drawing items from counters[parity] and
 // zeroing counters[parity ^ 1]. Both counters must be zero before the
 // first launch and consecutive launches must alternate parity.
-// unal: the items' boxes have rows that do not start on 16-byte boundaries
-// (the staging variant that bulk-copies aligned interiors and plain-loads
-// the rest); one launch takes items of one kind.
-cudaError_t launch_step_batch(int storage, bool masked, bool tau_one, bool unal, const BatchInst* insts,
-                              const BatchItem* items, int nitems, int* counters, int parity, cudaStream_t s);
+cudaError_t launch_step_batch(int storage, bool masked, bool tau_one, const BatchInst* insts, const BatchItem* items,
+                              int nitems, int* counters, int parity, cudaStream_t s);
 // CTAs of the batched kernel that fit the GPU at once.
 int batch_resident_ctas(int storage, bool masked, bool tau_one);
-// Whether the two-cell staged step kernel can run on a box of width nx with
-// whole rows bulk-copied (nx % 16 == 0), or in its variant for other widths.
-bool step_tma2_allowed(int storage, int nx);
-bool step_tma2_unaligned_allowed(int nx);
 
 // Barrier / field / reduction kernels (barrier.cu).
-struct Workspace {
-  void* pops[2];
-  float* rho;          // N: density of the current state (relabel, fields)
-  int32_t* label;      // N
-  int32_t* owner;      // N (barrier)
-  uint8_t* mask;       // N (barrier)
-  uint8_t* open;       // N (barrier)
-  int8_t* sgn;         // N (barrier)
-  int* flags;          // FLAG_COUNT
-  double* partials;    // reduction partials
-  int partial_count;
-};
-
 struct FieldParams {
-  const void* pops;    // current populations (post-collision of the last step)
+  const void* pops;    // column 0 of the current populations (post-collision of the last step)
   int storage;
   int nx, ny;
-  long long N;
+  int pitch, mpitch;
+  long long plane;
+  long long N;         // cells
   float G, rho0, inv_rho0, tau;
   float wref[Q];
 };
@@ -234,7 +258,7 @@ cudaError_t launch_owner(int nx, int ny, int R, const int32_t* label, int32_t* o
 cudaError_t launch_rupture(int nx, int ny, float G, float rho0, float eps, const float* rho,
                            const int32_t* owner, int8_t* sgn, uint8_t* open, int* flags,
                            cudaStream_t s);
-cudaError_t launch_mask(int nx, int ny, const int32_t* owner, const uint8_t* open, uint8_t* mask,
+cudaError_t launch_mask(int nx, int ny, int mpitch, const int32_t* owner, const uint8_t* open, uint8_t* mask,
                         cudaStream_t s);
 // Diagnostics (fields.cu). Any of rho, u and p in one pass (nullptr: not asked for).
 struct FieldOuts {
@@ -256,10 +280,10 @@ cudaError_t launch_diag_stats(const FieldParams& fp, float threshold, int32_t* l
 // Labels, areas, and the (root, area) pairs in any order with their count.
 cudaError_t launch_diag_areas(const FieldParams& fp, float threshold, int32_t* label, int32_t* area, int32_t* list,
                               int* count, void* scratch, int* flags, cudaStream_t s);
-cudaError_t launch_init_from_rho(int storage, void* pops, const double* rho, int nx, int ny,
-                                 const float* wref, cudaStream_t s);
-cudaError_t launch_load_plane(int storage, void* pops, const float* f_plane, int plane, int nx,
-                              int ny, const float* wref, cudaStream_t s);
+// Initialisation of the buffer fp.pops: rest equilibrium at rho (nine planes),
+// or the incoming plane `plane` from f (dense rows).
+cudaError_t launch_init_from_rho(const FieldParams& fp, const double* rho, cudaStream_t s);
+cudaError_t launch_load_plane(const FieldParams& fp, const float* f, int plane, cudaStream_t s);
 cudaError_t launch_bubbles_rho(const lbm_bubble* d_bubbles, int n, double rho_l, double rho_g,
                                double width, int nx, int ny, double* rho, cudaStream_t s);
 cudaError_t launch_mass(const FieldParams& fp, double* partials, int nparts, double* out_dev,
@@ -294,6 +318,8 @@ struct RelabelBox {
   float* pr;  // two components: mixture pressure written by the density
               // phase and used by the rupture test (nullptr: one component)
   int nx, ny, ntx, nty, R, cur;
+  int pitch, mpitch;  // pops and mask point at column 0
+  long long plane;
   float threshold, G, rho0, eps;
   float G_mg, G_gg;  // two components: melt-gas and gas-gas couplings
   float wref[Q];
@@ -315,7 +341,7 @@ struct RelabelEntry {
 // the latest tiled relabel of each box in the entry list found holding a
 // blocked edge, on buffer pops[cur ^ q] (total_list = the entries' list-CTA
 // total).
-cudaError_t launch_bounce(int storage, bool two, void* pops, const uint8_t* mask, int nx, int ny, cudaStream_t s);
+cudaError_t launch_bounce(const FieldParams& fp, bool two, void* pops, const uint8_t* mask, cudaStream_t s);
 cudaError_t launch_bounce_boxes(int storage, bool two, const RelabelBox* boxes, const RelabelEntry* entries, int m,
                                 int total_list, int q, cudaStream_t s);
 
@@ -335,9 +361,9 @@ int mass_partials_needed();
 // released[parity ^ 1] (consecutive steps alternate parity).
 cudaError_t launch_gas_census(const float* rho, long long N, float threshold, int32_t* list, int* count,
                               cudaStream_t s);
-cudaError_t launch_growth(int storage, void* pops, const int32_t* list, const int* count, long long N,
-                          double rate, double budget, double* released, int parity, cudaStream_t s);
-cudaError_t launch_nucleate(int storage, void* pops, const lbm_bubble* nuclei, int n, double rho_g, int nx,
-                            int ny, const float* wref, cudaStream_t s);
+cudaError_t launch_growth(const FieldParams& fp, void* pops, const int32_t* list, const int* count, double rate,
+                          double budget, double* released, int parity, cudaStream_t s);
+cudaError_t launch_nucleate(const FieldParams& fp, void* pops, const lbm_bubble* nuclei, int n, double rho_g,
+                            cudaStream_t s);
 
 }  // namespace lbm

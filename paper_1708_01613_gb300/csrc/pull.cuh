@@ -1,10 +1,8 @@
-// Pulled populations of four cells (x .. x + 3) of row y per thread, shared by
-// the relabel's density phase and the diagnostics: f_i(x) = B_i(x - e_i).
-// Where a row's start is aligned to four values and the cells with the columns
-// they pull from lie inside the row, a plane arrives in one vector load (16
-// bytes FP32, 8 bytes 16-bit), a plane the pull shifts by one column adds the
-// value (or 4-byte word) beside it; other cells (the box's first and last
-// columns, ragged tiles, other widths) load one by one with the periodic wrap.
+// Pulled populations of four cells (x .. x + 3, x a multiple of 4) of row y
+// per thread, shared by the relabel's density phase and the diagnostics:
+// f_i(x) = B_i(x - e_i). A plane arrives in one vector load (16 bytes FP32, 8
+// bytes 16-bit), a plane the pull shifts by one column adds the value (or
+// 4-byte word) beside it; the ghost columns stand in for the periodic wrap.
 #pragma once
 #include "lbm_internal.cuh"
 
@@ -24,65 +22,45 @@ __device__ __forceinline__ float2 dec16x2(uint32_t bits) {
 
 __device__ __forceinline__ int pull_wrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
-// Cells (x, x + 1) in fa and (x + 2, x + 3) in fb; cells outside the box read
-// as stored zeros. `base`: the buffer's 16-byte alignment was checked.
+// Cells (x, x + 1) in fa and (x + 2, x + 3) in fb; 0 <= x < nx, 0 <= y < ny.
+// Cells beyond the box's last column take whatever lies there.
 template <int S>
-__device__ __forceinline__ void pull4(const typename Store<S>::T* __restrict__ pops, const float (&wref)[Q], int nx,
-                                      int ny, int x, int y, bool base, float2 (&fa)[Q], float2 (&fb)[Q]) {
-  const size_t N = (size_t)nx * ny;
-  const bool rowin = y < ny;
-  const int yi = rowin ? y : 0;
-  const size_t r0 = (size_t)yi * nx, rm = (size_t)pull_wrap(yi - 1, ny) * nx, rp = (size_t)pull_wrap(yi + 1, ny) * nx;
-  constexpr int K = S == LBM_F32 ? 1 : 2;  // columns x - K .. x + 3 + K are touched
-  const bool vec = rowin && base && (nx & 3) == 0 && x >= K && x + 4 + K <= nx;
-  if (vec) {
+__device__ __forceinline__ void pull4(const typename Store<S>::T* __restrict__ pops, long long plane, int pitch,
+                                      const float (&wref)[Q], int ny, int x, int y, float2 (&fa)[Q], float2 (&fb)[Q]) {
+  const size_t r0 = (size_t)y * pitch + x;
+  const size_t rm = (size_t)(y == 0 ? ny - 1 : y - 1) * pitch + x, rp = (size_t)(y == ny - 1 ? 0 : y + 1) * pitch + x;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      if constexpr (S == LBM_F32) {
-        const float* q = pops + (size_t)i * N + row + x;
-        const float4 w = __ldg(reinterpret_cast<const float4*>(q));  // columns x .. x + 3
-        if (cx(i) > 0) {  // columns x - 1 .. x + 2
-          fa[i] = make_float2(__ldg(q - 1), w.x);
-          fb[i] = make_float2(w.y, w.z);
-        } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
-          fa[i] = make_float2(w.y, w.z);
-          fb[i] = make_float2(w.w, __ldg(q + 4));
-        } else {
-          fa[i] = make_float2(w.x, w.y);
-          fb[i] = make_float2(w.z, w.w);
-        }
+  for (int i = 0; i < Q; ++i) {
+    const size_t at = (size_t)i * plane + (cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0));
+    if constexpr (S == LBM_F32) {
+      const float* q = pops + at;
+      const float4 w = __ldg(reinterpret_cast<const float4*>(q));  // columns x .. x + 3
+      if (cx(i) > 0) {  // columns x - 1 .. x + 2
+        fa[i] = make_float2(__ldg(q - 1), w.x);
+        fb[i] = make_float2(w.y, w.z);
+      } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
+        fa[i] = make_float2(w.y, w.z);
+        fb[i] = make_float2(w.w, __ldg(q + 4));
       } else {
-        const unsigned short* q = reinterpret_cast<const unsigned short*>(pops) + (size_t)i * N + row + x;
-        const uint2 w = __ldg(reinterpret_cast<const uint2*>(q));  // columns x .. x + 3
-        uint32_t lo = w.x, hi = w.y;
-        if (cx(i) > 0) {  // columns x - 1 .. x + 2
-          const uint32_t wm = __ldg(reinterpret_cast<const uint32_t*>(q - 2));
-          lo = __byte_perm(wm, w.x, 0x5432);
-          hi = __byte_perm(w.x, w.y, 0x5432);
-        } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
-          const uint32_t wp = __ldg(reinterpret_cast<const uint32_t*>(q + 4));
-          lo = __byte_perm(w.x, w.y, 0x5432);
-          hi = __byte_perm(w.y, wp, 0x5432);
-        }
-        const float2 wr = make_float2(wref[i], wref[i]);
-        fa[i] = __fadd2_rn(wr, dec16x2<S>(lo));
-        fb[i] = __fadd2_rn(wr, dec16x2<S>(hi));
+        fa[i] = make_float2(w.x, w.y);
+        fb[i] = make_float2(w.z, w.w);
       }
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      const typename Store<S>::T* q = pops + (size_t)i * N + row;
-      float v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (rowin && x + j < nx) v[j] = Store<S>::load(q, (size_t)pull_wrap(x + j - cx(i), nx), wref[i]);
-        else v[j] = wref[i];
+    } else {
+      const unsigned short* q = reinterpret_cast<const unsigned short*>(pops) + at;
+      const uint2 w = __ldg(reinterpret_cast<const uint2*>(q));  // columns x .. x + 3
+      uint32_t lo = w.x, hi = w.y;
+      if (cx(i) > 0) {  // columns x - 1 .. x + 2
+        const uint32_t wm = __ldg(reinterpret_cast<const uint32_t*>(q - 2));
+        lo = __byte_perm(wm, w.x, 0x5432);
+        hi = __byte_perm(w.x, w.y, 0x5432);
+      } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
+        const uint32_t wp = __ldg(reinterpret_cast<const uint32_t*>(q + 4));
+        lo = __byte_perm(w.x, w.y, 0x5432);
+        hi = __byte_perm(w.y, wp, 0x5432);
       }
-      fa[i] = make_float2(v[0], v[1]);
-      fb[i] = make_float2(v[2], v[3]);
+      const float2 wr = make_float2(wref[i], wref[i]);
+      fa[i] = __fadd2_rn(wr, dec16x2<S>(lo));
+      fb[i] = __fadd2_rn(wr, dec16x2<S>(hi));
     }
   }
 }

@@ -32,15 +32,14 @@ constexpr int kBX2C = 256;
 __device__ __forceinline__ int wrap_1(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
 // The nine pulled populations of one component at (x, row r), rows given
-// as offsets of r - 1, r, r + 1 and columns x - 1, x, x + 1 (wrapped).
-__device__ __forceinline__ void pull9(const float* __restrict__ src, long long N, long long rowm, long long row0,
-                                      long long rowp, int xm, int x, int xp, float f[Q]) {
+// as offsets of r - 1, r, r + 1.
+__device__ __forceinline__ void pull9(const float* __restrict__ src, long long plane, long long rowm, long long row0,
+                                      long long rowp, int x, float f[Q]) {
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     // f_i(x) = B_i(x - e_i)
     const long long row = cy(i) > 0 ? rowm : (cy(i) < 0 ? rowp : row0);
-    const int xs = cx(i) > 0 ? xm : (cx(i) < 0 ? xp : x);
-    f[i] = __ldg(src + (size_t)i * N + row + xs);
+    f[i] = __ldg(src + (long long)i * plane + row + (x - cx(i)));
   }
 }
 
@@ -101,7 +100,7 @@ __device__ __forceinline__ void finish2(const Step2Params& p, const float (*ring
                                         const float (*ring_g)[kBX2C + 2], int sm, int s0, int sp, int jc, unsigned m,
                                         float pm[Q], float pg[Q], float rm, float jxm, float jym, float rg, float jxg,
                                         float jyg, float* __restrict__ dst, float* __restrict__ dstg, size_t base,
-                                        int& bad) {
+                                        int x, int& bad) {
   float Smx, Smy, Sgx, Sgy;
   nsum(ring_m, sm, s0, sp, jc, m, Smx, Smy);
   nsum(ring_g, sm, s0, sp, jc, m, Sgx, Sgy);
@@ -121,11 +120,19 @@ __device__ __forceinline__ void finish2(const Step2Params& p, const float (*ring
   const float ugy = rg > 0.f ? uy + tg * Fgy : uy;
   collide9(pm, rm, umx, umy, p.inv_tau_m, TAU_ONE);
   collide9(pg, rg, ugx, ugy, p.inv_tau_g, TAU_ONE);
-  const size_t N = (size_t)p.N;
+  const size_t N = (size_t)p.plane;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     dst[(size_t)i * N + base] = pm[i];
     dstg[(size_t)i * N + base] = pg[i];
+  }
+  if (x < 2 || x >= p.nx - 2) {  // the ghost of an outer column
+    const size_t ghost = x < 2 ? base + p.nx : base - p.nx;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      dst[(size_t)i * N + ghost] = pm[i];
+      dstg[(size_t)i * N + ghost] = pg[i];
+    }
   }
 }
 
@@ -137,7 +144,7 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
   __shared__ float ring_g[4][kBX2C + 2];
   const float* __restrict__ src = static_cast<const float*>(p.src);
   float* __restrict__ dst = static_cast<float*>(p.dst);
-  const long long N = p.N;
+  const long long N = p.plane;
   const float* __restrict__ srcg = src + 9 * N;
   float* __restrict__ dstg = dst + 9 * N;
   const int nx = p.nx, ny = p.ny;
@@ -149,10 +156,6 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
   const int y0 = blockIdx.y * p.rows_per_chunk;
   const int y1 = min(y0 + p.rows_per_chunk, ny);
   if (y0 >= y1) return;  // uniform over the block
-  const int xc = active ? x : last;
-  const int xm = wrap_1(xc - 1, nx), xp = wrap_1(xc + 1, nx);
-  const int xl = wrap_1(x0 - 1, nx), xlm = wrap_1(x0 - 2, nx);
-  const int xr = wrap_1(last + 1, nx), xrp = wrap_1(last + 2, nx);
   const int jc = tid + 1;
 
   float pm[Q], pg[Q];
@@ -160,14 +163,14 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
   int bad = 0;
   for (int r = y0 - 1, k = 0; r <= y1; ++r, ++k) {
     const int rr = wrap_1(r, ny);  // r in [-1, ny]
-    const long long row0 = (long long)rr * nx;
-    const long long rowm = (long long)wrap_1(rr - 1, ny) * nx;
-    const long long rowp = (long long)wrap_1(rr + 1, ny) * nx;
+    const long long row0 = (long long)rr * p.pitch;
+    const long long rowm = (long long)wrap_1(rr - 1, ny) * p.pitch;
+    const long long rowp = (long long)wrap_1(rr + 1, ny) * p.pitch;
     float fm[Q], fg[Q];
     float rm = 1.f, jxm = 0.f, jym = 0.f, rg = 0.f, jxg = 0.f, jyg = 0.f;
     if (active) {
-      pull9(src, N, rowm, row0, rowp, xm, x, xp, fm);
-      pull9(srcg, N, rowm, row0, rowp, xm, x, xp, fg);
+      pull9(src, N, rowm, row0, rowp, x, fm);
+      pull9(srcg, N, rowm, row0, rowp, x, fg);
       mom(fm, rm, jxm, jym);
       mom(fg, rg, jxg, jyg);
       ring_m[k & 3][jc] = psi2(rm, p);
@@ -182,8 +185,7 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
       if (i < Q) {
         const float* base = lane < 16 ? src : srcg;
         const long long row = cy(i) > 0 ? rowm : (cy(i) < 0 ? rowp : row0);
-        const int xs = cx(i) > 0 ? (right ? last : xlm) : (cx(i) < 0 ? (right ? xrp : x0) : (right ? xr : xl));
-        v = __ldg(base + (size_t)i * N + row + xs);
+        v = __ldg(base + (long long)i * N + row + ((right ? last + 1 : x0 - 1) - cx(i)));
       }
       v += __shfl_xor_sync(0xffffffffu, v, 1);
       v += __shfl_xor_sync(0xffffffffu, v, 2);
@@ -196,9 +198,9 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
     __syncthreads();
     if (k >= 2 && active) {
       const int rc = r - 1;
-      const unsigned m = MASKED ? p.mask[(size_t)rc * nx + x] : 0u;
+      const unsigned m = MASKED ? p.mask[(size_t)rc * p.mpitch + x] : 0u;
       finish2<TAU_ONE>(p, ring_m, ring_g, (k - 2) & 3, (k - 1) & 3, k & 3, jc, m, pm, pg, rm_p, jxm_p, jym_p,
-                       rg_p, jxg_p, jyg_p, dst, dstg, (size_t)rc * nx + x, bad);
+                       rg_p, jxg_p, jyg_p, dst, dstg, (size_t)rc * p.pitch + x, x, bad);
     }
     if (!TAU_ONE) {
 #pragma unroll
@@ -221,9 +223,9 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
 // The same march with the 18 source rows of every output row (with a
 // 16-byte halo) copied into shared-memory stages by cp.async.bulk, issued
 // NSTAGE - 1 rows ahead by a ninth warp that also sums the four halo cells
-// (melt and gas, left and right) lane-parallel. Needs nx % 16 == 0 (16-byte
-// rows and mask pieces) and nx >= kBX2C + 16 (a staged row wraps at most
-// once).
+// (melt and gas, left and right) lane-parallel. A ragged last strip copies
+// whole windows too; what lies beyond the ghosts is not used, and the slices
+// after the buffer and the mask keep the over-read inside the workspace.
 constexpr int kPad2C = 4;                        // halo pad: 16 bytes of FP32
 constexpr int kWin2C = kBX2C + 2 * kPad2C;       // floats per staged row
 constexpr int kRow2C = kWin2C * 4;               // bytes, a multiple of 16
@@ -248,7 +250,7 @@ __device__ __forceinline__ void issue2c(const Step2Params& p, unsigned char* sta
   unsigned char* st = stages + (size_t)slot * STAGE;
   uint64_t* bar = bars + slot;
   const int r = y0 - 1 + k;
-  const int ny = p.ny, nx = p.nx;
+  const int ny = p.ny;
   if (lane < 2 * Q + (MASKED ? 1 : 0)) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (lane == 0) mbar_expect_tx(bar, STAGE);
   __syncwarp();
@@ -257,11 +259,11 @@ __device__ __forceinline__ void issue2c(const Step2Params& p, unsigned char* sta
     int g = r - cy(i);
     g = g < 0 ? g + ny : (g >= ny ? g - ny : g);
     g = g < 0 ? g + ny : (g >= ny ? g - ny : g);
-    const float* row = static_cast<const float*>(p.src) + (size_t)lane * p.N + (size_t)g * nx;
-    copy_row_wrapped<float>(reinterpret_cast<float*>(st + lane * kRow2C), row, x0 - kPad2C, kWin2C, nx, bar);
+    const float* row = static_cast<const float*>(p.src) + (long long)lane * p.plane + (long long)g * p.pitch;
+    bulk_g2s(st + lane * kRow2C, row + (x0 - kPad2C), kRow2C, bar);
   } else if (MASKED && lane == 2 * Q) {
     const int g = r < 0 ? r + ny : (r >= ny ? r - ny : r);
-    copy_row_wrapped<uint8_t>(st + 2 * Q * kRow2C, p.mask + (size_t)g * nx, x0, kBX2C, nx, bar);
+    bulk_g2s(st + 2 * Q * kRow2C, p.mask + (long long)g * p.mpitch + x0, kBX2C, bar);
   }
 }
 
@@ -292,7 +294,7 @@ __device__ __forceinline__ bool march2c(const Step2Params& p, const Smem2C<MASKE
                                         unsigned& gstage, int& bad) {
   constexpr int STAGE = stage2c_bytes<MASKED>();
   float* __restrict__ dst = static_cast<float*>(p.dst);
-  float* __restrict__ dstg = dst + (size_t)Q * p.N;
+  float* __restrict__ dstg = dst + (size_t)Q * p.plane;
   const int nx = p.nx;
   const int tid = threadIdx.x;
   const bool helper = tid >= kBX2C;
@@ -359,7 +361,7 @@ __device__ __forceinline__ bool march2c(const Step2Params& p, const Smem2C<MASKE
     } else if (k >= 2 && active) {
       const int rc = y0 + k - 2;
       finish2<TAU_ONE>(p, sm.ring_m, sm.ring_g, (k - 2) & 3, (k - 1) & 3, k & 3, jc, m_prev, pm, pg, rm_p, jxm_p,
-                       jym_p, rg_p, jxg_p, jyg_p, dst, dstg, (size_t)rc * nx + x0 + tid, bad);
+                       jym_p, rg_p, jxg_p, jyg_p, dst, dstg, (size_t)rc * p.pitch + x0 + tid, x0 + tid, bad);
     }
     if (!TAU_ONE) {
 #pragma unroll
@@ -467,21 +469,21 @@ cudaError_t launch_step2_tma(const Step2Params& p, cudaStream_t s) {
 __global__ void k_fields2(const Step2Params p, float* __restrict__ rho_m, float* __restrict__ rho_g,
                           float* __restrict__ ux, float* __restrict__ uy, float* __restrict__ pr) {
   const float* src = static_cast<const float*>(p.src);
-  const long long N = p.N;
+  const long long N = (long long)p.nx * p.ny, P = p.plane;
   const int nx = p.nx, ny = p.ny;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
        c += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(c % nx), y = (int)(c / nx);
-    const unsigned m = p.mask ? p.mask[c] : 0u;
+    const unsigned m = p.mask ? p.mask[(size_t)y * p.mpitch + x] : 0u;
     float Sm[2] = {0.f, 0.f}, Sg[2] = {0.f, 0.f}, own[2] = {0.f, 0.f};
     float rm = 0.f, rg = 0.f, jx = 0.f, jy = 0.f;
     // densities of the cell and the neighbour sums from the neighbours' densities
     for (int i = 0; i < Q; ++i) {
-      const int xx = wrap_1(x + cx(i), nx), yy = wrap_1(y + cy(i), ny);
+      const int xx = x + cx(i), yy = wrap_1(y + cy(i), ny);
       float a = 0.f, b = 0.f, ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f;
       for (int j = 0; j < Q; ++j) {
-        const size_t idx = (size_t)wrap_1(yy - cy(j), ny) * nx + wrap_1(xx - cx(j), nx);
-        const float fa = src[(size_t)j * N + idx], fb = src[(size_t)(9 + j) * N + idx];
+        const long long idx = (long long)wrap_1(yy - cy(j), ny) * p.pitch + (xx - cx(j));
+        const float fa = src[j * P + idx], fb = src[(9 + j) * P + idx];
         a += fa;
         b += fb;
         ax += cx(j) * fa;
@@ -522,9 +524,12 @@ __global__ void k_fields2(const Step2Params p, float* __restrict__ rho_m, float*
 
 }  // namespace
 
+// Narrower boxes march with plain loads: a staged window copies whole strips.
+static constexpr int kStaged2C = 256;
+
 cudaError_t launch_step2(const Step2Params& p, cudaStream_t s) {
   const bool one = p.tau_m == 1.0f && p.tau_g == 1.0f;
-  if (p.nx % 16 == 0 && p.nx >= kBX2C + 16) {  // staged rows
+  if (p.nx >= kStaged2C) {
     if (p.mask) return one ? launch_step2_tma<true, true>(p, s) : launch_step2_tma<true, false>(p, s);
     return one ? launch_step2_tma<false, true>(p, s) : launch_step2_tma<false, false>(p, s);
   }
@@ -547,7 +552,7 @@ cudaError_t launch_step2(const Step2Params& p, cudaStream_t s) {
 
 cudaError_t launch_fields2(const Step2Params& p, float* rho_m, float* rho_g, float* ux, float* uy, float* pr,
                            cudaStream_t s) {
-  long long b = (p.N + 255) / 256;
+  long long b = ((long long)p.nx * p.ny + 255) / 256;
   if (b > device_sm_count() * 8LL) b = device_sm_count() * 8LL;
   k_fields2<<<(unsigned)b, 256, 0, s>>>(p, rho_m, rho_g, ux, uy, pr);
   return cudaGetLastError();

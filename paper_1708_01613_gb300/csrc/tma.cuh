@@ -56,15 +56,5 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
-// Copy len elements of a periodic row starting at column start (may be
-// negative) into dst, in one or two pieces (len <= row length).
-template <typename T>
-__device__ __forceinline__ void copy_row_wrapped(T* dst, const T* row, int start, int len, int nx, uint64_t* bar) {
-  const int s0 = start < 0 ? start + nx : start;
-  const int first = min(len, nx - s0);
-  bulk_g2s(dst, row + s0, (uint32_t)(first * sizeof(T)), bar);
-  if (first < len) bulk_g2s(dst + first, row, (uint32_t)((len - first) * sizeof(T)), bar);
-}
-
 }  // namespace
 }  // namespace lbm
