@@ -567,6 +567,10 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   if (rc) return rc;
   const lbm_config& c = h->cfg;
   StepParams p = handle_step_params(h);
+  // between two steps of this call without a relabel the tile kernel's
+  // pull does the bounce-back
+  const bool pulls = c.barrier && c.components == 1 && step_tiles(c.storage, p);
+  p.pull_bounce = 0;
   for (int64_t s = 0; s < nsteps && !h->halted; ++s) {
     bool stop_after = false;
     if (c.barrier && h->t % c.relabel_every == 0) {
@@ -601,8 +605,11 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
       h->launches += 1;
     }
     if (c.barrier) {  // populations that would cross a blocked edge bounce back
-      CUDA_TRY(h, bounce_after_step(h));
-      h->launches += 1;
+      p.pull_bounce = pulls && s + 1 < nsteps && !stop_after && (h->t + 1) % c.relabel_every != 0;
+      if (!p.pull_bounce) {
+        CUDA_TRY(h, bounce_after_step(h));
+        h->launches += 1;
+      }
     }
     h->cur ^= 1;
     h->t += 1;

@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "labels.cuh"
+#include "launch.cuh"
 #include "pull.cuh"
 
 namespace lbm {
@@ -129,7 +130,7 @@ __global__ void k_owner(int nx, int ny, int R, const int32_t* __restrict__ L, in
       for (int dx = -R; dx <= R; ++dx) {
         const int d2 = dx * dx + dy * dy;
         if (d2 > R * R || d2 > bd) continue;
-        const int l = __ldg(L + row + wrapi(x + dx, nx));
+        const int l = __ldcg(L + row + wrapi(x + dx, nx));
         if (l < 0) continue;
         if (d2 < bd) {
           bd = d2;
@@ -418,6 +419,7 @@ __device__ __forceinline__ int find_entry(const RelabelEntry* __restrict__ e, in
 template <int S, bool TWO>
 __global__ void __launch_bounds__(kTX * kTY) kb_density_label(const RelabelBox* __restrict__ boxes,
                                                               const RelabelEntry* __restrict__ e, int m, int parity) {
+  grid_begin();
   using T = typename Store<S>::T;
   const int k = find_entry<kOffTiles>(e, m, blockIdx.x);
   const RelabelBox& B = boxes[e[k].box];
@@ -444,7 +446,7 @@ __global__ void __launch_bounds__(kTX * kTY) kb_density_label(const RelabelBox* 
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       const size_t row = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
-      g += __ldg(pg + (size_t)i * P + row + (x - cx(i)));
+      g += __ldcg(pg + (size_t)i * P + row + (x - cx(i)));
     }
     const float a = B.rho0 * (1.0f - expf(-r / B.rho0)), b = B.rho0 * (1.0f - expf(-g / B.rho0));
     B.pr[c] = (r + g) * (1.0f / 3.0f) + (B.G * a * a + 2.0f * B.G_mg * a * b + B.G_gg * b * b) * (1.0f / 6.0f);
@@ -536,6 +538,7 @@ template <int S>
 __global__ void __launch_bounds__(kTX / 4 * kTY, 16) kb_density_label4(const RelabelBox* __restrict__ boxes,
                                                                        const RelabelEntry* __restrict__ e, int m,
                                                                        int parity) {
+  grid_begin();
   using T = typename Store<S>::T;
   const int k = find_entry<kOffTiles>(e, m, blockIdx.x);
   const RelabelBox& B = boxes[e[k].box];
@@ -555,6 +558,7 @@ __global__ void __launch_bounds__(kTX / 4 * kTY, 16) kb_density_label4(const Rel
 // relabel) to the box's list; the order of the list does not affect any
 // result.
 __global__ void kb_active(const RelabelBox* __restrict__ boxes, const RelabelEntry* __restrict__ e, int m) {
+  grid_begin();
   const int k = find_entry<kOffScan>(e, m, blockIdx.x);
   const RelabelBox& B = boxes[e[k].box];
   const int t = (blockIdx.x - e[k].off_scan) * blockDim.x + threadIdx.x;
@@ -593,6 +597,7 @@ __device__ __forceinline__ ListWalk list_walk(const RelabelBox* __restrict__ box
 
 __global__ void __launch_bounds__(kTX * kTY) kb_union(const RelabelBox* __restrict__ boxes,
                                                       const RelabelEntry* __restrict__ e, int m) {
+  grid_begin();
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
   const int nx = B.nx, ny = B.ny;
@@ -623,6 +628,7 @@ __global__ void __launch_bounds__(kTX * kTY) kb_union(const RelabelBox* __restri
 
 __global__ void __launch_bounds__(kTX * kTY) kb_flatten(const RelabelBox* __restrict__ boxes,
                                                         const RelabelEntry* __restrict__ e, int m) {
+  grid_begin();
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
   int32_t* L = B.label;
@@ -643,6 +649,7 @@ __global__ void __launch_bounds__(kTX * kTY) kb_flatten(const RelabelBox* __rest
 // holds the earlier labels the density phase parked there.
 __global__ void __launch_bounds__(kTX * kTY) kb_merge(const RelabelBox* __restrict__ boxes,
                                                       const RelabelEntry* __restrict__ e, int m) {
+  grid_begin();
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
   int n = 0;
@@ -692,6 +699,7 @@ __device__ __forceinline__ int nearest_label(const int* row0) {
 
 __global__ void __launch_bounds__(kTX * kTY) kb_owner(const RelabelBox* __restrict__ boxes,
                                                       const RelabelEntry* __restrict__ e, int m) {
+  grid_begin();
   __shared__ int32_t sl[(kTY + 2 * kOMaxR) * (kTX + 2 * kOMaxR)];
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
@@ -729,6 +737,7 @@ __global__ void __launch_bounds__(kTX * kTY) kb_owner(const RelabelBox* __restri
 template <bool TWO>
 __global__ void __launch_bounds__(kTX * kTY) kb_rupture(const RelabelBox* __restrict__ boxes,
                                                         const RelabelEntry* __restrict__ e, int m) {
+  grid_begin();
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
   const int nx = B.nx, ny = B.ny;
@@ -782,6 +791,7 @@ __global__ void __launch_bounds__(kTX * kTY) kb_rupture(const RelabelBox* __rest
 // tiles outside the list are inactive in both, so only listed tiles change.
 __global__ void __launch_bounds__(kTX * kTY) kb_mask(const RelabelBox* __restrict__ boxes,
                                                      const RelabelEntry* __restrict__ e, int m) {
+  grid_begin();
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
   const int nx = B.nx, ny = B.ny;
@@ -863,6 +873,7 @@ __global__ void k_bounce(T* __restrict__ pops, const uint8_t* __restrict__ mask,
 template <typename T, bool TWO>
 __global__ void __launch_bounds__(kTX * kTY) kb_bounce(const RelabelBox* __restrict__ boxes,
                                                        const RelabelEntry* __restrict__ e, int m, int q) {
+  grid_begin();
   const ListWalk lw = list_walk(boxes, e, m);
   const RelabelBox& B = *lw.B;
   T* pops = static_cast<T*>(const_cast<void*>(B.pops[B.cur ^ q]));
@@ -966,29 +977,29 @@ cudaError_t launch_relabel_boxes(int storage, const RelabelBox* boxes, const Rel
   const dim3 block(kTX, kTY);
   if (two) {  // two components: FP32 only
     if (storage != LBM_F32) return cudaErrorInvalidValue;
-    kb_density_label<LBM_F32, true><<<totals[0], block, 0, s>>>(boxes, entries, m, parity);
+    LBM_TRY(launch_chain(kb_density_label<LBM_F32, true>, dim3(totals[0]), block, 0, s, boxes, entries, m, parity));
   } else {
     switch (storage) {
       case LBM_F32: 
-        kb_density_label4<LBM_F32><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
+        LBM_TRY(launch_chain(kb_density_label4<LBM_F32>, dim3(totals[0]), dim3(kTX / 4, kTY), 0, s, boxes, entries, m, parity));
         break;
       case LBM_F16_DEV:
-        kb_density_label4<LBM_F16_DEV><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
+        LBM_TRY(launch_chain(kb_density_label4<LBM_F16_DEV>, dim3(totals[0]), dim3(kTX / 4, kTY), 0, s, boxes, entries, m, parity));
         break;
       case LBM_BF16_DEV:
-        kb_density_label4<LBM_BF16_DEV><<<totals[0], dim3(kTX / 4, kTY), 0, s>>>(boxes, entries, m, parity);
+        LBM_TRY(launch_chain(kb_density_label4<LBM_BF16_DEV>, dim3(totals[0]), dim3(kTX / 4, kTY), 0, s, boxes, entries, m, parity));
         break;
       default: return cudaErrorInvalidValue;
     }
   }
-  kb_active<<<totals[1], kThreads, 0, s>>>(boxes, entries, m);
-  kb_union<<<totals[2], block, 0, s>>>(boxes, entries, m);
-  kb_flatten<<<totals[2], block, 0, s>>>(boxes, entries, m);
-  kb_merge<<<totals[2], block, 0, s>>>(boxes, entries, m);
-  kb_owner<<<totals[2], block, 0, s>>>(boxes, entries, m);
-  if (two) kb_rupture<true><<<totals[2], block, 0, s>>>(boxes, entries, m);
-  else kb_rupture<false><<<totals[2], block, 0, s>>>(boxes, entries, m);
-  kb_mask<<<totals[2], block, 0, s>>>(boxes, entries, m);
+  LBM_TRY(launch_chain(kb_active, dim3(totals[1]), dim3(kThreads), 0, s, boxes, entries, m));
+  LBM_TRY(launch_chain(kb_union, dim3(totals[2]), block, 0, s, boxes, entries, m));
+  LBM_TRY(launch_chain(kb_flatten, dim3(totals[2]), block, 0, s, boxes, entries, m));
+  LBM_TRY(launch_chain(kb_merge, dim3(totals[2]), block, 0, s, boxes, entries, m));
+  LBM_TRY(launch_chain(kb_owner, dim3(totals[2]), block, 0, s, boxes, entries, m));
+  if (two) LBM_TRY(launch_chain(kb_rupture<true>, dim3(totals[2]), block, 0, s, boxes, entries, m));
+  else LBM_TRY(launch_chain(kb_rupture<false>, dim3(totals[2]), block, 0, s, boxes, entries, m));
+  LBM_TRY(launch_chain(kb_mask, dim3(totals[2]), block, 0, s, boxes, entries, m));
   return cudaGetLastError();
 }
 
@@ -1010,11 +1021,11 @@ cudaError_t launch_bounce_boxes(int storage, bool two, const RelabelBox* boxes, 
   const dim3 block(kTX, kTY);
   if (two) {
     if (storage != LBM_F32) return cudaErrorInvalidValue;
-    kb_bounce<uint32_t, true><<<total_list, block, 0, s>>>(boxes, entries, m, q);
+    LBM_TRY(launch_chain(kb_bounce<uint32_t, true>, dim3(total_list), block, 0, s, boxes, entries, m, q));
   } else if (storage == LBM_F32) {
-    kb_bounce<uint32_t, false><<<total_list, block, 0, s>>>(boxes, entries, m, q);
+    LBM_TRY(launch_chain(kb_bounce<uint32_t, false>, dim3(total_list), block, 0, s, boxes, entries, m, q));
   } else {
-    kb_bounce<uint16_t, false><<<total_list, block, 0, s>>>(boxes, entries, m, q);
+    LBM_TRY(launch_chain(kb_bounce<uint16_t, false>, dim3(total_list), block, 0, s, boxes, entries, m, q));
   }
   return cudaGetLastError();
 }

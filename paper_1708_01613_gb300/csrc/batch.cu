@@ -63,7 +63,8 @@ struct lbm_batch {
   RelabelEntry* d_bent = nullptr;
   std::vector<int> bounce_first;          // tiled boxes among the first k stepping boxes
   std::vector<int> bounce_ctas;           // list CTAs of the first k tiled boxes
-  int strip = 512, rows = 0;
+  int strip = 512, rows = 0;   // work items of the staged kernel (lbm_batch_set_tiles)
+  int tiled = 0;               // the current item list is for the tile kernel (tile.cu)
   int use_graph = 1;
   int dirty = 1;               // descriptors/items must be re-uploaded
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // K-step block starting at parity 0 / 1
@@ -109,6 +110,32 @@ void drop_graphs(lbm_batch* b) {
     }
 }
 
+// Items of the tile kernel: one CTA's tile each.
+void build_tile_items(lbm_batch* b) {
+  int cols, rows;
+  tile_item_size(b->storage, b->tau_one != 0, &cols, &rows);
+  for (int i = 0; i < b->n; ++i) {
+    if (!b->active[i]) continue;
+    const int nx = b->h[i]->cfg.nx, ny = b->h[i]->cfg.ny;
+    for (int y0 = 0; y0 < ny; y0 += rows)
+      for (int x0 = 0; x0 < nx; x0 += cols)
+        b->items.push_back({i, x0, std::min(cols, nx - x0), y0, std::min(y0 + rows, ny)});
+  }
+  b->nitems = (int)b->items.size();
+}
+
+// Whether the active boxes step with the tile kernel: it needs no
+// minimum width and beats the staged kernel while the state is small.
+bool batch_tiles(const lbm_batch* b) {
+  long long cells = 0;
+  for (int i = 0; i < b->n; ++i) {
+    if (!b->active[i]) continue;
+    if (!tile_fits(b->storage, b->h[i]->shape.plane)) return false;
+    cells += (long long)b->h[i]->cfg.nx * b->h[i]->cfg.ny;
+  }
+  return cells <= tile_cells(b->storage, b->tau_one != 0);
+}
+
 // Work items. A CTA walks its item row by row, each row a dependent
 // load-compute-store round of a few microseconds, so a launch lasts about
 // (rows per item) x (items per CTA) such rounds. While the tuned height
@@ -122,6 +149,8 @@ void drop_graphs(lbm_batch* b) {
 // too.
 void build_items(lbm_batch* b, bool spread) {
   b->items.clear();
+  b->tiled = batch_tiles(b);
+  if (b->tiled) return build_tile_items(b);
   const int res = std::max(1, batch_resident_ctas(b->storage, b->masked != 0, b->tau_one != 0));
   auto count = [&](int rows) {
     long long c = 0;
@@ -301,9 +330,16 @@ int enqueue_relabel(lbm_batch* b, int parity, int64_t j, int live, Stepping step
   return LBM_OK;
 }
 
-// The batched kernel of one step over the first n items.
-int enqueue_items(lbm_batch* b, int parity, int n) {
+// The batched kernel of one step over the first n items; pull_bounce: the step
+// before left its bounce-back to this one (tile kernel only).
+int enqueue_items(lbm_batch* b, int parity, int n, bool pull_bounce) {
   if (n <= 0) return LBM_OK;
+  if (b->tiled) {
+    BCUDA(b, launch_tile_batch(b->storage, b->masked != 0, b->tau_one != 0, b->d_insts, b->d_items, n, parity,
+                                pull_bounce, b->stream));
+    b->launches += 1;
+    return LBM_OK;
+  }
   BCUDA(b, launch_step_batch(b->storage, b->masked != 0, b->tau_one != 0, b->d_insts, b->d_items, n, b->d_counter,
                              parity, b->stream));
   b->launches += 1;
@@ -314,6 +350,7 @@ int enqueue_items(lbm_batch* b, int parity, int n) {
 // each, on the buffers of parity `parity`, on the batch stream.
 template <class Stepping>
 int enqueue_lone(lbm_batch* b, int parity, Stepping stepping) {
+  if (b->tiled) return LBM_OK;  // every width is in the item list
   for (int i = 0; i < b->n; ++i) {
     if (!b->lone[i] || !stepping(i)) continue;
     lbm_handle* h = b->h[i];
@@ -358,15 +395,29 @@ void advance(lbm_batch* b, int64_t n) {
     }
 }
 
+// Whether any box relabels at batch count T.
+bool relabel_due(const lbm_batch* b, int64_t T) {
+  const int r = b->h[0]->cfg.relabel_every;
+  if (b->groups.count((int)(T % r))) return true;
+  for (int i : b->untiled)
+    if ((b->h[i]->t + (T - b->t)) % r == 0) return true;
+  return false;
+}
+
 // Enqueues one step `j` steps after the boxes' current state (relabel of
-// every box whose own step count is then due, then the batched kernel).
-int enqueue_step(lbm_batch* b, int parity, int64_t j) {
+// every box whose own step count is then due, then the batched kernel). With
+// `more` another step of the same run of steps follows: unless a box relabels
+// there, its pull does the bounce-back (`pull`: this step's pull does the one
+// before; updated for the next).
+int enqueue_step(lbm_batch* b, int parity, int64_t j, bool more, bool& pull) {
   int rc;
   if (b->masked && (rc = enqueue_relabel(b, parity, j, -1, [&](int i) { return b->active[i] != 0; })))
     return rc;
-  if ((rc = enqueue_items(b, parity, b->nitems))) return rc;
+  if ((rc = enqueue_items(b, parity, b->nitems, pull))) return rc;
   if ((rc = enqueue_lone(b, parity, [&](int i) { return b->active[i] != 0; }))) return rc;
-  if (b->masked && (rc = enqueue_bounce(b, parity, -1, [&](int i) { return b->active[i] != 0; }))) return rc;
+  if (!b->masked) return LBM_OK;
+  pull = b->tiled && more && !relabel_due(b, b->t + j + 1);
+  if (!pull && (rc = enqueue_bounce(b, parity, -1, [&](int i) { return b->active[i] != 0; }))) return rc;
   return LBM_OK;
 }
 
@@ -375,7 +426,8 @@ int build_graph(lbm_batch* b, int start_parity) {
   BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   const int64_t saved = b->launches;
   int rc = LBM_OK;
-  for (int j = 0; j < b->K && rc == LBM_OK; ++j) rc = enqueue_step(b, start_parity ^ (j & 1), j);
+  bool pull = false;
+  for (int j = 0; j < b->K && rc == LBM_OK; ++j) rc = enqueue_step(b, start_parity ^ (j & 1), j, j + 1 < b->K, pull);
   const cudaError_t e = cudaStreamEndCapture(b->stream, &g);
   b->graph_launches[start_parity] = b->launches - saved;
   b->launches = saved;  // counted again at every replay
@@ -554,12 +606,13 @@ int lbm_batch_step(lbm_batch* b, int64_t nsteps) {
   rc = upload(b);
   if (rc) return rc;
   int64_t left = nsteps;
+  bool pull = false;
   // blocks start where the batch counter is a multiple of K; each box's
   // relabel offset to that counter is fixed while the membership is, so a
   // block's relabel schedule (captured in the graph) repeats; buffer parity
   // repeats after 2K steps (two graphs)
   while (left > 0 && b->use_graph && b->t % b->K != 0) {
-    if ((rc = enqueue_step(b, b->par, 0))) return rc;
+    if ((rc = enqueue_step(b, b->par, 0, left > 1 && (b->t + 1) % b->K != 0, pull))) return rc;
     advance(b, 1);
     --left;
   }
@@ -572,7 +625,7 @@ int lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     left -= b->K;
   }
   while (left > 0) {
-    if ((rc = enqueue_step(b, b->par, 0))) return rc;
+    if ((rc = enqueue_step(b, b->par, 0, left > 1, pull))) return rc;
     advance(b, 1);
     --left;
   }
@@ -621,6 +674,7 @@ int lbm_batch_step_each(lbm_batch* b, const int64_t* nsteps, int32_t n) {
   std::map<int, int> glive;  // members of each barrier group still stepping
   for (const auto& kv : b->groups) glive[kv.first] = (int)kv.second.members.size();
   size_t live = order.size();
+  bool pull = false;
   for (int64_t j = 0; j < most; ++j) {
     while (live > 0 && nsteps[order[live - 1]] <= j) --live;
     const int parity = (int)(j & 1);
@@ -636,9 +690,12 @@ int lbm_batch_step_each(lbm_batch* b, const int64_t* nsteps, int32_t n) {
       }
       if ((rc = enqueue_relabel(b, parity, j, gl, [&](int i) { return nsteps[i] > j; }))) return rc;
     }
-    if ((rc = enqueue_items(b, parity, prefix[live]))) return rc;
+    if ((rc = enqueue_items(b, parity, prefix[live], pull))) return rc;
     if ((rc = enqueue_lone(b, parity, [&](int i) { return nsteps[i] > j; }))) return rc;
-    if (b->masked && (rc = enqueue_bounce(b, parity, (int)live, [&](int i) { return nsteps[i] > j; }))) return rc;
+    if (!b->masked) continue;
+    // the next step's pull does the bounce-back where it steps the same boxes and none relabels
+    pull = b->tiled && nsteps[order[live - 1]] > j + 1 && !relabel_due(b, b->t + j + 1);
+    if (!pull && (rc = enqueue_bounce(b, parity, (int)live, [&](int i) { return nsteps[i] > j; }))) return rc;
   }
   for (int i = 0; i < n; ++i) {
     b->h[i]->t += nsteps[i];

@@ -11,6 +11,7 @@
 //
 // Nucleation: cells within a nucleus radius become gas at rest, incoming
 // f_i(x) = w_i rho_g, i.e. B_i(x - e_i) in the buffer the next step reads.
+#include "launch.cuh"
 #include "lbm_internal.cuh"
 
 namespace lbm {
@@ -42,9 +43,9 @@ __global__ void k_gas_census(const float* __restrict__ rho, long long N, float t
 }
 
 template <int S>
-__global__ void k_growth(typename Store<S>::T* __restrict__ pops, const int32_t* __restrict__ list,
-                         const int* __restrict__ count, int nx, int pitch, long long plane, double rate,
-                         double budget, double* __restrict__ released, int parity) {
+__global__ void k_growth(typename Store<S>::T* pops, const int32_t* list, const int* count, int nx, int pitch,
+                         long long plane, double rate, double budget, double* released, int parity) {
+  grid_begin();
   const int n = *count;
   const double before = released[parity];
   double release = 0.0;
@@ -128,11 +129,11 @@ cudaError_t launch_growth(const FieldParams& fp, void* pops, const int32_t* list
                           double budget, double* released, int parity, cudaStream_t s) {
   const unsigned g = (unsigned)device_sm_count() * 4;
 #define CALL(S, T)                                                                                                   \
-  k_growth<S><<<g, kThreadsG, 0, s>>>(static_cast<T*>(pops), list, count, fp.nx, fp.pitch, fp.plane, rate, budget, \
-                                      released, parity)
+  LBM_TRY(launch_chain(k_growth<S>, dim3(g), dim3(kThreadsG), 0, s, static_cast<T*>(pops), list, count, fp.nx, fp.pitch, \
+                       fp.plane, rate, budget, released, parity))
   LBM_BY_STORAGE(fp.storage, CALL)
 #undef CALL
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 cudaError_t launch_nucleate(const FieldParams& fp, void* pops, const lbm_bubble* nuclei, int n, double rho_g,

@@ -54,11 +54,11 @@ template <>
 struct Store<LBM_F32> {
   using T = float;
   static constexpr int bytes = 4;
-  __device__ static __forceinline__ float load(const T* p, size_t i, float) { return __ldg(p + i); }
+  __device__ static __forceinline__ float load(const T* p, size_t i, float) { return __ldcg(p + i); }
   __device__ static __forceinline__ float load_smem(const T* p, int i, float) { return p[i]; }
   __device__ static __forceinline__ T of(float v, float) { return v; }
   // raw stored value (FP32: the population itself)
-  __device__ static __forceinline__ float raw(const T* p, size_t i) { return __ldg(p + i); }
+  __device__ static __forceinline__ float raw(const T* p, size_t i) { return __ldcg(p + i); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return p[i]; }
   __device__ static __forceinline__ void store_raw(T* p, size_t i, float v) { p[i] = v; }
   __device__ static __forceinline__ T enc(float v) { return v; }
@@ -69,7 +69,7 @@ struct Store<LBM_F16_DEV> {
   using T = __half;
   static constexpr int bytes = 2;
   __device__ static __forceinline__ float load(const T* p, size_t i, float base) {
-    return __fadd_rn(base, __half2float(__ldg(p + i)));
+    return __fadd_rn(base, __half2float(__ldcg(p + i)));
   }
   __device__ static __forceinline__ float load_smem(const T* p, int i, float base) {
     return __fadd_rn(base, __half2float(p[i]));
@@ -77,7 +77,7 @@ struct Store<LBM_F16_DEV> {
   // the stored word of a full population value
   __device__ static __forceinline__ T of(float v, float base) { return __float2half_rn(__fsub_rn(v, base)); }
   // raw stored value: the deviation g = f - w_i rho_ref
-  __device__ static __forceinline__ float raw(const T* p, size_t i) { return __half2float(__ldg(p + i)); }
+  __device__ static __forceinline__ float raw(const T* p, size_t i) { return __half2float(__ldcg(p + i)); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return __half2float(p[i]); }
   __device__ static __forceinline__ void store_raw(T* p, size_t i, float g) { p[i] = __float2half_rn(g); }
   __device__ static __forceinline__ T enc(float g) { return __float2half_rn(g); }
@@ -88,13 +88,13 @@ struct Store<LBM_BF16_DEV> {
   using T = __nv_bfloat16;
   static constexpr int bytes = 2;
   __device__ static __forceinline__ float load(const T* p, size_t i, float base) {
-    return __fadd_rn(base, __bfloat162float(__ldg(p + i)));
+    return __fadd_rn(base, __bfloat162float(__ldcg(p + i)));
   }
   __device__ static __forceinline__ float load_smem(const T* p, int i, float base) {
     return __fadd_rn(base, __bfloat162float(p[i]));
   }
   __device__ static __forceinline__ T of(float v, float base) { return __float2bfloat16_rn(__fsub_rn(v, base)); }
-  __device__ static __forceinline__ float raw(const T* p, size_t i) { return __bfloat162float(__ldg(p + i)); }
+  __device__ static __forceinline__ float raw(const T* p, size_t i) { return __bfloat162float(__ldcg(p + i)); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return __bfloat162float(p[i]); }
   __device__ static __forceinline__ void store_raw(T* p, size_t i, float g) { p[i] = __float2bfloat16_rn(g); }
   __device__ static __forceinline__ T enc(float g) { return __float2bfloat16_rn(g); }
@@ -169,6 +169,7 @@ struct StepParams {
   int pitch, mpitch;     // row strides: population values, mask bytes (src, dst and mask point at column 0)
   long long plane;       // plane stride
   int rows_per_chunk;    // rows marched by one CTA
+  int pull_bounce;       // tile kernel: src holds populations that have not bounced back yet
   int force_generic;     // kernel variant: 0 automatic, 1 plain loads, 2 one-cell staged, 3 two-cell staged,
                          // 4 two-cell staged with dynamically scheduled row chunks
   float tau, inv_tau, G, rho0, inv_rho0;
@@ -219,6 +220,19 @@ int device_sm_count();
 
 // Launch of the fused step (step.cu). Returns a cudaError_t.
 cudaError_t launch_step(int storage, const StepParams& p, cudaStream_t s);
+// Whether launch_step takes the tile kernel (tile.cu) for this box (automatic
+// variant): then the bounce-back of the step before may be left to the pull
+// (pull_bounce).
+bool step_tiles(int storage, const StepParams& p);
+cudaError_t launch_tile(int storage, const StepParams& p, cudaStream_t s);
+// The same over many boxes, items of at most cols x rows cells (x0 a multiple
+// of cols). Boxes need tile_fits.
+bool tile_fits(int storage, long long plane);
+void tile_item_size(int storage, bool tau_one, int* cols, int* rows);
+// Cells up to which the tile kernel beats the staged ones.
+long long tile_cells(int storage, bool tau_one);
+cudaError_t launch_tile_batch(int storage, bool masked, bool tau_one, const BatchInst* insts, const BatchItem* items,
+                              int nitems, int parity, bool pull_bounce, cudaStream_t s);
 // Launch geometry the fused step uses for a box (for tests/benchmarks).
 void step_geometry(int nx, int ny, int* grid_x, int* grid_y, int* rows_per_chunk, int* block);
 // Widths the staged variants accept (lbm_set_step_variant): 2 takes widths

@@ -34,27 +34,27 @@ __device__ __forceinline__ void pull4(const typename Store<S>::T* __restrict__ p
     const size_t at = (size_t)i * plane + (cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0));
     if constexpr (S == LBM_F32) {
       const float* q = pops + at;
-      const float4 w = __ldg(reinterpret_cast<const float4*>(q));  // columns x .. x + 3
+      const float4 w = __ldcg(reinterpret_cast<const float4*>(q));  // columns x .. x + 3
       if (cx(i) > 0) {  // columns x - 1 .. x + 2
-        fa[i] = make_float2(__ldg(q - 1), w.x);
+        fa[i] = make_float2(__ldcg(q - 1), w.x);
         fb[i] = make_float2(w.y, w.z);
       } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
         fa[i] = make_float2(w.y, w.z);
-        fb[i] = make_float2(w.w, __ldg(q + 4));
+        fb[i] = make_float2(w.w, __ldcg(q + 4));
       } else {
         fa[i] = make_float2(w.x, w.y);
         fb[i] = make_float2(w.z, w.w);
       }
     } else {
       const unsigned short* q = reinterpret_cast<const unsigned short*>(pops) + at;
-      const uint2 w = __ldg(reinterpret_cast<const uint2*>(q));  // columns x .. x + 3
+      const uint2 w = __ldcg(reinterpret_cast<const uint2*>(q));  // columns x .. x + 3
       uint32_t lo = w.x, hi = w.y;
       if (cx(i) > 0) {  // columns x - 1 .. x + 2
-        const uint32_t wm = __ldg(reinterpret_cast<const uint32_t*>(q - 2));
+        const uint32_t wm = __ldcg(reinterpret_cast<const uint32_t*>(q - 2));
         lo = __byte_perm(wm, w.x, 0x5432);
         hi = __byte_perm(w.x, w.y, 0x5432);
       } else if (cx(i) < 0) {  // columns x + 1 .. x + 4
-        const uint32_t wp = __ldg(reinterpret_cast<const uint32_t*>(q + 4));
+        const uint32_t wp = __ldcg(reinterpret_cast<const uint32_t*>(q + 4));
         lo = __byte_perm(w.x, w.y, 0x5432);
         hi = __byte_perm(w.y, wp, 0x5432);
       }

@@ -37,6 +37,7 @@
 // (the rest of the row, the next row, after the last row the workspace's next
 // slice) are never used.
 #include "cellmath.cuh"
+#include "launch.cuh"
 #include "tma.cuh"
 
 namespace lbm {
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kBX) k_step_strip(const StepParams p) {
   const int last = min(x0 + kBX, nx) - 1;
   const int y0 = blockIdx.y * p.rows_per_chunk;
   const int y1 = min(y0 + p.rows_per_chunk, ny);
+  grid_begin();
   if (y0 >= y1) return;  // uniform over the block
   const int jc = tid + 1;
 
@@ -212,7 +214,6 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_tma(const StepParams
   const bool active = !helper && tid < width;
   const int y0 = blockIdx.y * p.rows_per_chunk;
   const int y1 = min(y0 + p.rows_per_chunk, ny);
-  if (y0 >= y1) return;
   const int nst = (y1 - y0) + 2;  // stages = rows y0-1 .. y1
 
   if (tid == 0) {
@@ -221,6 +222,8 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_tma(const StepParams
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  grid_begin();
+  if (y0 >= y1) return;  // uniform over the block
   if (helper)
     for (int k = 0; k < NSTAGE - 1 && k < nst; ++k) issue_stage<S, MASKED, NSTAGE>(p, src, stages, bars, k, y0, x0, lane);
 
@@ -565,6 +568,7 @@ __device__ __forceinline__ void march2_init(const Tma2Smem<S, MASKED, NSTAGE>& s
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  grid_begin();
 }
 
 // One box, one work item per CTA: strip blockIdx.x (kBX2 columns), row chunk blockIdx.y.
@@ -575,8 +579,8 @@ __global__ void __launch_bounds__(kTmaThreads, MINB) k_step_tma2(const StepParam
   const int x0 = blockIdx.x * kBX2;
   const int y0 = blockIdx.y * p.rows_per_chunk;
   const int y1 = min(y0 + p.rows_per_chunk, p.ny);
-  if (y0 >= y1) return;
   march2_init(sm);
+  if (y0 >= y1) return;
   unsigned gstage = 0;
   uint32_t worst = 0;
   const int width = min(kBX2, p.nx - x0);
@@ -733,22 +737,23 @@ cudaError_t launch_tma(const StepParams& p, cudaStream_t s) {
   tma_geometry(p.nx, p.ny, resident, &gx, &gy, &rows);
   StepParams q = p;
   q.rows_per_chunk = rows;
-  kern<<<dim3(gx, gy), kTmaThreads, smem, s>>>(q);
-  return cudaGetLastError();
+  return launch_chain(kern, dim3(gx, gy), dim3(kTmaThreads), smem, s, q);
 }
 
 // Measured at 8192^2 (FP16): 4 stages at 4 CTAs per SM (56 registers, no
 // spills) beat deeper rings and 3 or 5 CTAs per SM.
 template <int S>
 constexpr int tma2_stages() { return S == LBM_F32 ? 3 : 4; }
-constexpr int kTma2MinBlocks = 4;
+// FP32 stages allow 3 CTAs per SM: its register budget follows
+template <int S, bool TAU_ONE>
+constexpr int tma2_min_blocks() { return TAU_ONE ? (S == LBM_F32 ? 3 : 4) : 2; }
 constexpr int kDynRows = 48;  // row chunk of the dynamically scheduled step
 
 template <int S, bool MASKED, bool TAU_ONE>
 cudaError_t launch_tma2(const StepParams& p, cudaStream_t s) {
   constexpr int NS = tma2_stages<S>();
   // the relaxation blend (tau != 1) keeps both population sets live: fewer CTAs
-  auto kern = k_step_tma2<S, MASKED, TAU_ONE, NS, TAU_ONE ? kTma2MinBlocks : 2>;
+  auto kern = k_step_tma2<S, MASKED, TAU_ONE, NS, tma2_min_blocks<S, TAU_ONE>()>;
   constexpr size_t smem = tma2_smem_bytes_c<S, MASKED, NS>();
   static int resident = 0;  // per instantiation
   if (resident == 0) {
@@ -766,14 +771,13 @@ cudaError_t launch_tma2(const StepParams& p, cudaStream_t s) {
   StepParams q = p;
   q.rows_per_chunk = (p.ny + g - 1) / g;
   const int gy = (p.ny + q.rows_per_chunk - 1) / q.rows_per_chunk;
-  kern<<<dim3(gx, gy), kTmaThreads, smem, s>>>(q);
-  return cudaGetLastError();
+  return launch_chain(kern, dim3(gx, gy), dim3(kTmaThreads), smem, s, q);
 }
 
 template <int S, bool MASKED, bool TAU_ONE>
 cudaError_t launch_dyn(const StepParams& p, cudaStream_t s) {
   constexpr int NS = tma2_stages<S>();
-  auto kern = k_step_dyn<S, MASKED, TAU_ONE, NS, TAU_ONE ? kTma2MinBlocks : 2>;
+  auto kern = k_step_dyn<S, MASKED, TAU_ONE, NS, tma2_min_blocks<S, TAU_ONE>()>;
   constexpr size_t smem = tma2_smem_bytes_c<S, MASKED, NS>();
   static int resident = 0;  // per instantiation: CTAs that fit the GPU at once
   if (resident == 0) {
@@ -800,8 +804,7 @@ cudaError_t launch_dyn(const StepParams& p, cudaStream_t s) {
   // few microseconds, a large part of a small box's step)
   if (p.force_generic == 0 && nitems <= resident) return launch_tma2<S, MASKED, TAU_ONE>(p, s);
   const int grid = nitems < resident ? nitems : resident;
-  kern<<<grid, kTmaThreads, smem, s>>>(p, rows, gx, nitems);
-  return cudaGetLastError();
+  return launch_chain(kern, dim3(grid), dim3(kTmaThreads), smem, s, p, rows, gx, nitems);
 }
 
 template <int S, bool MASKED, bool TAU_ONE>
@@ -810,8 +813,7 @@ cudaError_t launch_strip(const StepParams& p, cudaStream_t s) {
   step_geometry(p.nx, p.ny, &gx, &gy, &rows, &block);
   StepParams q = p;
   q.rows_per_chunk = rows;
-  k_step_strip<S, MASKED, TAU_ONE><<<dim3(gx, gy), block, 0, s>>>(q);
-  return cudaGetLastError();
+  return launch_chain(k_step_strip<S, MASKED, TAU_ONE>, dim3(gx, gy), dim3(block), 0, s, q);
 }
 
 // Variant 0 (automatic): the two-cell staged march over dynamically
@@ -823,6 +825,7 @@ cudaError_t launch_strip(const StepParams& p, cudaStream_t s) {
 template <int S, bool MASKED, bool TAU_ONE>
 cudaError_t launch_variant(const StepParams& p, cudaStream_t s) {
   const int v = p.force_generic;
+  if (step_tiles(S, p)) return launch_tile(S, p, s);
   if ((v == 4 || v == 0) && tma2_ok(p.nx)) return launch_dyn<S, MASKED, TAU_ONE>(p, s);
   if (v == 3 && tma2_ok(p.nx)) return launch_tma2<S, MASKED, TAU_ONE>(p, s);
   if (v == 2 && tma_ok<S>(p.nx)) return launch_tma<S, MASKED, TAU_ONE>(p, s);
@@ -870,7 +873,7 @@ namespace {
 template <int S, bool MASKED, bool TAU_ONE>
 struct BatchKernel {
   static constexpr int NS = tma2_stages<S>();
-  static constexpr int MINB = TAU_ONE ? kTma2MinBlocks : 2;
+  static constexpr int MINB = tma2_min_blocks<S, TAU_ONE>();
   static constexpr size_t SMEM = tma2_smem_bytes_c<S, MASKED, NS>();
   static int resident() {  // CTAs that fit the GPU at once
     static int r = 0;
@@ -889,9 +892,8 @@ struct BatchKernel {
     if (res == 0) return cudaErrorInvalidConfiguration;
     const int grid = nitems < res ? nitems : res;
     if (grid <= 0) return cudaMemsetAsync(counters, 0, 2 * sizeof(int), s);  // no launch resets them
-    k_step_batch<S, MASKED, TAU_ONE, NS, MINB>
-        <<<grid, kTmaThreads, SMEM, s>>>(insts, items, nitems, counters, parity);
-    return cudaGetLastError();
+    return launch_chain(k_step_batch<S, MASKED, TAU_ONE, NS, MINB>, dim3(grid), dim3(kTmaThreads), SMEM, s, insts, items,
+                        nitems, counters, parity);
   }
 };
 

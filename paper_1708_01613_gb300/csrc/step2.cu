@@ -21,6 +21,7 @@
 // the previous row from registers. k_step2_tma (below) is the same march
 // with the rows staged by cp.async.bulk over row chunks drawn from a device
 // counter; both use the per-cell functions here.
+#include "launch.cuh"
 #include "lbm_internal.cuh"
 #include "tma.cuh"
 
@@ -39,7 +40,7 @@ __device__ __forceinline__ void pull9(const float* __restrict__ src, long long p
   for (int i = 0; i < Q; ++i) {
     // f_i(x) = B_i(x - e_i)
     const long long row = cy(i) > 0 ? rowm : (cy(i) < 0 ? rowp : row0);
-    f[i] = __ldg(src + (long long)i * plane + row + (x - cx(i)));
+    f[i] = __ldcg(src + (long long)i * plane + row + (x - cx(i)));
   }
 }
 
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
   const int last = min(x0 + kBX2C, nx) - 1;
   const int y0 = blockIdx.y * p.rows_per_chunk;
   const int y1 = min(y0 + p.rows_per_chunk, ny);
+  grid_begin();
   if (y0 >= y1) return;  // uniform over the block
   const int jc = tid + 1;
 
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(kBX2C, TAU_ONE ? 4 : 2) k_step2_strip(const St
       if (i < Q) {
         const float* base = lane < 16 ? src : srcg;
         const long long row = cy(i) > 0 ? rowm : (cy(i) < 0 ? rowp : row0);
-        v = __ldg(base + (long long)i * N + row + ((right ? last + 1 : x0 - 1) - cx(i)));
+        v = __ldcg(base + (long long)i * N + row + ((right ? last + 1 : x0 - 1) - cx(i)));
       }
       v += __shfl_xor_sync(0xffffffffu, v, 1);
       v += __shfl_xor_sync(0xffffffffu, v, 2);
@@ -408,6 +410,7 @@ __global__ void __launch_bounds__(kThreads2C, MINB) k_step2_tma(const Step2Param
     *sm.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  grid_begin();
   unsigned gstage = 0;
   int bad = 0;
   for (int guard = 0; guard < nitems + 1; ++guard) {
@@ -460,8 +463,7 @@ cudaError_t launch_step2_tma(const Step2Params& p, cudaStream_t s) {
   const long long items = (long long)gx * ((p.ny + rows - 1) / rows);
   if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int nitems = (int)items;
-  kern<<<nitems < resident ? nitems : resident, kThreads2C, smem, s>>>(p, rows, gx, nitems);
-  return cudaGetLastError();
+  return launch_chain(kern, dim3(nitems < resident ? nitems : resident), dim3(kThreads2C), smem, s, p, rows, gx, nitems);
 }
 
 // Diagnostics: melt and gas densities, the physical mixture velocity
@@ -540,14 +542,13 @@ cudaError_t launch_step2(const Step2Params& p, cudaStream_t s) {
   Step2Params q = p;
   q.rows_per_chunk = (p.ny + g - 1) / g;
   const int gy = (p.ny + q.rows_per_chunk - 1) / q.rows_per_chunk;
+  const dim3 grid(gx, gy);
   if (p.mask) {
-    if (one) k_step2_strip<true, true><<<dim3(gx, gy), kBX2C, 0, s>>>(q);
-    else k_step2_strip<true, false><<<dim3(gx, gy), kBX2C, 0, s>>>(q);
-  } else {
-    if (one) k_step2_strip<false, true><<<dim3(gx, gy), kBX2C, 0, s>>>(q);
-    else k_step2_strip<false, false><<<dim3(gx, gy), kBX2C, 0, s>>>(q);
+    return one ? launch_chain(k_step2_strip<true, true>, grid, dim3(kBX2C), 0, s, q)
+               : launch_chain(k_step2_strip<true, false>, grid, dim3(kBX2C), 0, s, q);
   }
-  return cudaGetLastError();
+  return one ? launch_chain(k_step2_strip<false, true>, grid, dim3(kBX2C), 0, s, q)
+             : launch_chain(k_step2_strip<false, false>, grid, dim3(kBX2C), 0, s, q);
 }
 
 cudaError_t launch_fields2(const Step2Params& p, float* rho_m, float* rho_g, float* ux, float* uy, float* pr,
