@@ -82,11 +82,9 @@ Layout layout_for(const lbm_config& c) {
     L.sgn = take(N);
     L.ntiles = relabel_tile_count(c.nx, c.ny);
     L.tiles = take(3 * (size_t)L.ntiles);  // gas, active, previous active
-    L.tile_list = take(8 * (size_t)L.ntiles);  // work list, then the tiles with a blocked edge
-    L.rbox = take(sizeof(RelabelBox) + 2 * sizeof(RelabelEntry));
+    L.tile_list = take(8 * (size_t)L.ntiles);  // tiles to visit, film tiles
   }
   if (c.growth) L.gas_list = take(4 * N);
-  if (c.components == 2 && c.barrier) L.pr = take(4 * N);
   L.flags = take(sizeof(int) * FLAG_COUNT);
   L.nparts = mass_partials_needed();
   L.partials = take(sizeof(double) * L.nparts);
@@ -197,28 +195,14 @@ int reset_state(lbm_handle* h) {
   return LBM_OK;
 }
 
-// Descriptor and one-box entry list of the tiled barrier pipeline, written
-// into the workspace once (pointers into the workspace do not move).
-int upload_relabel_box(lbm_handle* h) {
-  if (!handle_relabel_tiled(h)) return LBM_OK;
-  const RelabelBox b = handle_relabel_box(h);
-  RelabelEntry e[2] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
-  relabel_entry_sizes(h->cfg.nx, h->cfg.ny, &e[1].off_tiles, &e[1].off_scan, &e[1].off_list);
-  CUDA_TRY(h, cudaMemcpyAsync(h->rbox(), &b, sizeof(b), cudaMemcpyHostToDevice, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(h->rentries(), e, sizeof(e), cudaMemcpyHostToDevice, h->stream));
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));  // the sources live on this stack frame
-  return LBM_OK;
-}
-
 // Barrier pipeline on the current populations (Sec. 2.1.5).
 int relabel(lbm_handle* h) {
   const FieldParams fp = field_params(h);
   const lbm_config& c = h->cfg;
   if (handle_relabel_tiled(h)) {
-    int totals[3];
-    relabel_entry_sizes(c.nx, c.ny, &totals[0], &totals[1], &totals[2]);
-    CUDA_TRY(h, launch_relabel_boxes(c.storage, h->rbox(), h->rentries(), 1, totals, h->cur, h->stream,
-                                     h->comps() == 2));
+    RelabelBox b = handle_relabel_box(h);
+    b.cur = h->cur;
+    CUDA_TRY(h, launch_relabel_lone(c.storage, b, h->comps() == 2, h->stream));
     h->launches += kRelabelLaunches;
     return LBM_OK;
   }
@@ -228,7 +212,7 @@ int relabel(lbm_handle* h) {
   CUDA_TRY(h, launch_rupture(c.nx, c.ny, (float)c.G, (float)c.rho0, (float)c.rupture_eps, h->rho(),
                              h->owner(), h->sgn(), h->open(), h->flags(), h->stream));
   CUDA_TRY(h, launch_mask(c.nx, c.ny, mask_pitch(c.nx), h->owner(), h->open(), h->mask(), h->stream));
-  h->launches += kRelabelLaunches;
+  h->launches += kUntiledLaunches;
   return LBM_OK;
 }
 
@@ -239,9 +223,9 @@ cudaError_t bounce_after_step(lbm_handle* h) {
   const lbm_config& c = h->cfg;
   const bool two = h->comps() == 2;
   if (handle_relabel_tiled(h)) {
-    int totals[3];
-    relabel_entry_sizes(c.nx, c.ny, &totals[0], &totals[1], &totals[2]);
-    return launch_bounce_boxes(c.storage, two, h->rbox(), h->rentries(), 1, totals[2], h->cur ^ 1, h->stream);
+    RelabelBox b = handle_relabel_box(h);
+    b.cur = h->cur ^ 1;
+    return launch_bounce_lone(c.storage, b, two, h->stream);
   }
   return launch_bounce(field_params(h), two, h->col0(1 - h->cur), h->mask(), h->stream);
 }
@@ -320,9 +304,11 @@ int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_de
     if (!dst[b]) continue;
     const size_t nb = b == 5 ? 4 * N : N;
     const int fill = b == 5 ? 0xff : 0;
-    if (state[b - 5] && b == 6)  // rows without their padding
-      CUDA_TRY(h, cudaMemcpy2DAsync(dst[b], h->cfg.nx, state[b - 5], mask_pitch(h->cfg.nx), h->cfg.nx, h->cfg.ny, d2x,
-                                    h->stream));
+    if (state[b - 5] && b == 6) {  // rows without their padding
+      uint8_t* m = static_cast<uint8_t*>(dst_is_device ? dst[b] : static_cast<void*>(stage));
+      CUDA_TRY(h, launch_mask_out(fp, h->mask(), m, h->stream));
+      if (!dst_is_device) CUDA_TRY(h, cudaMemcpyAsync(dst[b], m, nb, d2x, h->stream));
+    }
     else if (state[b - 5]) CUDA_TRY(h, cudaMemcpyAsync(dst[b], state[b - 5], nb, d2x, h->stream));
     else if (dst_is_device) CUDA_TRY(h, cudaMemsetAsync(dst[b], fill, nb, h->stream));
     else memset(dst[b], fill, nb);
@@ -377,8 +363,8 @@ RelabelBox handle_relabel_box(lbm_handle* h) {
   b.pitch = h->shape.pitch;
   b.plane = h->shape.plane;
   b.mpitch = mask_pitch(c.nx);
-  b.rho = h->rho();
   b.label = h->label();
+  b.old = reinterpret_cast<int32_t*>(h->rho());  // idle outside initialisation
   b.owner = h->owner();
   b.sgn = h->sgn();
   b.open = h->open();
@@ -388,8 +374,8 @@ RelabelBox handle_relabel_box(lbm_handle* h) {
   b.tile_prev = h->tiles(2);
   b.tile_list = reinterpret_cast<int*>(h->ws + h->L.tile_list);
   b.film_list = b.tile_list + h->L.ntiles;
+  b.gas_list = h->gas_list();
   b.flags = h->flags();
-  b.pr = h->pr();
   b.G_mg = (float)c.G_mg;
   b.G_gg = (float)c.G_gg;
   b.nx = c.nx;
@@ -487,7 +473,7 @@ int lbm_create(const lbm_config* cfg, void* d_workspace, size_t bytes, void* cud
     delete h;
     return LBM_EINVAL;
   }
-  if (reset_state(h) != LBM_OK || upload_relabel_box(h) != LBM_OK) {
+  if (reset_state(h) != LBM_OK) {
     delete h;
     return LBM_ECUDA;
   }
@@ -584,7 +570,7 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
       }
     }
     const bool growing = h->growth_rate > 0.0;
-    if (growing && h->t % c.relabel_every == 0) {  // gas census with the barrier pipeline
+    if (growing && h->t % c.relabel_every == 0 && !handle_relabel_tiled(h)) {  // gas census with the barrier pipeline
       if (!c.barrier) CUDA_TRY(h, launch_density(field_params(h), h->rho(), h->stream));
       CUDA_TRY(h, launch_gas_census(h->rho(), (long long)h->N(), (float)c.gas_threshold, h->gas_list(),
                                     h->flags() + FLAG_GAS, h->stream));

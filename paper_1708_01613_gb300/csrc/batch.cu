@@ -15,7 +15,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <array>
 #include <map>
 #include <new>
 #include <vector>
@@ -51,7 +50,7 @@ struct lbm_batch {
   struct Group {
     int start = 0;                        // first entry in d_rent
     std::vector<int> members;             // box indices, upload order
-    std::vector<std::array<int, 3>> tot;  // CTA totals of the first k members
+    std::vector<RelabelEntry> tot;        // CTA totals of the first k members
   };
   std::map<int, Group> groups;            // by residue of the step count
   std::vector<int> untiled;               // boxes relabelled one by one
@@ -250,14 +249,12 @@ int upload(lbm_batch* b, const std::vector<int>& order = {}) {
     for (int i : ord) {  // bounce-back entries: the tiled boxes in stepping order
       const bool tiled = handle_relabel_tiled(b->h[i]);
       if (tiled) {
-        int t0, t1, t2;
-        relabel_entry_sizes(b->h[i]->cfg.nx, b->h[i]->cfg.ny, &t0, &t1, &t2);
-        bents.push_back({i, 0, 0, b->bounce_ctas.back()});
-        b->bounce_ctas.push_back(b->bounce_ctas.back() + t2);
+        bents.push_back({i, 0, 0, 0, b->bounce_ctas.back()});
+        b->bounce_ctas.push_back(b->bounce_ctas.back() + relabel_entry_sizes(b->h[i]->cfg.nx, b->h[i]->cfg.ny).off_film);
       }
       b->bounce_first.push_back(b->bounce_first.back() + (tiled ? 1 : 0));
     }
-    bents.push_back({-1, 0, 0, b->bounce_ctas.back()});
+    bents.push_back({-1, 0, 0, 0, b->bounce_ctas.back()});
     for (int i : ord) {
       lbm_handle* h = b->h[i];
       if (!handle_relabel_tiled(h)) {
@@ -271,16 +268,20 @@ int upload(lbm_batch* b, const std::vector<int>& order = {}) {
     for (auto& kv : b->groups) {
       lbm_batch::Group& g = kv.second;
       g.start = (int)ents.size();
-      std::array<int, 3> acc = {0, 0, 0};
+      RelabelEntry acc{};
       g.tot.push_back(acc);
       for (int i : g.members) {
-        ents.push_back({i, acc[0], acc[1], acc[2]});
-        int t0, t1, t2;
-        relabel_entry_sizes(b->h[i]->cfg.nx, b->h[i]->cfg.ny, &t0, &t1, &t2);
-        acc = {acc[0] + t0, acc[1] + t1, acc[2] + t2};
+        acc.box = i;
+        ents.push_back(acc);
+        const RelabelEntry e = relabel_entry_sizes(b->h[i]->cfg.nx, b->h[i]->cfg.ny);
+        acc.off_tiles += e.off_tiles;
+        acc.off_scan += e.off_scan;
+        acc.off_list += e.off_list;
+        acc.off_film += e.off_film;
         g.tot.push_back(acc);
       }
-      ents.push_back({-1, acc[0], acc[1], acc[2]});
+      acc.box = -1;
+      ents.push_back(acc);
     }
     BCUDA(b, cudaMemcpyAsync(b->d_rboxes, rboxes.data(), sizeof(RelabelBox) * b->n, cudaMemcpyHostToDevice,
                              b->stream));
@@ -309,7 +310,7 @@ int enqueue_relabel(lbm_batch* b, int parity, int64_t j, int live, Stepping step
     const lbm_batch::Group& g = it->second;
     const int m = live < 0 ? (int)g.members.size() : std::min(live, (int)g.members.size());
     if (m > 0) {
-      BCUDA(b, launch_relabel_boxes(b->storage, b->d_rboxes, b->d_rent + g.start, m, g.tot[m].data(), parity,
+      BCUDA(b, launch_relabel_boxes(b->storage, b->d_rboxes, b->d_rent + g.start, m, g.tot[m], parity,
                                     b->stream));
       b->launches += kRelabelLaunches;
     }
@@ -325,7 +326,7 @@ int enqueue_relabel(lbm_batch* b, int parity, int64_t j, int live, Stepping step
     h->stream = hs;
     h->cur = saved;
     if (rc) return bfail(b, rc, "relabel of box %d: %s", i, h->err);
-    b->launches += kRelabelLaunches;
+    b->launches += kUntiledLaunches;
   }
   return LBM_OK;
 }
@@ -371,8 +372,7 @@ int enqueue_bounce(lbm_batch* b, int parity, int first, Stepping stepping) {
   const int total = (int)b->bounce_first.size() - 1;
   const int k = b->bounce_first[first < 0 || first > total ? total : first];
   if (k > 0) {
-    BCUDA(b, launch_bounce_boxes(b->storage, false, b->d_rboxes, b->d_bent, k, b->bounce_ctas[k], parity ^ 1,
-                                 b->stream));
+    BCUDA(b, launch_bounce_boxes(b->storage, b->d_rboxes, b->d_bent, k, b->bounce_ctas[k], parity ^ 1, b->stream));
     b->launches += 1;
   }
   for (int i : b->untiled) {

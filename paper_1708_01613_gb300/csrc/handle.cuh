@@ -11,7 +11,7 @@ namespace lbm {
 
 // Offsets of the slices of the caller's workspace.
 struct Layout {
-  size_t pops[2], rho, label, owner, mask, open, sgn, tiles, tile_list, rbox, gas_list, pr, flags, partials,
+  size_t pops[2], rho, label, owner, mask, open, sgn, tiles, tile_list, gas_list, flags, partials,
       scalars, total;
   int nparts, ntiles;
 };
@@ -52,16 +52,12 @@ struct lbm_handle {
   int32_t* gas_list() { return cfg.growth ? reinterpret_cast<int32_t*>(ws + L.gas_list) : nullptr; }
   // released growth total, two slots taking turns with the step parity
   double* released() { return reinterpret_cast<double*>(ws + L.scalars) + 14; }
-  // the box's own barrier-pipeline descriptor and its one-box entry list
-  lbm::RelabelBox* rbox() { return reinterpret_cast<lbm::RelabelBox*>(ws + L.rbox); }
-  lbm::RelabelEntry* rentries() { return reinterpret_cast<lbm::RelabelEntry*>(rbox() + 1); }
   double* partials() { return reinterpret_cast<double*>(ws + L.partials); }
   double* scalars() { return reinterpret_cast<double*>(ws + L.scalars); }
   size_t N() const { return (size_t)cfg.nx * cfg.ny; }
   int comps() const { return cfg.components == 2 ? 2 : 1; }
   // bytes of one buffer's populations without padding (all components): what staging may use
   size_t pops_bytes() const { return (size_t)lbm::Q * comps() * N() * lbm::storage_bytes(cfg.storage); }
-  float* pr() { return cfg.components == 2 && cfg.barrier ? reinterpret_cast<float*>(ws + L.pr) : nullptr; }
 };
 
 namespace lbm {

@@ -81,25 +81,36 @@ __device__ __forceinline__ int32_t tile_root_index(const int* sp, int li, int x0
 // tile, from their gas decisions: -1 for liquid, else the smallest index of
 // the cell's piece of the tile. Returns whether the tile holds gas (uniform
 // over the CTA). Contains barriers: every thread of the CTA calls it.
+//
+// The gas of a row is a 32-bit mask, so every cell starts with its run's first
+// cell as parent, and only the first cell of each overlap with the row below
+// unites: a few links per tile instead of two per gas cell.
 __device__ __forceinline__ int tile_labels4(const bool (&gas)[4], int x, int y, int nx, int32_t (&lab)[4], int* flags) {
   __shared__ int sp[kTX * kTY];
-  const int la = threadIdx.y * kTX + 4 * threadIdx.x;
+  __shared__ unsigned rows[kTY];
+  const int col = 4 * threadIdx.x, la = threadIdx.y * kTX + col;
+  const unsigned own = (gas[0] ? 1u : 0u) | (gas[1] ? 2u : 0u) | (gas[2] ? 4u : 0u) | (gas[3] ? 8u : 0u);
+  unsigned row = own << col;
+#pragma unroll
+  for (int d = 1; d < 8; d *= 2) row |= __shfl_xor_sync(0xffffffffu, row, d);
+  if (threadIdx.x == 0) rows[threadIdx.y] = row;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    sp[la + j] = gas[j] ? la + j : -1;
+    const unsigned liquid = ~row & ((1u << (col + j)) - 1u);  // liquid cells to the left
+    sp[la + j] = gas[j] ? (int)threadIdx.y * kTX + 32 - __clz(liquid) : -1;
     lab[j] = -1;
   }
-  const int any = __syncthreads_or(gas[0] || gas[1] || gas[2] || gas[3]);
+  const int any = __syncthreads_or(own);
   if (any) {
     int fail = 0;
+    if (own && threadIdx.y + 1 < kTY) {
+      const unsigned both = row & rows[threadIdx.y + 1], first = both & ~(both << 1);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (!gas[j]) continue;
-      if (j < 3 ? gas[j + 1] : (4 * threadIdx.x + 4 < kTX && sp[la + 4] >= 0)) tile_unite(sp, la + j, la + j + 1, &fail);
-      if (threadIdx.y + 1 < kTY && sp[la + j + kTX] >= 0) tile_unite(sp, la + j, la + j + kTX, &fail);
+      for (int j = 0; j < 4; ++j)
+        if ((first >> (col + j)) & 1u) tile_unite(sp, la + j, la + j + kTX, &fail);
     }
     __syncthreads();
-    const int x0 = x - 4 * threadIdx.x, y0 = y - threadIdx.y;
+    const int x0 = x - col, y0 = y - threadIdx.y;
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       if (gas[j]) lab[j] = tile_root_index(sp, la + j, x0, y0, nx, &fail);
@@ -109,20 +120,27 @@ __device__ __forceinline__ int tile_labels4(const bool (&gas)[4], int x, int y, 
 }
 
 // Joins the gas cells of tile (x0, y0) to the next tile's across its bottom
-// and right borders (periodic wrap included); one warp, `lane` its lane.
+// and right borders (periodic wrap included); one warp, `lane` its lane, all
+// lanes call. One link per run of facing gas cells: the cells of a run are
+// joined within each tile already.
 __device__ __forceinline__ void tile_union_borders(int32_t* L, int x0, int y0, int nx, int ny, int lane, int* fail) {
+  int a = -1, b = -1, ra = -1, rb = -1;
   {
     const int x = x0 + lane, y = min(y0 + kTY, ny) - 1;
     if (x < nx) {
-      const int c = y * nx + x, down = (y + 1 == ny ? 0 : y + 1) * nx + x;
-      if (L[c] >= 0 && L[down] >= 0) unite(L, c, down, fail);
+      a = L[y * nx + x];
+      b = L[(y + 1 == ny ? 0 : y + 1) * nx + x];
     }
   }
   if (lane < kTY && y0 + lane < ny) {
     const int x = min(x0 + kTX, nx) - 1, y = y0 + lane;
-    const int c = y * nx + x, right = y * nx + (x + 1 == nx ? 0 : x + 1);
-    if (L[c] >= 0 && L[right] >= 0) unite(L, c, right, fail);
+    ra = L[y * nx + x];
+    rb = L[y * nx + (x + 1 == nx ? 0 : x + 1)];
   }
+  const unsigned down = __ballot_sync(0xffffffffu, a >= 0 && b >= 0),
+                 right = __ballot_sync(0xffffffffu, ra >= 0 && rb >= 0);
+  if (((down & ~(down << 1)) >> lane) & 1u) unite(L, a, b, fail);
+  if (((right & ~(right << 1)) >> lane) & 1u) unite(L, ra, rb, fail);
 }
 
 }  // namespace

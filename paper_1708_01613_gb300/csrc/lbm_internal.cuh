@@ -38,7 +38,7 @@ enum Flag : int {
   FLAG_GAS = 4,       // gas points in the growth list
   FLAG_ITEM = 5,      // work-item counter of the dynamically scheduled step (0 between launches)
   FLAG_DONE = 6,      // CTAs of that launch that have finished (0 between launches)
-  FLAG_FILM = 7,      // tiles in the list of tiles holding a blocked edge
+  FLAG_FILM = 7,      // tiles in the list of film tiles
   FLAG_MERGES = 8,    // coalescence events counted by the relabels since the last init
   FLAG_HIST = 64,     // 64 histogram counters
   FLAG_COUNT = 128
@@ -279,6 +279,8 @@ struct FieldOuts {
   float *rho, *ux, *uy, *p;
 };
 cudaError_t launch_fields(const FieldParams& fp, const uint8_t* mask, const FieldOuts& out, cudaStream_t s);
+// The mask in dense rows.
+cudaError_t launch_mask_out(const FieldParams& fp, const uint8_t* mask, uint8_t* out, cudaStream_t s);
 // Planes plane0 .. plane0 + planes of the incoming state, back to back.
 cudaError_t launch_pops_out(const FieldParams& fp, int plane0, int planes, float* out, cudaStream_t s);
 // Scratch the three label passes need beside their arrays (8-byte aligned).
@@ -303,22 +305,23 @@ cudaError_t launch_bubbles_rho(const lbm_bubble* d_bubbles, int n, double rho_l,
 cudaError_t launch_mass(const FieldParams& fp, double* partials, int nparts, double* out_dev,
                         cudaStream_t s);
 constexpr int kMaxHistBins = 64;
-// Tiled barrier pipeline (barrier.cu): density + labels + tile flags, then
-// union, flatten, owner, rupture and mask restricted to tiles near gas.
-// One launch per phase serves any number of boxes.
+// Tiled barrier pipeline (relabel.cu). One launch per phase serves one box or
+// any number of boxes.
 bool relabel_tiled_ok(int nx, int ny, int R);
 int relabel_tile_count(int nx, int ny);
 constexpr int kRelabelTileX = 32, kRelabelTileY = 8;  // tile of the pipeline
-// Launches of one relabel: density, tile scan (tiled) or label init (untiled),
-// union, flatten, coalescence count, owner, rupture, mask.
-constexpr int kRelabelLaunches = 8;
+constexpr int kRelabelLaunches = 4;
+// Launches of an untiled relabel: density, label init, union, flatten,
+// coalescence count, owner, rupture, mask.
+constexpr int kUntiledLaunches = 8;
 
-// A box as the pipeline sees it (device memory). Populations are read from
-// pops[cur ^ parity], parity being the launch argument.
+// A box as the pipeline sees it (a kernel argument, or device memory).
+// Populations are read from pops[cur ^ parity], parity being the launch
+// argument.
 struct RelabelBox {
-  const void* pops[2];
-  float* rho;
+  const void* pops[2];  // column 0, like mask
   int32_t* label;
+  int32_t* old;  // scratch: labels of the previous relabel at gas cells
   int32_t* owner;
   int8_t* sgn;
   uint8_t* open;
@@ -326,13 +329,12 @@ struct RelabelBox {
   uint8_t* tile_gas;
   uint8_t* tile_active;
   uint8_t* tile_prev;
-  int* tile_list;
-  int* film_list;  // tiles of the work list holding a blocked edge (bounce-back)
+  int* tile_list;     // tiles to visit
+  int* film_list;     // tiles of it where owners meet (mask, bounce-back)
+  int32_t* gas_list;  // gas cells for the growth source (nullptr: no source)
   int* flags;
-  float* pr;  // two components: mixture pressure written by the density
-              // phase and used by the rupture test (nullptr: one component)
   int nx, ny, ntx, nty, R, cur;
-  int pitch, mpitch;  // pops and mask point at column 0
+  int pitch, mpitch;
   long long plane;
   float threshold, G, rho0, eps;
   float G_mg, G_gg;  // two components: melt-gas and gas-gas couplings
@@ -340,35 +342,37 @@ struct RelabelBox {
 };
 
 // Box `box` in a launch's entry list, with the CTAs of the entries before it
-// in each kind of phase (per-tile, tile-scan, tile-list). An entry list of m
-// boxes has m + 1 entries: the last holds the totals.
+// in each kind of phase (per-tile, tile-scan, tile-list, film-list). An entry
+// list of m boxes has m + 1 entries: the last holds the totals.
 struct RelabelEntry {
-  int box, off_tiles, off_scan, off_list;
+  int box, off_tiles, off_scan, off_list, off_film;
 };
+
+// CTAs a box takes in each kind of phase.
+RelabelEntry relabel_entry_sizes(int nx, int ny);
+// The phases over a box (state: pops[cur]), or over the first m entries;
+// totals = entries[m]. two: two components (FP32).
+cudaError_t launch_relabel_lone(int storage, const RelabelBox& box, bool two, cudaStream_t s);
+cudaError_t launch_relabel_boxes(int storage, const RelabelBox* boxes, const RelabelEntry* entries, int m,
+                                 const RelabelEntry& totals, int parity, cudaStream_t s);
 
 // Halfway bounce-back across the blocked edges of the mask (the barrier of
 // Sec. 2.1.5), run on the buffer a step has just written (after the growth
 // source, if any): the two slots of each blocked edge trade values, so the
 // next step's pull returns every population that would cross the wall to
 // its own cell in the opposite direction. `two`: 18 planes (two lattices).
-// launch_bounce scans every cell; launch_bounce_boxes visits the tiles that
-// the latest tiled relabel of each box in the entry list found holding a
-// blocked edge, on buffer pops[cur ^ q] (total_list = the entries' list-CTA
-// total).
+// launch_bounce scans every cell; the others visit the tiles that the latest
+// tiled relabel found holding a blocked edge, on buffer pops[cur ^ q] (q = 0
+// for a lone box; ctas = the entries' film-CTA total).
 cudaError_t launch_bounce(const FieldParams& fp, bool two, void* pops, const uint8_t* mask, cudaStream_t s);
-cudaError_t launch_bounce_boxes(int storage, bool two, const RelabelBox* boxes, const RelabelEntry* entries, int m,
-                                int total_list, int q, cudaStream_t s);
-
-// CTAs a box takes in each kind of phase.
-void relabel_entry_sizes(int nx, int ny, int* tiles, int* scan, int* list);
-// The seven phases over the first m entries; totals = entries[m]'s offsets.
-// two_component: the boxes are two-component (FP32; mixture pressure).
-cudaError_t launch_relabel_boxes(int storage, const RelabelBox* boxes, const RelabelEntry* entries, int m,
-                                 const int totals[3], int parity, cudaStream_t s, bool two_component = false);
+cudaError_t launch_bounce_lone(int storage, const RelabelBox& box, bool two, cudaStream_t s);
+cudaError_t launch_bounce_boxes(int storage, const RelabelBox* boxes, const RelabelEntry* entries, int m, int ctas,
+                                int q, cudaStream_t s);
 int mass_partials_needed();
 
 // Nucleation and growth (growth.cu). The gas census appends every cell with
-// rho < threshold to `list` (order irrelevant) and sets *count. The growth
+// rho < threshold to `list` (order irrelevant) and sets *count (the tiled
+// relabel takes its census itself). The growth
 // kernel adds w_i drho to the post-collision populations of the listed
 // cells, drho = min(rate, budget - released) / count, reading the released
 // total from released[parity] and writing the new total to
