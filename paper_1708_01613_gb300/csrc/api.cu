@@ -578,6 +578,7 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     }
     p.src = h->col0(h->cur);
     p.dst = h->col0(1 - h->cur);
+    p.odd = h->cur;
     if (c.components == 2) {
       const Step2Params q = step2_params(h);
       CUDA_TRY(h, launch_step2(q, h->stream));

@@ -169,6 +169,7 @@ struct StepParams {
   int pitch, mpitch;     // row strides: population values, mask bytes (src, dst and mask point at column 0)
   long long plane;       // plane stride
   int rows_per_chunk;    // rows marched by one CTA
+  int odd;               // tile kernel: every second step (tiles in reverse)
   int pull_bounce;       // tile kernel: src holds populations that have not bounced back yet
   int force_generic;     // kernel variant: 0 automatic, 1 plain loads, 2 one-cell staged, 3 two-cell staged,
                          // 4 two-cell staged with dynamically scheduled row chunks

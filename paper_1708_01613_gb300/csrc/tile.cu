@@ -30,6 +30,7 @@ struct TileBox {
   int* flags;
   int nx, ny;
   uint32_t row_bytes, mask_row;  // strides
+  int reverse;                   // tiles from the last to the first
   int pull_bounce;               // src holds populations that have not bounced back yet
   StepParams s;                  // constants of the arithmetic
 };
@@ -239,27 +240,20 @@ __device__ __forceinline__ void tile_step(const TileBox& b, int xo, int y0, int 
   uint32_t worst = 0;
 #pragma unroll
   for (int q = 0; q < P; ++q) {
-    float2 s[Q];
-    s[1] = B.r[q];
-    s[2] = N.c[q];
-    s[3] = B.l[q];
-    s[4] = A.c[q];
-    s[5] = N.r[q];
-    s[6] = N.l[q];
-    s[7] = A.l[q];
-    s[8] = A.r[q];
-    if (MASKED && mask) {
+    float2 Fx, Fy, f[Q];
+    const float2 s[Q] = {B.c[q], B.r[q], N.c[q], B.l[q], A.c[q], N.r[q], N.l[q], A.l[q], A.r[q]};
+    if (MASKED && mask) {  // a path of its own keeps the other free of copies
+      float2 v[Q];
       const unsigned ma = (mask >> (16 * q)) & 0xffu, mb = (mask >> (16 * q + 8)) & 0xffu;
 #pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        if ((ma >> (i - 1)) & 1u) s[i].x = B.c[q].x;
-        if ((mb >> (i - 1)) & 1u) s[i].y = B.c[q].y;
-      }
+      for (int i = 1; i < Q; ++i)
+        v[i] = make_float2((ma >> (i - 1)) & 1u ? B.c[q].x : s[i].x, (mb >> (i - 1)) & 1u ? B.c[q].y : s[i].y);
+      force_of(v, B.c[q], b.s.G, Fx, Fy);
+    } else {
+      force_of(s, B.c[q], b.s.G, Fx, Fy);
     }
-    float2 Fx, Fy, f[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) f[i] = g[i][q];
-    force_of(s, B.c[q], b.s.G, Fx, Fy);
     uint32_t pair_worst = 0;  // a pair that starts in the box pulls valid columns only
     collide<TAU_ONE, S != LBM_F32>(f, rho[q], jx[q], jy[q], Fx, Fy, b.s, pair_worst);
     if (x + 2 * q < nx) worst = max(worst, pair_worst);
@@ -317,8 +311,9 @@ __host__ __device__ __forceinline__ void tile_planes(TileBox& b, const void* src
 
 template <int S, bool MASKED, bool TAU_ONE, typename G>
 __global__ void __launch_bounds__(G::THREADS, G::CTAS) k_step_tile(const TileBox b, int gx) {
-  const int y0 = (int)(blockIdx.x / gx) * G::ROWS;
-  tile_step<S, MASKED, TAU_ONE, G>(b, (int)(blockIdx.x % gx) * G::COLS, y0, min(y0 + G::ROWS, b.ny));
+  const int t = b.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  const int y0 = t / gx * G::ROWS;
+  tile_step<S, MASKED, TAU_ONE, G>(b, t % gx * G::COLS, y0, min(y0 + G::ROWS, b.ny));
 }
 
 // One item per CTA. The item and its box's descriptor are constant while the
@@ -327,8 +322,8 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS) k_step_tile(const TileBox
 template <int S, bool MASKED, bool TAU_ONE, typename G>
 __global__ void __launch_bounds__(G::THREADS, G::CTAS)
     k_step_tile_batch(const BatchInst* __restrict__ insts, const BatchItem* __restrict__ items, int parity,
-                      int pull_bounce) {
-  const BatchItem it = items[blockIdx.x];
+                      int pull_bounce, int reverse) {
+  const BatchItem it = items[reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x];
   const BatchInst& in = insts[it.inst];
   TileBox b;
   const int c = in.cur ^ parity;
@@ -350,6 +345,14 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
   tile_step<S, MASKED, TAU_ONE, G>(b, it.x0, it.y0, it.y1);
 }
 
+// Every second step takes the tiles from the last to the first while the two
+// buffers (`bytes`) are of the order of the L2: its reads then start with what
+// the step before wrote last, which is still there. 2000 x 1504 BF16 29.9 ->
+// 26.9 us, 2048^2 FP16 35.4 -> 33.6 and FP32 48.7 -> 47.3, 3000^2 FP16 67.0 ->
+// 66.1. Below (all of it stays in L2) and above (4096^2 FP16, 600 MB) it gives
+// nothing, or costs 1 %.
+bool tile_turns(size_t bytes) { return bytes >= 64u << 20 && bytes <= 512u << 20; }
+
 template <int S, bool MASKED, bool TAU_ONE, typename G>
 cudaError_t launch_tile_g(const TileBox& b, cudaStream_t s) {
   const int gx = (b.nx + G::COLS - 1) / G::COLS;
@@ -369,6 +372,7 @@ cudaError_t launch_tile_t(const StepParams& p, cudaStream_t s) {
   b.row_bytes = (uint32_t)p.pitch * E;
   b.mask_row = (uint32_t)p.mpitch;
   b.pull_bounce = p.pull_bounce;
+  b.reverse = p.odd && tile_turns(2 * Q * (size_t)p.plane * E);
   b.s = p;
   using Small = typename Tiles<S, TAU_ONE>::Small;
   using Large = typename Tiles<S, TAU_ONE>::Large;
@@ -385,21 +389,21 @@ cudaError_t launch_tile_s(const StepParams& p, cudaStream_t s) {
 }
 
 template <int S, bool MASKED, bool TAU_ONE>
-cudaError_t launch_tile_batch_t(const BatchInst* insts, const BatchItem* items, int nitems, int parity, int pull_bounce,
+cudaError_t launch_tile_batch_t(const BatchInst* insts, const BatchItem* items, int nitems, int parity, int pull_bounce, int reverse,
                                 cudaStream_t s) {
   using G = typename Tiles<S, TAU_ONE>::Large;
   return launch_chain(k_step_tile_batch<S, MASKED, TAU_ONE, G>, dim3(nitems), dim3(G::THREADS), 0, s, insts, items,
-                      parity, pull_bounce);
+                      parity, pull_bounce, reverse);
 }
 
 template <int S>
 cudaError_t launch_tile_batch_s(bool masked, bool one, const BatchInst* insts, const BatchItem* items, int nitems,
-                                int parity, int pull_bounce, cudaStream_t s) {
+                                int parity, int pull_bounce, int reverse, cudaStream_t s) {
   if (masked)
-    return one ? launch_tile_batch_t<S, true, true>(insts, items, nitems, parity, pull_bounce, s)
-               : launch_tile_batch_t<S, true, false>(insts, items, nitems, parity, pull_bounce, s);
-  return one ? launch_tile_batch_t<S, false, true>(insts, items, nitems, parity, pull_bounce, s)
-             : launch_tile_batch_t<S, false, false>(insts, items, nitems, parity, pull_bounce, s);
+    return one ? launch_tile_batch_t<S, true, true>(insts, items, nitems, parity, pull_bounce, reverse, s)
+               : launch_tile_batch_t<S, true, false>(insts, items, nitems, parity, pull_bounce, reverse, s);
+  return one ? launch_tile_batch_t<S, false, true>(insts, items, nitems, parity, pull_bounce, reverse, s)
+             : launch_tile_batch_t<S, false, false>(insts, items, nitems, parity, pull_bounce, reverse, s);
 }
 
 // f(Tiles<S, TAU_ONE>) for a storage and relaxation known at run time.
@@ -445,12 +449,15 @@ cudaError_t launch_tile(int storage, const StepParams& p, cudaStream_t s) {
 cudaError_t launch_tile_batch(int storage, bool masked, bool tau_one, const BatchInst* insts, const BatchItem* items,
                               int nitems, int parity, bool pull_bounce, cudaStream_t s) {
   if (nitems <= 0) return cudaSuccess;
+  int cols, rows;
+  tile_item_size(storage, tau_one, &cols, &rows);
+  const int reverse = parity && tile_turns((size_t)nitems * cols * rows * 2 * Q * storage_bytes(storage));
   switch (storage) {
-    case LBM_F32: return launch_tile_batch_s<LBM_F32>(masked, tau_one, insts, items, nitems, parity, pull_bounce, s);
+    case LBM_F32: return launch_tile_batch_s<LBM_F32>(masked, tau_one, insts, items, nitems, parity, pull_bounce, reverse, s);
     case LBM_F16_DEV:
-      return launch_tile_batch_s<LBM_F16_DEV>(masked, tau_one, insts, items, nitems, parity, pull_bounce, s);
+      return launch_tile_batch_s<LBM_F16_DEV>(masked, tau_one, insts, items, nitems, parity, pull_bounce, reverse, s);
     case LBM_BF16_DEV:
-      return launch_tile_batch_s<LBM_BF16_DEV>(masked, tau_one, insts, items, nitems, parity, pull_bounce, s);
+      return launch_tile_batch_s<LBM_BF16_DEV>(masked, tau_one, insts, items, nitems, parity, pull_bounce, reverse, s);
     default: return cudaErrorInvalidValue;
   }
 }
