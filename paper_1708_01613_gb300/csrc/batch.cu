@@ -42,6 +42,8 @@ struct lbm_batch {
   int max_items = 0;
   int nitems = 0;
   std::vector<BatchItem> items;
+  std::vector<BatchInst> insts;                // as uploaded
+  std::vector<int> tile_order, tile_first;     // tiled: boxes in stepping order, items before each
   // barrier pipeline: tiled boxes relabel together, one launch per phase for
   // all boxes due at the same step; boxes are grouped by the residue of their
   // step count modulo the relabel period (relative to the batch counter)
@@ -116,6 +118,8 @@ void build_tile_items(lbm_batch* b) {
   for (int i = 0; i < b->n; ++i) {
     if (!b->active[i]) continue;
     const int nx = b->h[i]->cfg.nx, ny = b->h[i]->cfg.ny;
+    b->tile_order.push_back(i);
+    b->tile_first.push_back((int)b->items.size());
     for (int y0 = 0; y0 < ny; y0 += rows)
       for (int x0 = 0; x0 < nx; x0 += cols)
         b->items.push_back({i, x0, std::min(cols, nx - x0), y0, std::min(y0 + rows, ny)});
@@ -148,6 +152,8 @@ bool batch_tiles(const lbm_batch* b) {
 // too.
 void build_items(lbm_batch* b, bool spread) {
   b->items.clear();
+  b->tile_order.clear();
+  b->tile_first.clear();
   b->tiled = batch_tiles(b);
   if (b->tiled) return build_tile_items(b);
   const int res = std::max(1, batch_resident_ctas(b->storage, b->masked != 0, b->tau_one != 0));
@@ -200,7 +206,8 @@ void build_items(lbm_batch* b, bool spread) {
 // active boxes, by index; a non-empty order means multi-rate steps).
 int upload(lbm_batch* b, const std::vector<int>& order = {}) {
   if (!b->dirty) return LBM_OK;
-  std::vector<BatchInst> insts(b->n);
+  std::vector<BatchInst>& insts = b->insts;
+  insts.assign(b->n, BatchInst());
   std::vector<RelabelBox> rboxes(b->masked ? b->n : 0);
   for (int i = 0; i < b->n; ++i) {
     lbm_handle* h = b->h[i];
@@ -336,8 +343,18 @@ int enqueue_relabel(lbm_batch* b, int parity, int64_t j, int live, Stepping step
 int enqueue_items(lbm_batch* b, int parity, int n, bool pull_bounce) {
   if (n <= 0) return LBM_OK;
   if (b->tiled) {
-    BCUDA(b, launch_tile_batch(b->storage, b->masked != 0, b->tau_one != 0, b->d_insts, b->d_items, n, parity,
-                                pull_bounce, b->stream));
+    TileBatch t{b->masked != 0, b->tau_one != 0, pull_bounce, parity, n, nullptr, b->d_insts, b->d_items};
+    BatchBoxes boxes;
+    boxes.n = 0;
+    for (size_t k = 0; k < b->tile_order.size() && b->tile_first[k] < n && boxes.n <= BatchBoxes::kMost; ++k) {
+      if (boxes.n < BatchBoxes::kMost) {
+        boxes.first[boxes.n] = b->tile_first[k];
+        boxes.in[boxes.n] = b->insts[b->tile_order[k]];
+      }
+      ++boxes.n;
+    }
+    if (boxes.n <= BatchBoxes::kMost) t.boxes = &boxes;
+    BCUDA(b, launch_tile_batch(b->storage, t, b->stream));
     b->launches += 1;
     return LBM_OK;
   }
@@ -667,6 +684,10 @@ int lbm_batch_step_each(lbm_batch* b, const int64_t* nsteps, int32_t n) {
     for (const BatchItem& it : b->items)
       if (it.inst == order[k]) sorted.push_back(it);
     prefix[k + 1] = (int)sorted.size();
+  }
+  if (b->tiled) {
+    b->tile_order = order;
+    b->tile_first.assign(prefix.begin(), prefix.end() - 1);
   }
   if (!sorted.empty())
     BCUDA(b, cudaMemcpyAsync(b->d_items, sorted.data(), sizeof(BatchItem) * sorted.size(), cudaMemcpyHostToDevice,

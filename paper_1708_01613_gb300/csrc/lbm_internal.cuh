@@ -232,8 +232,22 @@ bool tile_fits(int storage, long long plane);
 void tile_item_size(int storage, bool tau_one, int* cols, int* rows);
 // Cells up to which the tile kernel beats the staged ones.
 long long tile_cells(int storage, bool tau_one);
-cudaError_t launch_tile_batch(int storage, bool masked, bool tau_one, const BatchInst* insts, const BatchItem* items,
-                              int nitems, int parity, bool pull_bounce, cudaStream_t s);
+// The boxes of a batch as a kernel argument, with the tiles of the boxes
+// before each (rows of tiles, top to bottom).
+struct BatchBoxes {
+  static constexpr int kMost = 40;  // 4 KB of arguments
+  int n;
+  int first[kMost];
+  BatchInst in[kMost];
+};
+struct TileBatch {
+  bool masked, tau_one, pull_bounce;
+  int parity, nitems;
+  const BatchBoxes* boxes;  // host; nullptr: the tables below (device)
+  const BatchInst* insts;
+  const BatchItem* items;
+};
+cudaError_t launch_tile_batch(int storage, const TileBatch& t, cudaStream_t s);
 // Launch geometry the fused step uses for a box (for tests/benchmarks).
 void step_geometry(int nx, int ny, int* grid_x, int* grid_y, int* rows_per_chunk, int* block);
 // Widths the staged variants accept (lbm_set_step_variant): 2 takes widths
