@@ -579,9 +579,20 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     p.src = h->col0(h->cur);
     p.dst = h->col0(1 - h->cur);
     p.odd = h->cur;
+    // a small box takes its steps up to the next relabel in one launch
+    int64_t run = 1;
+    if (c.components == 1 && !growing && !stop_after && !p.pull_bounce) {
+      run = std::min<int64_t>(nsteps - s, 4096);
+      if (c.barrier) run = std::min<int64_t>(run, c.relabel_every - h->t % c.relabel_every);
+      if (!steps_resident(p, run)) run = 1;
+    }
     if (c.components == 2) {
       const Step2Params q = step2_params(h);
       CUDA_TRY(h, launch_step2(q, h->stream));
+    } else if (run > 1) {
+      CUDA_TRY(h, launch_resident(c.storage, p, (int)run, h->stream));
+      s += run - 1;
+      h->t += run - 1;
     } else {
       CUDA_TRY(h, launch_step(c.storage, p, h->stream));
     }
@@ -592,7 +603,7 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
       h->launches += 1;
     }
     if (c.barrier) {  // populations that would cross a blocked edge bounce back
-      p.pull_bounce = pulls && s + 1 < nsteps && !stop_after && (h->t + 1) % c.relabel_every != 0;
+      p.pull_bounce = pulls && run == 1 && s + 1 < nsteps && !stop_after && (h->t + 1) % c.relabel_every != 0;
       if (!p.pull_bounce) {
         CUDA_TRY(h, bounce_after_step(h));
         h->launches += 1;

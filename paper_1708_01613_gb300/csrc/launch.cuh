@@ -7,6 +7,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <mutex>
+#include <vector>
+
 namespace lbm {
 namespace {
 
@@ -31,6 +34,65 @@ inline cudaError_t launch_chain(void (*kern)(P...), dim3 grid, dim3 block, size_
   c.attrs = &attr;
   c.numAttrs = 1;
   return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
+// The same as one cluster of `size` CTAs (more than 8: not portable, so ask
+// cluster_fits first).
+template <typename... P, typename... A>
+inline cudaError_t launch_cluster(void (*kern)(P...), int size, dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && smem > 48 * 1024)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = size;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = attr;
+  c.numAttrs = 2;
+  return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
+// Whether the current device holds such a cluster (asked once per device and kernel).
+template <typename... P>
+inline bool cluster_fits(void (*kern)(P...), int size, int threads, size_t smem) {
+  struct Seen {
+    void (*kern)(P...);
+    int dev;
+    bool fits;
+  };
+  static std::mutex lock;
+  static std::vector<Seen> seen;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> g(lock);
+  for (const Seen& v : seen)
+    if (v.kern == kern && v.dev == dev) return v.fits;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && smem > 48 * 1024)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = size;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(size);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  int n = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, kern, &c);
+  if (e != cudaSuccess) cudaGetLastError();  // not an error of the caller's
+  seen.push_back({kern, dev, e == cudaSuccess && n > 0});
+  return seen.back().fits;
 }
 
 }  // namespace

@@ -224,6 +224,10 @@ cudaError_t launch_step(int storage, const StepParams& p, cudaStream_t s);
 // Whether launch_step takes the tile kernel (tile.cu) for this box (automatic
 // variant): then the bounce-back of the step before may be left to the pull
 // (pull_bounce).
+// Many steps in one launch, src to dst, for a box that fits a cluster's shared
+// memory (resident.cu); src has bounced back already, dst has not.
+bool steps_resident(const StepParams& p, long long steps);
+cudaError_t launch_resident(int storage, const StepParams& p, int steps, cudaStream_t s);
 bool step_tiles(int storage, const StepParams& p);
 cudaError_t launch_tile(int storage, const StepParams& p, cudaStream_t s);
 // The same over many boxes, items of at most cols x rows cells (x0 a multiple
