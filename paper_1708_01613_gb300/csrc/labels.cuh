@@ -21,10 +21,20 @@ __device__ __forceinline__ int find_root(const int32_t* L, int a, int* fail) {
   return a;
 }
 
+// Both roots, the two walks side by side (each hop is a load's latency).
+__device__ __forceinline__ void find_roots(const int32_t* L, int& a, int& b, int* fail) {
+  for (int it = 0; it < kUnionIters; ++it) {
+    const int p = L[a], q = L[b];
+    if (p == a && q == b) return;
+    a = p;
+    b = q;
+  }
+  *fail = 1;
+}
+
 __device__ __forceinline__ void unite(int32_t* L, int a, int b, int* fail) {
   for (int it = 0; it < kUnionIters; ++it) {
-    a = find_root(L, a, fail);
-    b = find_root(L, b, fail);
+    find_roots(L, a, b, fail);
     if (a == b) return;
     if (a < b) {
       const int t = a;

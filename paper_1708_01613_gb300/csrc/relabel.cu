@@ -31,8 +31,10 @@
 // most, by the chain of dependent loads of each tile. Microseconds of the
 // phases 1 to 4 (the chain of eight launches this replaces, where a label pass
 // wrote densities and every listed tile went through five of them): 160 x 80
-// 5.1 + 6.4 + 9.1 + 2.9 (36 in all); 1024^2 FP16 8.4 + 8.6 + 11.5 + 3.7 (41);
-// 4096^2 FP32 103 + 12.5 + 36 + 3.5 (212); 8192^2 FP32 380 + 23 + 136 + 4 (705).
+// 5.1 + 4.6 + 8.0 + 2.9 (36 in all); 1024^2 FP16 8.3 + 6.2 + 11 + 3.6 (41);
+// 4096^2 FP32 104 + 9.2 + 37 + 3.3 (212); 8192^2 FP32 384 + 17 + 145 + 4 (705).
+// Walks to roots go side by side, and a cell's own state is loaded with the
+// window (one after the other: scan 6.4 and zone 9.1 us at 160 x 80).
 // A launch of its own for final labels and another for the mask over all listed
 // tiles, as before, cost 5 to 45 us and 4 to 100 us more.
 #include <algorithm>
@@ -170,9 +172,16 @@ __global__ void __launch_bounds__(32 * kScanTiles) kb_scan(const __grid_constant
   const int ntx = B.ntx, nty = B.nty, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = src.template first<kScan>(k) * kScanTiles + lane;
   grid_begin();
+  const bool in = t < ntx * nty;
+  bool gas = false;
   if (warp == 0) {
-    const bool in = t < ntx * nty;
-    bool gas = false;
+    gas = in && B.tile_gas[t] != 0;
+    const unsigned g = __ballot_sync(0xffffffffu, gas);
+    if (gas) gas_tiles[__popc(g & ((1u << lane) - 1u))] = t;
+    if (lane == 0) ngas = __popc(g);
+  }
+  __syncthreads();
+  if (warp == 0) {  // the list, while the other warps unite
     int a = 0;
     if (in) {
       // tiles within reach of R cells; across the periodic seam of a box with a
@@ -184,19 +193,15 @@ __global__ void __launch_bounds__(32 * kScanTiles) kb_scan(const __grid_constant
         const int row = wrap_any(ty + dy, nty) * ntx;
         for (int dx = -spx; dx <= spx; ++dx) a |= B.tile_gas[row + wrap_any(tx + dx, ntx)];
       }
-      gas = B.tile_gas[t] != 0;
       B.tile_active[t] = (uint8_t)(a != 0);
     }
     const bool visit = in && (a || B.tile_prev[t]);
     const int slot = warp_slot(visit, B.flags + FLAG_TILES);
     if (visit) B.tile_list[slot] = a ? t : ~t;
-    const unsigned g = __ballot_sync(0xffffffffu, gas);
-    if (gas) gas_tiles[__popc(g & ((1u << lane) - 1u))] = t;
-    if (lane == 0) ngas = __popc(g);
   }
-  __syncthreads();
   int fail = 0;
-  for (int w = warp; w < ngas; w += blockDim.x / 32) {
+  const int warps = blockDim.x / 32;
+  for (int w = warp == 0 ? warps - 1 : warp - 1; w < ngas; w += warps) {
     const int g = gas_tiles[w];
     tile_union_borders(B.label, (g % ntx) * kTX, (g / ntx) * kTY, B.nx, B.ny, lane, &fail);
   }
@@ -323,6 +328,8 @@ __global__ void __launch_bounds__(kTileThreads, 5) kb_zone(const __grid_constant
     const bool in = x < nx && y < ny;
     const int c = y * nx + x;
     bool any = false;
+    // this cell's own state, on its way while the window is
+    const int was = act && in ? B.old[c] : 0, prevs = act && in ? B.sgn[c] : 0, open = act && in ? B.open[c] : 0;
     if (act) {
       for (int yb = warp; yb < H; yb += 3 * kTileWarps) {  // six loads in flight (R = 4: the whole window)
         for (int q = 0; 32 * q < W; q += 2) {
@@ -338,6 +345,20 @@ __global__ void __launch_bounds__(kTileThreads, 5) kb_zone(const __grid_constant
               l[k][u] = yy < H && xx < W ? L[row + min(wrap1(x0 - R - 1 + xx, nx), nx - 1)] : -1;
             }
           }
+          // every label to its root, the six walks side by side
+          bool walk = true;
+          for (int it = 0; walk && it < kUnionIters; ++it) {
+            walk = false;
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                const int up = l[k][u] >= 0 ? L[l[k][u]] : -1;
+                walk |= up != l[k][u];
+                l[k][u] = up;
+              }
+          }
+          if (walk) fail = 1;
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
             const int yy = yb + k * kTileWarps;
@@ -345,7 +366,6 @@ __global__ void __launch_bounds__(kTileThreads, 5) kb_zone(const __grid_constant
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
               const int xx = 32 * (q + u) + lane;
-              if (l[k][u] >= 0) l[k][u] = find_root(L, l[k][u], &fail);
               if (xx < W) win[yy * W + xx] = l[k][u];
               const unsigned b = __ballot_sync(0xffffffffu, l[k][u] >= 0);
               if (lane == 0 && q + u < 4) bits[yy][q + u] = b;
@@ -371,7 +391,7 @@ __global__ void __launch_bounds__(kTileThreads, 5) kb_zone(const __grid_constant
     const int root = in ? win[(warp + R + 1) * W + lane + R + 1] : -1;
     if (root >= 0) {
       B.label[c] = root;
-      if (root != c) merged += merge_vote(B.old, root, B.old[c]);
+      if (root != c) merged += merge_vote(B.old, root, was);
     }
     if (B.gas_list) {
       const int slot = warp_slot(root >= 0, B.flags + FLAG_GAS);
@@ -420,8 +440,7 @@ __global__ void __launch_bounds__(kTileThreads, 5) kb_zone(const __grid_constant
         const float pm = pressure_at<S, TWO>(B, p, wrap1(x - ex, nx), wrap1(y - ey, ny));
         const float d2 = pp - 2.0f * p0 + pm;
         const int sg = (d2 > 0.f) - (d2 < 0.f);
-        const int prevs = B.sgn[c];
-        if (B.eps >= 0.f && !B.open[c] && (fabsf(d2) <= B.eps || (prevs != 0 && sg != prevs))) {
+        if (B.eps >= 0.f && !open && (fabsf(d2) <= B.eps || (prevs != 0 && sg != prevs))) {
           B.open[c] = 1;
           ++opened;
         }
