@@ -83,6 +83,10 @@ Layout layout_for(const lbm_config& c) {
     L.ntiles = relabel_tile_count(c.nx, c.ny);
     L.tiles = take(3 * (size_t)L.ntiles);  // gas, active, previous active
     L.tile_list = take(8 * (size_t)L.ntiles);  // tiles to visit, film tiles
+    // scratch of the coalescence count: the density slice, idle during a
+    // relabel; two lattices have a slice of their own (a workspace of theirs
+    // holds more than two of one lattice, which callers may count on)
+    L.old = comps == 2 ? take(4 * N) : L.rho;
   }
   if (c.growth) L.gas_list = take(4 * N);
   L.flags = take(sizeof(int) * FLAG_COUNT);
@@ -364,7 +368,7 @@ RelabelBox handle_relabel_box(lbm_handle* h) {
   b.plane = h->shape.plane;
   b.mpitch = mask_pitch(c.nx);
   b.label = h->label();
-  b.old = reinterpret_cast<int32_t*>(h->rho());  // idle outside initialisation
+  b.old = reinterpret_cast<int32_t*>(h->ws + h->L.old);
   b.owner = h->owner();
   b.sgn = h->sgn();
   b.open = h->open();

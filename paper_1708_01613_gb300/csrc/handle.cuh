@@ -11,7 +11,7 @@ namespace lbm {
 
 // Offsets of the slices of the caller's workspace.
 struct Layout {
-  size_t pops[2], rho, label, owner, mask, open, sgn, tiles, tile_list, gas_list, flags, partials,
+  size_t pops[2], rho, label, old, owner, mask, open, sgn, tiles, tile_list, gas_list, flags, partials,
       scalars, total;
   int nparts, ntiles;
 };
