@@ -174,13 +174,18 @@ int select_device(lbm_handle* h) {
   return LBM_OK;
 }
 
-int check_flags(lbm_handle* h) {
-  int f[3] = {0, 0, 0};
-  CUDA_TRY(h, cudaMemcpyAsync(f, h->flags(), sizeof(f), cudaMemcpyDeviceToHost, h->stream));
+// Reads the first n flags in one copy, waits, and reports the faults among them.
+int read_flags(lbm_handle* h, int* f, int n) {
+  CUDA_TRY(h, cudaMemcpyAsync(f, h->flags(), sizeof(int) * n, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   if (f[FLAG_NUMERIC]) return fail(h, LBM_ENUMERIC, "NaN/Inf or rho <= 0 met by the step kernel");
   if (f[FLAG_TIMEOUT]) return fail(h, LBM_ETIMEOUT, "a bounded labelling loop gave up");
   return LBM_OK;
+}
+
+int check_flags(lbm_handle* h) {
+  int f[2] = {0, 0};
+  return read_flags(h, f, 2);
 }
 
 int reset_state(lbm_handle* h) {
@@ -747,29 +752,26 @@ int lbm_bubble_stats(lbm_handle* h, lbm_stats* out, double* hist, int32_t nbins,
   // labels, areas and the tiles' sums in the idle population buffer (>= 18 bytes per cell)
   int32_t* lab = static_cast<int32_t*>(h->pops(1 - h->cur));
   int32_t* area = lab + h->N();
+  double* sums = reinterpret_cast<double*>(h->flags() + FLAG_SUMS);
   CUDA_TRY(h, launch_diag_stats(fp, (float)h->cfg.gas_threshold, lab, area, area + h->N(), h->flags(), h->partials(),
-                                h->L.nparts, h->scalars(), h->flags() + FLAG_HIST, hist ? nbins : 0, hist ? dmin : 1.0,
+                                h->L.nparts, sums, h->flags() + FLAG_HIST, hist ? nbins : 0, hist ? dmin : 1.0,
                                 hist ? dmax : 2.0, h->stream));
+  // sums, histogram, counts and faults come in one copy (each costs the host about 10 us)
+  int f[FLAG_COUNT];
+  if ((rc = read_flags(h, f, FLAG_COUNT))) return rc;
   double sc[4];
-  int hc[kMaxHistBins];
-  int opened = 0, merges = 0;
-  CUDA_TRY(h, cudaMemcpyAsync(sc, h->scalars(), sizeof(sc), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(hc, h->flags() + FLAG_HIST, sizeof(hc), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(&opened, h->flags() + FLAG_OPENED, sizeof(int), cudaMemcpyDeviceToHost,
-                              h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(&merges, h->flags() + FLAG_MERGES, sizeof(int), cudaMemcpyDeviceToHost,
-                              h->stream));
-  if ((rc = check_flags(h))) return rc;
+  memcpy(sc, f + FLAG_SUMS, sizeof(sc));
+  const int* hc = f + FLAG_HIST;
   double mass = sc[3];  // of the labelled component; two lattices are summed on their own
   if (h->comps() == 2 && (rc = lbm_mass(h, &mass))) return rc;
   memset(out, 0, sizeof(*out));
   out->step = h->t;
   out->n_bubbles = (int32_t)llround(sc[0]);
-  out->n_open = opened;
+  out->n_open = f[FLAG_OPENED];
   out->gas_fraction = sc[1] / (double)h->N();
   out->mean_eq_diameter = sc[0] > 0 ? sc[2] / sc[0] : 0.0;
   out->mass = mass;
-  out->n_merges = merges;
+  out->n_merges = f[FLAG_MERGES];
   if (hist)
     for (int b = 0; b < nbins; ++b) hist[b] = hc[b];
   return LBM_OK;
@@ -791,14 +793,20 @@ int lbm_bubble_areas(lbm_handle* h, int32_t capacity, int32_t* labels, double* a
   int* count = h->flags() + FLAG_HIST;  // the histogram slots serve as scratch here
   CUDA_TRY(h, launch_diag_areas(fp, (float)h->cfg.gas_threshold, lab, area, list, count,
                                 reinterpret_cast<char*>(lab) + align8(12 * N), h->flags(), h->stream));
-  int n = 0;
-  CUDA_TRY(h, cudaMemcpyAsync(&n, count, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  if ((rc = check_flags(h))) return rc;
+  // the first entries come along with their count, so a short list takes one wait
+  constexpr int kFirst = 1024;
+  const int ahead = (int)std::min<size_t>({(size_t)kFirst, (size_t)capacity, N / 2});
+  std::vector<int32_t> pairs(2 * (size_t)ahead);
+  if (ahead)
+    CUDA_TRY(h, cudaMemcpyAsync(pairs.data(), list, sizeof(int32_t) * pairs.size(), cudaMemcpyDeviceToHost, h->stream));
+  int f[FLAG_HIST + 1];
+  if ((rc = read_flags(h, f, FLAG_HIST + 1))) return rc;
+  const int n = f[FLAG_HIST];
   *n_out = n;
   if (n > capacity) return fail(h, LBM_EINVAL, "%d bubbles, capacity %d", n, capacity);
-  std::vector<int32_t> pairs(2 * (size_t)n);
-  if (n) {
-    CUDA_TRY(h, cudaMemcpyAsync(pairs.data(), list, sizeof(int32_t) * 2 * n, cudaMemcpyDeviceToHost, h->stream));
+  if (n > ahead) {
+    pairs.resize(2 * (size_t)n);
+    CUDA_TRY(h, cudaMemcpyAsync(pairs.data(), list, sizeof(int32_t) * pairs.size(), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   }
   std::vector<int> order(n);

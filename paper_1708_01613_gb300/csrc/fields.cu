@@ -14,6 +14,8 @@
 //    flags the tiles holding gas; the passes after it visit only those.
 #include <math.h>
 
+#include <algorithm>
+
 #include "labels.cuh"
 #include "pull.cuh"
 
@@ -49,12 +51,20 @@ __global__ void __launch_bounds__(kThreads) k_density(const FieldParams fp, floa
 }
 
 // --- populations: plane i of the incoming state, f_i(x) = B_i(x - e_i) ---
-// Four columns of kRows rows per thread. The source row's four columns start
+// Four columns of a few rows per thread. The source row's four columns start
 // at x - e_x: an aligned vector load, and the word beside it for a shifted
 // plane. Dense output rows of a width that is not a multiple of four are
-// written one value at a time. 8192^2, all planes: see the launcher's users;
-// a launch per plane with a division per cell took 2452 us (FP32) and 2330 us
-// (FP16), one value per thread in one launch 822 and 1707 us.
+// written one value at a time. Bound by HBM (FP32) and by bytes in flight
+// (16-bit words: 8192^2 with 1, 2, 4, 8 rows 2001, 1183, 811, 1060 us, FP32
+// 804, 772, 881, 1175). All planes of 8192^2 take 772 us (FP32, 6.3 TB/s) and
+// 811 us (FP16; 861 without the streaming hint, which costs FP32 nothing and
+// gives it nothing); a launch per plane with a division per cell took 2452 and
+// 2330 us.
+template <int S>
+constexpr int pop_rows() {
+  return S == LBM_F32 ? 2 : 4;
+}
+
 template <int S>
 __device__ __forceinline__ float4 load4(const typename Store<S>::T* q, int ex, float base) {
   if constexpr (S == LBM_F32) {
@@ -81,6 +91,7 @@ template <int S>
 __global__ void __launch_bounds__(kThreads) k_pops_out(const FieldParams fp, int plane0, bool vec,
                                                        float* __restrict__ out) {
   using T = typename Store<S>::T;
+  constexpr int ROWS = pop_rows<S>();
   const int nx = fp.nx, ny = fp.ny;
   const int x = 4 * (blockIdx.x * kThreads + threadIdx.x);
   if (x >= nx) return;
@@ -90,17 +101,18 @@ __global__ void __launch_bounds__(kThreads) k_pops_out(const FieldParams fp, int
   const T* p = static_cast<const T*>(fp.pops) + (size_t)i * fp.plane + x;
   float* o = out + (size_t)blockIdx.z * fp.N + x;
   const float base = fp.wref[i];
-  for (int yb = blockIdx.y * kRows; yb < ny; yb += gridDim.y * kRows) {
-    float4 v[kRows];
+  for (int yb = blockIdx.y * ROWS; yb < ny; yb += gridDim.y * ROWS) {
+    float4 v[ROWS];
 #pragma unroll
-    for (int r = 0; r < kRows; ++r)
+    for (int r = 0; r < ROWS; ++r)
       if (yb + r < ny) v[r] = load4<S>(p + (size_t)pull_wrap(yb + r - ey, ny) * fp.pitch, ex, base);
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) {
+    for (int r = 0; r < ROWS; ++r) {
       if (yb + r >= ny) continue;
       float* q = o + (size_t)(yb + r) * nx;
       if (vec) {
-        *reinterpret_cast<float4*>(q) = v[r];
+        if (S == LBM_F32) *reinterpret_cast<float4*>(q) = v[r];
+        else __stcs(reinterpret_cast<float4*>(q), v[r]);
       } else {
         q[0] = v[r].x;
         if (x + 1 < nx) q[1] = v[r].y;
@@ -525,7 +537,9 @@ cudaError_t launch_density(const FieldParams& fp, float* rho, cudaStream_t s) {
 
 cudaError_t launch_pops_out(const FieldParams& fp, int plane0, int planes, float* out, cudaStream_t s) {
   const bool vec = fp.nx % 4 == 0 && base16(out) && fp.N % 4 == 0;
-  const dim3 grid = row_grid((fp.nx + 3) / 4, fp.ny, planes);
+  const int rows = fp.storage == LBM_F32 ? pop_rows<LBM_F32>() : pop_rows<LBM_F16_DEV>();
+  dim3 grid = row_grid((fp.nx + 3) / 4, fp.ny, planes);
+  grid.y = std::min((fp.ny + rows - 1) / rows, 65535);
 #define CALL(S) k_pops_out<S><<<grid, kThreads, 0, s>>>(fp, plane0, vec, out)
   LBM_BY_STORAGE(fp.storage, CALL)
 #undef CALL

@@ -40,6 +40,7 @@ enum Flag : int {
   FLAG_DONE = 6,      // CTAs of that launch that have finished (0 between launches)
   FLAG_FILM = 7,      // tiles in the list of film tiles
   FLAG_MERGES = 8,    // coalescence events counted by the relabels since the last init
+  FLAG_SUMS = 16,     // four FP64 sums of the statistics
   FLAG_HIST = 64,     // 64 histogram counters
   FLAG_COUNT = 128
 };
