@@ -96,7 +96,7 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-TRAFFIC_SOURCES = {"step": ("step.cu", "lbm_internal.cuh", "tma.cuh"),
+TRAFFIC_SOURCES = {"step": ("step.cu", "tile.cu", "cellmath.cuh", "lbm_internal.cuh", "tma.cuh"),
                    "step2": ("step2.cu", "lbm_internal.cuh", "tma.cuh")}
 
 
@@ -291,7 +291,7 @@ def run_gpu(args, world, rank, local):
                 "peak_kind": f"{peak_kind} (copy bandwidth, MEASURED_PEAKS.json hbm_gbs)"
                 if peak_kind == "measured" else peak_kind,
                 "algorithmic_bytes_per_cell": bytes_cell,
-                "kernel": "k_step_dyn" if n % 16 == 0 else "k_step_strip",
+                "kernel": "k_step_tile" if storage == "f32" or n * n <= 30_000_000 else "k_step_dyn",
                 "kernel_ms_avg": round(kern_ms, 5),
                 "kernel_mlups": round(N / (kern_ms * 1e-3) / 1e6, 1),
                 "roofline_mlups": round(peak * 1e9 / bytes_cell / 1e6, 1)}

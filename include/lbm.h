@@ -187,13 +187,11 @@ int64_t lbm_kernel_launches(const lbm_handle* h);
 
 /* Selects the fused-step kernel: 0 = automatic, 1 = plain-load kernel (any
  * box), 2 = TMA-staged kernel with one cell per thread (nx % 16 == 0 and
- * nx >= 272), 3 = TMA-staged kernel with two cells per thread, one row
- * chunk per CTA (nx >= 16), 4 = the same with row chunks drawn by the
- * CTAs from a counter (nx >= 16). Variants 3 and 4 bulk-copy whole rows
- * when nx % 16 == 0, else each row's 16-byte-aligned interior, with the
- * unaligned head, tail and wrapped halo loaded plainly. Automatic picks 4
- * where the box allows (3 when the box has no more chunks than CTAs fit the
- * GPU), else 1. A variant the box does not allow returns LBM_ENOTSUP. All
+ * nx >= 272), 3 = TMA-staged kernel with two cells per thread, one row chunk per CTA
+ * (nx >= 16), 4 = the same with row chunks drawn by the CTAs from a counter
+ * (nx >= 16). Automatic takes the tile kernel, many steps of a small box in
+ * one launch where the call allows it, and 3 or 4 for the large boxes that
+ * they step faster. A variant the box does not allow returns LBM_ENOTSUP. All
  * variants compute the same operations in the same order and give bitwise
  * the same populations. The same handle must not be stepped by two streams
  * at once (variant 4 keeps its chunk counter in the handle's workspace). */
@@ -282,10 +280,9 @@ void lbm_destroy(lbm_handle* h);
 /* ---------------------------------------------------------------------
  * Batches: many boxes advanced together. Not in the paper; it serves runs
  * of many independent foam simulations on one GPU. Every step of a batch is
- * one persistent launch of the two-cell staged kernel over a list of work
- * items (box, column strip, row chunk) of all active boxes with nx % 16 == 0,
- * one of its unaligned-row variant over the other boxes of at least 16
- * columns, and one plain-load step per narrower box,
+ * one launch of the tile kernel over the tiles of all active boxes (very
+ * large 16-bit batches: of the two-cell staged kernel over column strips and
+ * row chunks, with one plain-load step per box narrower than 16 columns),
  * preceded, when a relabel is due, by each box's barrier pipeline and
  * followed, with the barrier, by the bounce-back across blocked edges;
  * blocks of steps are captured as CUDA graphs and replayed. Each box evolves

@@ -265,8 +265,8 @@ class Simulation:
             self._call("lbm_load_populations", C.c_void_p(a.ctypes.data), 0)
 
     def set_step_variant(self, variant: int) -> None:
-        """0 automatic, 1 plain loads, 2 one-cell staged, 3 two-cell staged,
-        4 two-cell staged with dynamically drawn row chunks (3 and 4 need nx % 16 == 0)."""
+        """0 automatic, 1 plain loads, 2 one-cell staged (nx % 16 == 0, nx >= 272), 3 two-cell staged,
+        4 two-cell staged with dynamically drawn row chunks (3 and 4: nx >= 16)."""
         self._call("lbm_set_step_variant", int(variant))
 
     def step(self, n: int = 1) -> None:
@@ -361,7 +361,7 @@ class Simulation:
 class Batch:
     """Several Simulation boxes advanced together (lbm_batch_*).
 
-    Every step is one persistent launch over all active boxes; blocks of a
+    Every step is one launch over all active boxes; blocks of a
     relabel period are replayed as CUDA graphs. Boxes evolve bitwise as they
     would alone. The workspace is a torch uint8 tensor owned by this object.
     """
