@@ -1,13 +1,15 @@
 // Batched time stepping of many boxes (C ABI lbm_batch_*, include/lbm.h).
 //
 // A batch advances several independent boxes together: every step is one
-// persistent launch of the two-cell staged kernel over a list of work items
-// (box, column strip, row chunk) that covers all active boxes, preceded, when
-// a relabel is due, by each box's barrier pipeline and followed, with the
-// barrier, by the bounce-back across the boxes' blocked edges. Blocks of K steps (K =
-// relabel period) are captured once as CUDA graphs and replayed. The strip
-// width and chunk height of the work items are picked by lbm_batch_tune,
-// which times the candidates on the batch itself. Per-cell arithmetic is the
+// launch of the tile kernel over the tiles of all active boxes (tile.cu) or,
+// above its range, one persistent launch of the two-cell staged kernel over a
+// list of work items (box, column strip, row chunk), preceded, when a relabel
+// is due, by the boxes' barrier pipeline and followed, with the barrier, by the
+// bounce-back across the boxes' blocked edges where the next step's pull does
+// not do it. Blocks of K steps (K = relabel period) are captured once as CUDA
+// graphs and replayed. The strip width and chunk height of the staged work
+// items are picked by lbm_batch_tune, which times the candidates on the batch
+// itself. Per-cell arithmetic is the
 // one of the single-box kernels, so every box evolves bitwise as it would
 // alone.
 #include <stdarg.h>

@@ -28,7 +28,8 @@
 //  - k_step_tma2: the same staging over 512-column strips with two cells per
 //    thread (march2); one static row chunk per CTA.
 //  - k_step_dyn: march2 over row chunks that the resident CTAs draw from a
-//    device counter (the automatic choice).
+//    device counter (the automatic choice for the boxes that the tile kernel,
+//    tile.cu, steps more slowly).
 //  - k_step_batch: march2 over work items (box, strip, row chunk) of many
 //    boxes in one launch (batch.cu).
 //
