@@ -817,12 +817,12 @@ cudaError_t launch_strip(const StepParams& p, cudaStream_t s) {
   return launch_chain(k_step_strip<S, MASKED, TAU_ONE>, dim3(gx, gy), dim3(block), 0, s, q);
 }
 
-// Variant 0 (automatic): the two-cell staged march over dynamically
-// scheduled row chunks (measured fastest for every storage: 8192^2 FP32 0.757
-// ms against 0.815 for the one-cell static kernel; boxes with no more chunks
-// than resident CTAs take the static split of variant 3), plain loads for
-// boxes of fewer than 16 columns; 1: plain loads; 2: one-cell staged; 3:
-// two-cell staged, one chunk per CTA; 4: two-cell staged, dynamic chunks.
+// Variant 0 (automatic): the tile kernel in its range (step_tiles; the two
+// times are in tile.cu), beyond it the two-cell staged march over dynamically
+// scheduled row chunks (8192^2 FP16 434 us against 485 in tiles; boxes with no
+// more chunks than resident CTAs take the static split of variant 3). 1: plain
+// loads; 2: one-cell staged; 3: two-cell staged, one chunk per CTA; 4: two-cell
+// staged, dynamic chunks; plain loads where the box does not allow these.
 template <int S, bool MASKED, bool TAU_ONE>
 cudaError_t launch_variant(const StepParams& p, cudaStream_t s) {
   const int v = p.force_generic;
