@@ -231,6 +231,7 @@ int upload(lbm_batch* b, const std::vector<int>& order = {}) {
     d.inv_rho0 = (float)(1.0 / h->cfg.rho0);
     d.rho_ref = (float)h->cfg.rho_ref;
     d.cur = h->cur;
+    d.tau_one = d.tau == 1.0f;
     b->base_cur[i] = h->cur;
     if (b->masked && handle_relabel_tiled(h)) {
       rboxes[i] = handle_relabel_box(h);

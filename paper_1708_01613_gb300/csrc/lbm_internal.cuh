@@ -208,7 +208,8 @@ struct BatchInst {
   long long plane;
   float tau, inv_tau, G, rho0, inv_rho0, rho_ref;
   int cur;              // buffer holding the state when parity == 0
-  int pad;
+  int tau_one;          // tau == 1 (not asked of tau in a kernel: the compiler then
+                        // folds tau F + j into an add and contracts it with F's product)
 };
 
 // One work item of a batched launch: columns x0 .. x0+width, rows y0 .. y1.

@@ -682,13 +682,13 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     p.inv_rho0 = in.inv_rho0;
     p.rho_ref = in.rho_ref;
     uint32_t worst = 0;
-    // full strips take the compile-time-width march (with tau != 1 the two
-    // inlined copies would spill at this kernel's register budget)
-    const bool ok = TAU_ONE && it.width == kBX2
-                        ? march2<S, MASKED, TAU_ONE, NSTAGE, TAU_ONE>(p, sm, it.x0, it.width, it.y0, it.y1,
-                                                                             gstage, worst)
-                        : march2<S, MASKED, TAU_ONE, NSTAGE, false>(p, sm, it.x0, it.width, it.y0, it.y1,
-                                                                         gstage, worst);
+    bool ok;
+    if (TAU_ONE && it.width == kBX2)  // full strips take the compile-time-width march
+      ok = march2<S, MASKED, TAU_ONE, NSTAGE, TAU_ONE>(p, sm, it.x0, it.width, it.y0, it.y1, gstage, worst);
+    else if (!TAU_ONE && in.tau_one)  // a tau = 1 box among others: the collision it takes alone
+      ok = march2<S, MASKED, true, NSTAGE, false>(p, sm, it.x0, it.width, it.y0, it.y1, gstage, worst);
+    else  // (with tau != 1 a third copy would spill at this kernel's register budget)
+      ok = march2<S, MASKED, TAU_ONE, NSTAGE, false>(p, sm, it.x0, it.width, it.y0, it.y1, gstage, worst);
     if (!ok) return;
     report_faults(worst, p.flags);
   }

@@ -334,6 +334,15 @@ __device__ __forceinline__ void batch_box(TileBox& b, const BatchInst& in, int p
   b.s.rho_ref = in.rho_ref;
 }
 
+// A batch holds boxes of any tau. One with a tau other than 1 in it runs the
+// kernels for TAU_ONE = false, where a tau = 1 box still takes the collision it
+// takes alone (f = feq; the blend f + (feq - f) rounds feq - f first).
+template <int S, bool MASKED, bool TAU_ONE, typename G>
+__device__ __forceinline__ void batch_tile(const TileBox& b, int one, int xo, int y0, int y1) {
+  if (!TAU_ONE && one) tile_step<S, MASKED, true, G>(b, xo, y0, y1);  // uniform over the CTA
+  else tile_step<S, MASKED, TAU_ONE, G>(b, xo, y0, y1);
+}
+
 // One item per CTA. The item and its box's descriptor are constant while the
 // launches that use them run, so they are read before the wait for the kernel
 // before.
@@ -344,7 +353,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
   const BatchItem it = items[reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x];
   TileBox b;
   batch_box(b, insts[it.inst], parity, pull_bounce, MASKED, sizeof(typename Store<S>::T));
-  tile_step<S, MASKED, TAU_ONE, G>(b, it.x0, it.y0, it.y1);
+  batch_tile<S, MASKED, TAU_ONE, G>(b, insts[it.inst].tau_one, it.x0, it.y0, it.y1);
 }
 
 // The same with the boxes as a kernel argument: a CTA finds its tile from its
@@ -364,7 +373,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
   const int gx = (in.nx + G::COLS - 1) / G::COLS, k = t - boxes.first[lo], y0 = k / gx * G::ROWS;
   TileBox b;
   batch_box(b, in, parity, pull_bounce, MASKED, sizeof(typename Store<S>::T));
-  tile_step<S, MASKED, TAU_ONE, G>(b, k % gx * G::COLS, y0, min(y0 + G::ROWS, in.ny));
+  batch_tile<S, MASKED, TAU_ONE, G>(b, in.tau_one, k % gx * G::COLS, y0, min(y0 + G::ROWS, in.ny));
 }
 
 // Every second step takes the tiles from the last to the first while the two
