@@ -225,8 +225,16 @@ __global__ void __launch_bounds__(kThreads) k_fields(const FieldParams fp, const
       for (int i = 1; i < Q; ++i) {
         float s = psi[ly + 4 * q + 1 + cy(i)][lx + 1 + cx(i)];
         if ((m >> (i - 1)) & 1u) s = psi_c;
-        sx += static_cast<float>(wq(i)) * s * cx(i);
-        sy += static_cast<float>(wq(i)) * s * cy(i);
+        // explicit roundings: left to the compiler, a component asked for
+        // without the other is contracted differently and rounds differently
+        if (i < 5) {
+          const float t = __fmul_rn(wqf(i), s);
+          sx = __fmaf_rn(t, (float)cx(i), sx);
+          sy = __fmaf_rn(t, (float)cy(i), sy);
+        } else {
+          sx = __fmaf_rn(wqf(i) * cx(i), s, sx);
+          sy = __fmaf_rn(wqf(i) * cy(i), s, sy);
+        }
       }
       const float g = -fp.G * psi_c;
       if (out.ux) out.ux[c] = (jx[q] + 0.5f * (g * sx)) / r;
