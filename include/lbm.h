@@ -207,16 +207,17 @@ int lbm_halted(const lbm_handle* h);
 size_t lbm_fields_bytes(const lbm_handle* h, uint32_t fields);
 
 /* Writes the selected fields of the current state to dst (host or device,
- * dst_bytes >= lbm_fields_bytes). LABEL is recomputed from the current
- * density; OWNER/MASK/OPEN are those of the last relabel. Synchronises. */
+ * dst_bytes >= lbm_fields_bytes), back to back in increasing bit order with no
+ * padding between them: what follows MASK or OPEN of an odd number of cells
+ * starts at an odd byte. LABEL is recomputed from the current density;
+ * OWNER/MASK/OPEN are those of the last relabel. Synchronises. */
 int lbm_read_fields(lbm_handle* h, uint32_t fields, void* dst, size_t dst_bytes,
                     int dst_is_device);
 
 /* The same with a destination of its own for each selected field: dsts[k]
  * takes the k-th selected field in increasing bit order (host pointers, or
- * device pointers with dst_is_device = 1; a float or int32 field needs 4-byte
- * alignment). RHO, UX, UY and P selected together come from one pass over the
- * populations. Synchronises. */
+ * device pointers with dst_is_device = 1; of any alignment). RHO, UX, UY and P
+ * selected together come from one pass over the populations. Synchronises. */
 int lbm_read_fields_each(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_device);
 
 /* FP64 sum of rho over the box (of both components with two), reduced in

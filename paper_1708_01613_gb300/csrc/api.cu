@@ -269,8 +269,10 @@ constexpr int kFieldCount = 10;
 
 // The selected fields (increasing bit order) into dsts. rho, u and p come
 // from one pass over the populations; nothing is computed that was not
-// selected. Host destinations are staged in the idle population buffer
-// (18 bytes per cell at least: rho, u and p take 16).
+// selected. Host destinations, and device destinations of values that are not
+// aligned for them (a selection packed behind one-byte fields of an odd number
+// of cells), are staged in the idle population buffer (18 bytes per cell at
+// least: rho, u and p take 16) and copied from there.
 int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_device) {
   int rc = select_device(h);
   if (rc) return rc;
@@ -279,6 +281,7 @@ int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_de
   char* stage = static_cast<char*>(h->pops(1 - h->cur));
   const cudaMemcpyKind d2x = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   void* dst[kFieldCount] = {};  // by bit index
+  auto direct = [&](const void* d) { return dst_is_device && reinterpret_cast<uintptr_t>(d) % 4 == 0; };
   int n = 0;
   for (int b = 0; b < kFieldCount; ++b)
     if (fields & (1u << b)) dst[b] = dsts[n++];
@@ -287,15 +290,14 @@ int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_de
     const int bits[5] = {0, 1, 2, 3, 9};  // rho, ux, uy, p, gas density
     float* f[5] = {};
     for (int k = 0; k < 5; ++k)
-      if (dst[bits[k]]) f[k] = static_cast<float*>(dst_is_device ? dst[bits[k]] : static_cast<void*>(stage + 4 * N * k));
+      if (dst[bits[k]]) f[k] = static_cast<float*>(direct(dst[bits[k]]) ? dst[bits[k]] : static_cast<void*>(stage + 4 * N * k));
     if (h->comps() == 2) {  // 144 bytes per cell of staging
       CUDA_TRY(h, launch_fields2(step2_params(h), f[0], f[4], f[1], f[2], f[3], h->stream));
     } else {
       CUDA_TRY(h, launch_fields(fp, h->mask(), FieldOuts{f[0], f[1], f[2], f[3]}, h->stream));
     }
-    if (!dst_is_device)
-      for (int k = 0; k < (h->comps() == 2 ? 5 : 4); ++k)
-        if (dst[bits[k]]) CUDA_TRY(h, cudaMemcpyAsync(dst[bits[k]], f[k], 4 * N, d2x, h->stream));
+    for (int k = 0; k < (h->comps() == 2 ? 5 : 4); ++k)
+      if (f[k] != dst[bits[k]]) CUDA_TRY(h, cudaMemcpyAsync(dst[bits[k]], f[k], 4 * N, d2x, h->stream));
   }
   if (dst[9] && h->comps() != 2) {
     if (dst_is_device) CUDA_TRY(h, cudaMemsetAsync(dst[9], 0, 4 * N, h->stream));
@@ -304,9 +306,9 @@ int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_de
   if (dst[4]) {
     // into scratch: the relabel pipeline's own labels stay those of the
     // last relabel (the coalescence count compares the next one with them)
-    int32_t* lab = static_cast<int32_t*>(dst_is_device ? dst[4] : static_cast<void*>(stage));
+    int32_t* lab = static_cast<int32_t*>(direct(dst[4]) ? dst[4] : static_cast<void*>(stage));
     CUDA_TRY(h, launch_diag_labels(fp, (float)h->cfg.gas_threshold, lab, stage + align8(4 * N), h->flags(), h->stream));
-    if (!dst_is_device) CUDA_TRY(h, cudaMemcpyAsync(dst[4], lab, 4 * N, d2x, h->stream));
+    if (lab != dst[4]) CUDA_TRY(h, cudaMemcpyAsync(dst[4], lab, 4 * N, d2x, h->stream));
   }
   const void* state[3] = {h->owner(), h->mask(), h->open()};
   for (int b = 5; b <= 7; ++b) {
@@ -326,7 +328,7 @@ int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_de
     char* out = static_cast<char*>(dst[8]);
     for (int k = 0; k < h->comps(); ++k, out += 4 * Q * N) {
       const FieldParams fk = component_params(h, k);
-      if (dst_is_device) {
+      if (direct(out)) {
         CUDA_TRY(h, launch_pops_out(fk, 0, Q, reinterpret_cast<float*>(out), h->stream));
         continue;
       }
