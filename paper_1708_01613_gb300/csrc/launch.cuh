@@ -7,6 +7,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -58,6 +59,40 @@ inline cudaError_t launch_cluster(void (*kern)(P...), int size, dim3 grid, dim3 
   c.attrs = attr;
   c.numAttrs = 2;
   return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
+// A kernel's permission for more than 48 KB of dynamic shared memory and its
+// occupancy belong to a device, so a launcher keeps them per device. Threads
+// that ask for the first time together both ask, and store the same number.
+class PerDevice {
+ public:
+  // *out = what ask(out) found (> 0) on the current device
+  template <typename F>
+  cudaError_t get(F ask, int* out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool kept = dev >= 0 && dev < kDevices;
+    if (kept && (*out = found_[dev].load(std::memory_order_acquire)) > 0) return cudaSuccess;
+    e = ask(out);
+    if (e == cudaSuccess && kept) found_[dev].store(*out, std::memory_order_release);
+    return e;
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::atomic<int> found_[kDevices] = {};
+};
+
+// CTAs of a kernel that one SM of the current device holds, after allowing the
+// kernel its dynamic shared memory there.
+template <typename... P>
+inline cudaError_t ctas_per_sm(void (*kern)(P...), int threads, size_t smem, int* out) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kern, threads, smem);
+  if (e == cudaSuccess && *out < 1) *out = 1;
+  return e;
 }
 
 // Whether the current device holds such a cluster (asked once per device and kernel).

@@ -725,15 +725,9 @@ cudaError_t launch_tma(const StepParams& p, cudaStream_t s) {
   constexpr int NS = tma_stages<S>();
   auto kern = k_step_tma<S, MASKED, TAU_ONE, NS, kTmaMinBlocks>;
   constexpr size_t smem = tma_smem_bytes_c<S, MASKED, NS>();
-  static int resident = 0;  // per instantiation
-  if (resident == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kTmaThreads, smem);
-    if (e != cudaSuccess) return e;
-    resident = occ > 0 ? occ : 1;
-  }
+  static PerDevice per_sm;  // per instantiation
+  int resident = 0;
+  LBM_TRY(per_sm.get([&](int* n) { return ctas_per_sm(kern, kTmaThreads, smem, n); }, &resident));
   int gx, gy, rows;
   tma_geometry(p.nx, p.ny, resident, &gx, &gy, &rows);
   StepParams q = p;
@@ -756,15 +750,9 @@ cudaError_t launch_tma2(const StepParams& p, cudaStream_t s) {
   // the relaxation blend (tau != 1) keeps both population sets live: fewer CTAs
   auto kern = k_step_tma2<S, MASKED, TAU_ONE, NS, tma2_min_blocks<S, TAU_ONE>()>;
   constexpr size_t smem = tma2_smem_bytes_c<S, MASKED, NS>();
-  static int resident = 0;  // per instantiation
-  if (resident == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kTmaThreads, smem);
-    if (e != cudaSuccess) return e;
-    resident = occ > 0 ? occ : 1;
-  }
+  static PerDevice per_sm;  // per instantiation
+  int resident = 0;
+  LBM_TRY(per_sm.get([&](int* n) { return ctas_per_sm(kern, kTmaThreads, smem, n); }, &resident));
   const int gx = (p.nx + kBX2 - 1) / kBX2;
   int g = resident * sm_count() / gx;
   if (g < 1) g = 1;
@@ -780,15 +768,10 @@ cudaError_t launch_dyn(const StepParams& p, cudaStream_t s) {
   constexpr int NS = tma2_stages<S>();
   auto kern = k_step_dyn<S, MASKED, TAU_ONE, NS, tma2_min_blocks<S, TAU_ONE>()>;
   constexpr size_t smem = tma2_smem_bytes_c<S, MASKED, NS>();
-  static int resident = 0;  // per instantiation: CTAs that fit the GPU at once
-  if (resident == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kTmaThreads, smem);
-    if (e != cudaSuccess) return e;
-    resident = (occ > 0 ? occ : 1) * sm_count();
-  }
+  static PerDevice per_sm;  // per instantiation
+  int resident = 0;         // CTAs that fit the GPU at once
+  LBM_TRY(per_sm.get([&](int* n) { return ctas_per_sm(kern, kTmaThreads, smem, n); }, &resident));
+  resident *= sm_count();
   const int gx = (p.nx + kBX2 - 1) / kBX2;
   // 48-row chunks (best at 8192^2: 4.5 waves of 608 CTAs for 16-bit
   // storage, 6 of 456 for FP32) unless they make fewer than four waves;
@@ -843,15 +826,14 @@ cudaError_t launch_typed(const StepParams& p, cudaStream_t s) {
 }  // namespace
 
 int device_sm_count() {
-  static int cached[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  if (cached[dev] == 0) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 152;
-    cached[dev] = n;
-  }
-  return cached[dev];
+  static PerDevice sms;
+  int n = 0;
+  auto ask = [](int* out) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? cudaDeviceGetAttribute(out, cudaDevAttrMultiProcessorCount, dev) : e;
+  };
+  return sms.get(ask, &n) == cudaSuccess && n > 0 ? n : 152;
 }
 
 void step_geometry(int nx, int ny, int* grid_x, int* grid_y, int* rows_per_chunk, int* block) {
@@ -877,15 +859,10 @@ struct BatchKernel {
   static constexpr int MINB = tma2_min_blocks<S, TAU_ONE>();
   static constexpr size_t SMEM = tma2_smem_bytes_c<S, MASKED, NS>();
   static int resident() {  // CTAs that fit the GPU at once
-    static int r = 0;
-    if (r == 0) {
-      auto kern = k_step_batch<S, MASKED, TAU_ONE, NS, MINB>;
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM) != cudaSuccess) return 0;
-      int occ = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kTmaThreads, SMEM) != cudaSuccess) return 0;
-      r = (occ > 0 ? occ : 1) * sm_count();
-    }
-    return r;
+    static PerDevice per_sm;
+    int n = 0;
+    auto ask = [](int* out) { return ctas_per_sm(k_step_batch<S, MASKED, TAU_ONE, NS, MINB>, kTmaThreads, SMEM, out); };
+    return per_sm.get(ask, &n) == cudaSuccess ? n * sm_count() : 0;
   }
   static cudaError_t launch(const BatchInst* insts, const BatchItem* items, int nitems, int* counters, int parity,
                             cudaStream_t s) {

@@ -443,17 +443,10 @@ cudaError_t launch_step2_tma(const Step2Params& p, cudaStream_t s) {
   constexpr int NS = 3, MINB = TAU_ONE ? 3 : 2;
   auto kern = k_step2_tma<MASKED, TAU_ONE, NS, MINB>;
   constexpr size_t smem = smem2c_bytes<MASKED, NS>();
-  static int resident = 0;  // per instantiation
-  if (resident == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0, dev = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads2C, smem);
-    if (e != cudaSuccess) return e;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return cudaErrorInvalidDevice;
-    resident = (occ > 0 ? occ : 1) * sms;
-  }
+  static PerDevice per_sm;  // per instantiation
+  int resident = 0;
+  LBM_TRY(per_sm.get([&](int* n) { return ctas_per_sm(kern, kThreads2C, smem, n); }, &resident));
+  resident *= device_sm_count();
   const int gx = (p.nx + kBX2C - 1) / kBX2C;
   // 48-row chunks when they make at least eight waves (8192^2: twelve),
   // else whole waves, at least four once one is exceeded (measured with 2
