@@ -16,6 +16,7 @@
 
 #include <algorithm>
 
+#include "cellmath.cuh"
 #include "labels.cuh"
 #include "pull.cuh"
 
@@ -244,34 +245,82 @@ __global__ void __launch_bounds__(kThreads) k_fields(const FieldParams fp, const
 }
 
 // --- FP64 sums of FP32 values ---
-// A running sum as an unevaluated pair s + e of FP32 values (Knuth's TwoSum:
-// s and the rounding error of every addition, exactly), handed to FP64 after a
-// few dozen values. FP64 adds run at 1/64 of the FP32 rate here: one per value
-// took 0.61 ms at 4096^2 (FP32 storage) where the bytes take 0.09 ms.
-struct Sum2 {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add(float b) {
-    const float t = __fadd_rn(s, b), z = __fsub_rn(t, s);
-    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(b, z)));
-    s = t;
+// A running sum as an unevaluated triple s + e + r of FP32 values: s takes the
+// values, e the rounding error of every addition to s and r that of every
+// addition to e, both exact (Knuth's TwoSum; the cascade is the K-fold summation
+// of Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26, 2005). Over n values it is
+// within n^3 2^-77 of the sum of their magnitudes, which for the few dozen
+// before FP64 takes over is less than the rounding of one FP64 addition. FP64
+// adds run at 1/64 of the FP32 rate here: one per value took 0.61 ms at 4096^2
+// (FP32 storage) where the bytes take 0.09 ms. With V = float2 two sums run side
+// by side in packed instructions (6.5 per value): the statistics of 4096^2 take
+// 236 us (FP32) and 235 (FP16, whose density pass they bound), those of 8192^2
+// 656 and 651; a pair s + e, which loses what e cannot hold, took 233, 202, 634
+// and 532. A sum that leaves the FP32
+// range or meets an infinity or NaN is no longer finite, and its values are
+// added in FP64 instead.
+template <typename V>
+struct Sum3 {
+  V s{}, e{}, r{};
+  // a + b rounded, and its error
+  static __device__ __forceinline__ V two_sum(V a, V b, V& err) {
+    using O = VOps<V>;
+    const V t = O::add(a, b), z = O::sub(t, a);
+    err = O::add(O::sub(a, O::sub(t, z)), O::sub(b, z));
+    return t;
   }
-  __device__ __forceinline__ void add(const Sum2& o) {
+  __device__ __forceinline__ void add_error(V q) {
+    V d;
+    e = two_sum(e, q, d);
+    r = VOps<V>::add(r, d);
+  }
+  __device__ __forceinline__ void add(V b) {
+    V q;
+    s = two_sum(s, b, q);
+    add_error(q);
+  }
+  __device__ __forceinline__ void add(const Sum3& o) {
     add(o.s);
-    e = __fadd_rn(e, o.e);
+    add_error(o.e);
+    r = VOps<V>::add(r, o.r);
   }
-  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
 };
 
-// Sum of a Sum2 over the warp, in a fixed order (valid in lane 0).
-__device__ __forceinline__ double warp_sum(Sum2 a) {
+__device__ __forceinline__ Sum3<float> both(const Sum3<float2>& p) {
+  Sum3<float> a, b;
+  a.s = p.s.x, a.e = p.e.x, a.r = p.r.x;
+  b.s = p.s.y, b.e = p.e.y, b.r = p.r.y;
+  a.add(b);
+  return a;
+}
+__device__ __forceinline__ bool finite(const Sum3<float>& a) { return fabsf(a.s) < INFINITY; }
+__device__ __forceinline__ double value(const Sum3<float>& a) { return (double)a.s + ((double)a.e + (double)a.r); }
+
+// Sum of a sum over the warp, in a fixed order (valid in lane 0).
+__device__ __forceinline__ Sum3<float> warp_sum(Sum3<float> a) {
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) {
-    Sum2 b;
+    Sum3<float> b;
     b.s = __shfl_down_sync(0xffffffffu, a.s, d);
     b.e = __shfl_down_sync(0xffffffffu, a.e, d);
+    b.r = __shfl_down_sync(0xffffffffu, a.r, d);
     a.add(b);
   }
-  return a.value();
+  return a;
+}
+
+// FP64 sum of the populations of the cells (x .. x + n, y).
+template <int S>
+__device__ __forceinline__ double cells_sum64(const FieldParams& fp, int x, int y, int n) {
+  using T = typename Store<S>::T;
+  double sum = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < Q; ++i) {
+    const T* row = static_cast<const T*>(fp.pops) + (size_t)i * fp.plane + (size_t)pull_wrap(y - cy(i), fp.ny) * fp.pitch;
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) sum += (double)Store<S>::load(row + (x + j - cx(i)), 0, fp.wref[i]);
+  }
+  return sum;
 }
 
 // --- fixed-order FP64 reductions ---
@@ -296,31 +345,48 @@ __device__ void block_reduce_store(double (&v)[NV], double* __restrict__ out) {
     for (int j = 0; j < NV; ++j) out[j * gridDim.x + blockIdx.x] = sh[j][0];
 }
 
-// Sum of all stored populations: rows of one plane after another, four rows'
-// values in flight per thread.
+// Sum of all stored populations: rows of one plane after another, eight
+// values of a row in flight per thread (8192^2 FP32 562 us, FP16 575; with the
+// four rows' 32 values loaded first 480 and 1043).
 template <int S>
-__global__ void __launch_bounds__(kThreads) k_mass_partial(const FieldParams fp, double* partials) {
+__global__ void __launch_bounds__(kThreads) k_mass_partial(const __grid_constant__ FieldParams fp, double* partials) {
   using T = typename Store<S>::T;
   const T* p = static_cast<const T*>(fp.pops);
   const long long rows = (long long)Q * fp.ny;
   double acc[1] = {0.0};
   for (long long r0 = (long long)blockIdx.x * kRows; r0 < rows; r0 += (long long)gridDim.x * kRows) {
     for (int xb = 0; xb < fp.nx; xb += 8 * kThreads) {
-      Sum2 a;
+      const int x = xb + threadIdx.x;
+      auto row_at = [&](int r, float& base) {  // column 0 of the r-th row, nullptr beyond the last
+        const long long row = r0 + r;
+        const int i = (int)(row / fp.ny);
+        base = fp.wref[i < Q ? i : 0];
+        return row < rows ? p + (size_t)i * fp.plane + (size_t)(row - (long long)i * fp.ny) * fp.pitch : nullptr;
+      };
+      Sum3<float2> pair;
 #pragma unroll
       for (int r = 0; r < kRows; ++r) {
-        const long long row = r0 + r;
-        if (row >= rows) break;
-        const int i = (int)(row / fp.ny);
-        const T* q = p + (size_t)i * fp.plane + (size_t)(row - (long long)i * fp.ny) * fp.pitch;
-        const float base = fp.wref[i];
+        float base, v[8];
+        const T* q = row_at(r, base);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int x = xb + k * kThreads + threadIdx.x;
-          if (x < fp.nx) a.add(Store<S>::load(q, (size_t)x, base));
+        for (int k = 0; k < 8; ++k)
+          v[k] = q && x + k * kThreads < fp.nx ? Store<S>::load(q, (size_t)(x + k * kThreads), base) : 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) pair.add(make_float2(v[k], v[k + 1]));
+      }
+      const Sum3<float> a = both(pair);
+      if (finite(a)) {
+        acc[0] += value(a);
+      } else {
+#pragma unroll 1
+        for (int r = 0; r < kRows; ++r) {
+          float base;
+          const T* q = row_at(r, base);
+#pragma unroll 1
+          for (int k = 0; q && k < 8 && x + k * kThreads < fp.nx; ++k)
+            acc[0] += (double)Store<S>::load(q, (size_t)(x + k * kThreads), base);
         }
       }
-      acc[0] += a.value();
     }
   }
   block_reduce_store<1>(acc, partials);
@@ -343,7 +409,7 @@ __global__ void __launch_bounds__(kThreads) k_sum_partials(const double* partial
 // flag per tile; with AREA the area slots of its gas cells cleared; with MASS
 // the FP64 sum of the tile's populations.
 template <int S, bool AREA, bool MASS>
-__global__ void __launch_bounds__(kTX / 4 * kTY) kd_label(const FieldParams fp, float threshold, bool vec4,
+__global__ void __launch_bounds__(kTX / 4 * kTY, MASS ? 16 : 0) kd_label(const __grid_constant__ FieldParams fp, float threshold, bool vec4,
                                                           int32_t* __restrict__ label, int32_t* __restrict__ area,
                                                           uint8_t* __restrict__ tile_gas, double* __restrict__ tile_mass,
                                                           int* __restrict__ flags) {
@@ -363,16 +429,20 @@ __global__ void __launch_bounds__(kTX / 4 * kTY) kd_label(const FieldParams fp, 
     gas[j] = in[j] && r[j] < threshold;
   }
   if (MASS) {
-    Sum2 a;
+    Sum3<float2> pair;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      if (in[0]) a.add(fa[i].x);
-      if (in[1]) a.add(fa[i].y);
-      if (in[2]) a.add(fb[i].x);
-      if (in[3]) a.add(fb[i].y);
+      pair.add(make_float2(in[0] ? fa[i].x : 0.f, in[1] ? fa[i].y : 0.f));
+      pair.add(make_float2(in[2] ? fb[i].x : 0.f, in[3] ? fb[i].y : 0.f));
     }
     __shared__ double wm[2];
-    const double v = warp_sum(a);
+    const Sum3<float> a = warp_sum(both(pair));
+    double v = value(a);
+    if (!__shfl_sync(0xffffffffu, finite(a), 0)) {
+      v = in[0] ? cells_sum64<S>(fp, x, y, min(4, nx - x)) : 0.0;
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+    }
     const int tid = threadIdx.y * (kTX / 4) + threadIdx.x;
     if ((tid & 31) == 0) wm[tid >> 5] = v;
     __syncthreads();
