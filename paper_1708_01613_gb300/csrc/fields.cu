@@ -248,17 +248,16 @@ __global__ void __launch_bounds__(kThreads) k_fields(const FieldParams fp, const
 // A running sum as an unevaluated triple s + e + r of FP32 values: s takes the
 // values, e the rounding error of every addition to s and r that of every
 // addition to e, both exact (Knuth's TwoSum; the cascade is the K-fold summation
-// of Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26, 2005). Over n values it is
-// within n^3 2^-77 of the sum of their magnitudes, which for the few dozen
-// before FP64 takes over is less than the rounding of one FP64 addition. FP64
-// adds run at 1/64 of the FP32 rate here: one per value took 0.61 ms at 4096^2
-// (FP32 storage) where the bytes take 0.09 ms. With V = float2 two sums run side
-// by side in packed instructions (6.5 per value): the statistics of 4096^2 take
-// 236 us (FP32) and 235 (FP16, whose density pass they bound), those of 8192^2
-// 656 and 651; a pair s + e, which loses what e cannot hold, took 233, 202, 634
-// and 532. A sum that leaves the FP32
-// range or meets an infinity or NaN is no longer finite, and its values are
-// added in FP64 instead.
+// of Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26, 2005). A chain of n
+// additions is within n^3 2^-72 of the sum of the magnitudes (n is 24 at most
+// here: 2^-58), less than the rounding of one FP64 addition. FP64 adds run at
+// 1/64 of the FP32 rate here: one per value took 0.61 ms at 4096^2 (FP32
+// storage) where the bytes take 0.09 ms. With V = float2 two sums run side by
+// side in packed instructions (6.5 per value): the statistics of 4096^2 take 236
+// us (FP32) and 235 (FP16, whose density pass they bound), those of 8192^2 656
+// and 651; a pair s + e, which loses what e cannot hold, took 233, 202, 634 and
+// 532. A sum that leaves the FP32 range or meets an infinity or NaN is no longer
+// finite, and its values are added in FP64 instead.
 template <typename V>
 struct Sum3 {
   V s{}, e{}, r{};
