@@ -43,10 +43,11 @@ __global__ void k_gas_census(const float* __restrict__ rho, long long N, float t
 }
 
 // The release is worked out in FP64 by nine lanes of each CTA that has cells
-// (by every thread it was the most of the kernel: FP64 runs at 1/64 of the
-// FP32 rate; 1024^2 with 3 % gas 11.5 us, now 4.1), while the cells' nine
-// loads, all issued before the first store, are on their way. The grid is what
-// the SMs hold (six CTAs): 8192^2 with 1.8 % gas 45 us, with two per SM 71.
+// (FP64 runs at 1/64 of the FP32 rate: 1024^2 with 3 % gas takes 3.1 us, with
+// the release worked out by every thread 11.5), while the cells' nine loads, all
+// issued before the first store, are on their way. Six CTAs per SM (five fit at
+// its 48 registers; capped to 40, with a spill, it is slower at every size):
+// 8192^2 with 1.8 % gas 39 us, 4096^2 9.3; two CTAs per SM 71 and 20.
 template <int S>
 __global__ void __launch_bounds__(kThreadsG) k_growth(typename Store<S>::T* pops, const int32_t* list, const int* count,
                                                       int nx, int pitch, long long plane, double rate, double budget,
@@ -54,20 +55,20 @@ __global__ void __launch_bounds__(kThreadsG) k_growth(typename Store<S>::T* pops
   __shared__ float add[Q];
   __shared__ int some;
   grid_begin();
-  const int n = *count, stride = gridDim.x * blockDim.x;
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = *count;
+  StridedIndex k{(int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x), n};
   if (blockIdx.x != 0 && (int)(blockIdx.x * blockDim.x) >= n) return;
   float f[Q];
   typename Store<S>::T* cell = pops;  // row of the cell, and its column
   int x = 0;
   auto fetch = [&]() {
-    const int c = list[k], y = c / nx;
+    const int c = list[k.at], y = c / nx;
     x = c - y * nx;
     cell = pops + (size_t)y * pitch;
 #pragma unroll
     for (int i = 0; i < Q; ++i) f[i] = Store<S>::raw(cell + (size_t)i * plane, x);
   };
-  if (k < n) fetch();
+  if (k.in()) fetch();
   if (threadIdx.x < Q) {
     const double before = released[parity];
     double release = 0.0;
@@ -76,17 +77,17 @@ __global__ void __launch_bounds__(kThreadsG) k_growth(typename Store<S>::T* pops
       release = rate < left ? rate : left;
       if (!(release > 0.0)) release = 0.0;
     }
-    if (k == 0) released[parity ^ 1] = before + release;
+    if (k.at == 0) released[parity ^ 1] = before + release;
     if (threadIdx.x == 0) some = release != 0.0;
     if (release != 0.0) add[threadIdx.x] = (float)(wq(threadIdx.x) * (release / (double)n));
   }
   __syncthreads();
   if (!some) return;
-  while (k < n) {
+  while (k.in()) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) put_cell(cell + (size_t)i * plane, x, nx, Store<S>::enc(__fadd_rn(f[i], add[i])));
-    k += stride;
-    if (k < n) fetch();
+    k.next();
+    if (k.in()) fetch();
   }
 }
 

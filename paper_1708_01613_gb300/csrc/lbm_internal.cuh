@@ -139,6 +139,15 @@ __device__ __forceinline__ void put_cell(T* row, int x, int nx, T v) {
   if (x >= nx - 2) row[x - nx] = v;
 }
 
+// The indices at, at + stride, ... below n of one thread of a grid; the last step
+// stops at n, because at + stride may be beyond 2^31 for a list of nearly 2^31
+// entries.
+struct StridedIndex {
+  int at, stride, n;
+  __host__ __device__ __forceinline__ bool in() const { return at < n; }
+  __host__ __device__ __forceinline__ void next() { at = at < n - stride ? at + stride : n; }
+};
+
 // Row-chunk height of a launch whose `resident` CTAs draw chunks (gx strips
 // by ny rows) from a counter. Chunks of max_rows rows give `items48` chunks;
 // if those make at least keep_waves waves (chunks / resident CTAs), the last
