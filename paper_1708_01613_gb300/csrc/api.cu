@@ -97,12 +97,6 @@ Layout layout_for(const lbm_config& c) {
   return L;
 }
 
-}  // namespace
-
-
-
-namespace {
-
 int fail(lbm_handle* h, int code, const char* fmt, ...) {
   if (h) {
     va_list ap;
@@ -346,16 +340,6 @@ int read_fields(lbm_handle* h, uint32_t fields, void* const* dsts, int dst_is_de
 }  // namespace
 
 namespace lbm {
-
-int handle_fail(lbm_handle* h, int code, const char* fmt, ...) {
-  if (h) {
-    va_list ap;
-    va_start(ap, fmt);
-    vsnprintf(h->err, sizeof(h->err), fmt, ap);
-    va_end(ap);
-  }
-  return code;
-}
 
 int handle_relabel(lbm_handle* h) { return relabel(h); }
 

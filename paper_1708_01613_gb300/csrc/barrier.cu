@@ -45,17 +45,10 @@ inline unsigned blocks_for(long long n, int threads = kThreads) {
 }
 
 // --- union-find labelling (min-root hooking: the root is the min index) ---
-__global__ void k_label_init(const float* __restrict__ rho, long long N, float th, int32_t* L) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-       c += (long long)gridDim.x * blockDim.x)
-    L[c] = rho[c] < th ? (int32_t)c : -1;
-}
-
-// Relabel variant of k_label_init: each new gas cell first parks its label of
-// the previous relabel in keep[c] (INT_MAX where it was liquid) for the
-// coalescence count; keep is the owner array, which the owner phase
-// rewrites afterwards.
-__global__ void k_label_init_keep(const float* __restrict__ rho, long long N, float th, int32_t* L,
+// Each new gas cell parks its label of the previous relabel in keep[c] (INT_MAX
+// where it was liquid) for the coalescence count; keep is the owner array, which
+// the owner phase rewrites afterwards.
+__global__ void k_label_init(const float* __restrict__ rho, long long N, float th, int32_t* L,
                                   int32_t* __restrict__ keep) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
        c += (long long)gridDim.x * blockDim.x) {
@@ -329,11 +322,10 @@ __global__ void k_bounce(T* __restrict__ pops, const uint8_t* __restrict__ mask,
 cudaError_t launch_labels(const FieldParams& fp, const float* rho, float threshold, int32_t* label,
                           int* flags, cudaStream_t s, int32_t* keep) {
   const unsigned b = blocks_for(fp.N);
-  if (keep) k_label_init_keep<<<b, kThreads, 0, s>>>(rho, fp.N, threshold, label, keep);
-  else k_label_init<<<b, kThreads, 0, s>>>(rho, fp.N, threshold, label);
+  k_label_init<<<b, kThreads, 0, s>>>(rho, fp.N, threshold, label, keep);
   k_label_union<<<b, kThreads, 0, s>>>(fp.nx, fp.ny, label, flags);
   k_label_flatten<<<b, kThreads, 0, s>>>(fp.N, label, flags);
-  if (keep) k_merge_count<<<b, kThreads, 0, s>>>(fp.N, label, keep, flags);
+  k_merge_count<<<b, kThreads, 0, s>>>(fp.N, label, keep, flags);
   return cudaGetLastError();
 }
 

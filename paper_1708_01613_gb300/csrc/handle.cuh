@@ -62,8 +62,6 @@ struct lbm_handle {
 
 namespace lbm {
 
-// Records a message on the handle and returns code.
-int handle_fail(lbm_handle* h, int code, const char* fmt, ...);
 // Enqueues the barrier pipeline on the handle's current populations.
 int handle_relabel(lbm_handle* h);
 // Synchronises the handle's stream and reports device-side faults.

@@ -56,12 +56,10 @@ struct Store<LBM_F32> {
   using T = float;
   static constexpr int bytes = 4;
   __device__ static __forceinline__ float load(const T* p, size_t i, float) { return __ldcg(p + i); }
-  __device__ static __forceinline__ float load_smem(const T* p, int i, float) { return p[i]; }
   __device__ static __forceinline__ T of(float v, float) { return v; }
   // raw stored value (FP32: the population itself)
   __device__ static __forceinline__ float raw(const T* p, size_t i) { return __ldcg(p + i); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return p[i]; }
-  __device__ static __forceinline__ void store_raw(T* p, size_t i, float v) { p[i] = v; }
   __device__ static __forceinline__ T enc(float v) { return v; }
 };
 
@@ -72,15 +70,11 @@ struct Store<LBM_F16_DEV> {
   __device__ static __forceinline__ float load(const T* p, size_t i, float base) {
     return __fadd_rn(base, __half2float(__ldcg(p + i)));
   }
-  __device__ static __forceinline__ float load_smem(const T* p, int i, float base) {
-    return __fadd_rn(base, __half2float(p[i]));
-  }
   // the stored word of a full population value
   __device__ static __forceinline__ T of(float v, float base) { return __float2half_rn(__fsub_rn(v, base)); }
   // raw stored value: the deviation g = f - w_i rho_ref
   __device__ static __forceinline__ float raw(const T* p, size_t i) { return __half2float(__ldcg(p + i)); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return __half2float(p[i]); }
-  __device__ static __forceinline__ void store_raw(T* p, size_t i, float g) { p[i] = __float2half_rn(g); }
   __device__ static __forceinline__ T enc(float g) { return __float2half_rn(g); }
 };
 
@@ -91,13 +85,9 @@ struct Store<LBM_BF16_DEV> {
   __device__ static __forceinline__ float load(const T* p, size_t i, float base) {
     return __fadd_rn(base, __bfloat162float(__ldcg(p + i)));
   }
-  __device__ static __forceinline__ float load_smem(const T* p, int i, float base) {
-    return __fadd_rn(base, __bfloat162float(p[i]));
-  }
   __device__ static __forceinline__ T of(float v, float base) { return __float2bfloat16_rn(__fsub_rn(v, base)); }
   __device__ static __forceinline__ float raw(const T* p, size_t i) { return __bfloat162float(__ldcg(p + i)); }
   __device__ static __forceinline__ float raw_smem(const T* p, int i) { return __bfloat162float(p[i]); }
-  __device__ static __forceinline__ void store_raw(T* p, size_t i, float g) { p[i] = __float2bfloat16_rn(g); }
   __device__ static __forceinline__ T enc(float g) { return __float2bfloat16_rn(g); }
 };
 
