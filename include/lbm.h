@@ -187,11 +187,12 @@ int64_t lbm_kernel_launches(const lbm_handle* h);
 
 /* Selects the fused-step kernel: 0 = automatic, 1 = plain-load kernel (any
  * box), 2 = TMA-staged kernel with one cell per thread (nx % 16 == 0 and
- * nx >= 272), 3 = TMA-staged kernel with two cells per thread, one row chunk per CTA
- * (nx >= 16), 4 = the same with row chunks drawn by the CTAs from a counter
+ * nx >= 272), 3 = TMA-staged kernel with two cells per thread, one row
+ * chunk per CTA (nx >= 16), 4 = the same with row chunks drawn by the CTAs from a counter
  * (nx >= 16). Automatic takes the tile kernel, many steps of a small box in
- * one launch where the call allows it, and 3 or 4 for the large boxes that
- * they step faster. A variant the box does not allow returns LBM_ENOTSUP. All
+ * one launch where the call allows it, and 3 or 4 for the boxes that they step
+ * faster (16-bit storage at tau = 1 above 30 M cells, FP32 at tau != 1 above
+ * 1.5 M). A variant the box does not allow returns LBM_ENOTSUP. All
  * variants compute the same operations in the same order and give bitwise
  * the same populations. The same handle must not be stepped by two streams
  * at once (variant 4 keeps its chunk counter in the handle's workspace). */
@@ -281,18 +282,20 @@ void lbm_destroy(lbm_handle* h);
 /* ---------------------------------------------------------------------
  * Batches: many boxes advanced together. Not in the paper; it serves runs
  * of many independent foam simulations on one GPU. Every step of a batch is
- * one launch of the tile kernel over the tiles of all active boxes (very
- * large 16-bit batches: of the two-cell staged kernel over column strips and
- * row chunks, with one plain-load step per box narrower than 16 columns),
+ * one launch of the tile kernel over the tiles of all active boxes (where
+ * they add up to more than 30 M cells with 16-bit storage and tau = 1 in all, or
+ * 1.5 M with FP32 and another tau among them: of the two-cell staged kernel over
+ * column strips and row chunks, with one plain-load step per box narrower than
+ * 16 columns),
  * preceded, when a relabel is due, by each box's barrier pipeline and
  * followed, with the barrier, by the bounce-back across blocked edges;
  * blocks of steps are captured as CUDA graphs and replayed. Each box evolves
  * bitwise as it would when stepped alone with lbm_step.
  *
  * Rules: all boxes share storage, barrier setting and relabel period, are
- * on one device, and do not stop on rupture. Boxes may be
- * at different step counts (each relabels when its own count is due). The batch works on a stream of its own (created by
- * lbm_batch_create; the legacy default stream cannot be captured into a
+ * on one device, and do not stop on rupture. Their tau may differ. Boxes may be
+ * at different step counts (each relabels when its own count is due). The batch
+ * works on a stream of its own (created by lbm_batch_create; the legacy default stream cannot be captured into a
  * graph), ordered by events after earlier work on the first box's stream,
  * and later work on that stream is ordered after each lbm_batch_step. A box
  * in a batch may not be stepped with lbm_step. */
@@ -308,15 +311,17 @@ size_t lbm_batch_workspace_bytes(lbm_handle* const* handles, int32_t n);
  * violations. */
 int lbm_batch_create(lbm_handle* const* handles, int32_t n, void* d_workspace, size_t bytes, lbm_batch** out);
 
-/* Work-item shape: strip width 256 or 512 columns, chunk height a multiple
- * of 8 rows. Changes invalidate the captured graphs. */
+/* Work-item shape of the staged kernel: strip width 256 or 512 columns, chunk
+ * height a multiple of 8 rows. It does not matter to batches that step in tiles,
+ * whose shape is fixed. Changes invalidate the captured graphs. */
 int lbm_batch_set_tiles(lbm_batch* b, int32_t strip_width, int32_t chunk_rows);
 int lbm_batch_get_tiles(const lbm_batch* b, int32_t* strip_width, int32_t* chunk_rows);
 
-/* Autotuner: times every (strip width, chunk height) candidate for
- * trial_steps steps on the batch itself and keeps the fastest. The boxes
+/* Autotuner of that shape: times every (strip width, chunk height) candidate
+ * for trial_steps steps on the batch itself and keeps the fastest. The boxes
  * advance by (trial_steps + 1) steps per candidate (10 candidates), as
- * ordinary steps (relabels included). */
+ * ordinary steps (relabels included), also where they step in tiles and the
+ * candidates do not differ; *best_ms_per_step is then the time of a step. */
 int lbm_batch_tune(lbm_batch* b, int32_t trial_steps, float* best_ms_per_step);
 
 /* 1 (default): replay captured graphs of whole relabel periods; 0: launch
@@ -331,7 +336,7 @@ int lbm_batch_step(lbm_batch* b, int64_t nsteps);
 
 /* Multi-rate steps: box i advances nsteps[i] steps (n = the batch's box
  * count; 0 = sits out; a switched-off box must get 0). Step j of the call is
- * one persistent launch over the boxes with nsteps[i] > j, so small boxes
+ * one launch over the boxes with nsteps[i] > j, so small boxes
  * can take many steps while large ones take few, as a server sharing the
  * GPU between requests wants. Relabels follow each box's own count. No
  * graphs are used; asynchronous, like lbm_batch_step. The batch's step

@@ -84,8 +84,8 @@ Layout layout_for(const lbm_config& c) {
     L.tiles = take(3 * (size_t)L.ntiles);  // gas, active, previous active
     L.tile_list = take(8 * (size_t)L.ntiles);  // tiles to visit, film tiles
     // scratch of the coalescence count: the density slice, idle during a
-    // relabel; two lattices have a slice of their own (a workspace of theirs
-    // holds more than two of one lattice, which callers may count on)
+    // relabel; two lattices have a slice of their own, which keeps a workspace of
+    // theirs larger than two of one lattice
     L.old = comps == 2 ? take(4 * N) : L.rho;
   }
   if (c.growth) L.gas_list = take(4 * N);

@@ -2,14 +2,15 @@
 //
 // A batch advances several independent boxes together: every step is one
 // launch of the tile kernel over the tiles of all active boxes (tile.cu) or,
-// above its range, one persistent launch of the two-cell staged kernel over a
-// list of work items (box, column strip, row chunk), preceded, when a relabel
+// above its range (tile_cells), one persistent launch of the two-cell staged
+// kernel over a list of work items (box, column strip, row chunk) and a plain step
+// for each box too narrow for it, preceded, when a relabel
 // is due, by the boxes' barrier pipeline and followed, with the barrier, by the
 // bounce-back across the boxes' blocked edges where the next step's pull does
 // not do it. Blocks of K steps (K = relabel period) are captured once as CUDA
 // graphs and replayed. The strip width and chunk height of the staged work
 // items are picked by lbm_batch_tune, which times the candidates on the batch
-// itself. Per-cell arithmetic is the
+// itself (tiles have one shape). Per-cell arithmetic is the
 // one of the single-box kernels, so every box evolves bitwise as it would
 // alone.
 #include <stdarg.h>
@@ -130,7 +131,12 @@ void build_tile_items(lbm_batch* b) {
 }
 
 // Whether the active boxes step with the tile kernel: it needs no
-// minimum width and beats the staged kernel while the state is small.
+// minimum width and beats the staged kernel while the state is small. The line is
+// the one for a lone box. Microseconds per step in tiles and staged (FP16, barrier,
+// relabel every 10 steps): 10 M cells in 16 boxes 96 and 123, 20 M in 16 176 and
+// 215, 30 M in 30 266 and 291, in 60 (more than the kernel argument holds) 305 and
+// 325. Beyond the line batches cross later than a lone box while their boxes fit
+// the argument: 45 M in 40 394 and 427, 64 M in 20 513 and 532, in 64 605 and 586.
 bool batch_tiles(const lbm_batch* b) {
   long long cells = 0;
   for (int i = 0; i < b->n; ++i) {

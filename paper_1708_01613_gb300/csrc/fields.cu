@@ -4,11 +4,10 @@
 // Every one of these is bound by memory, so each reads the populations once
 // and keeps what it needs on the chip:
 //  - the fields rho, u and p come from one pass that forms the densities of a
-//    tile with its halo in shared memory (a pass per field after a density
-//    pass read the populations up to eight times);
+//    tile with its halo in shared memory (4096^2 FP32 all four 190 us; a pass per
+//    field after a density pass takes 730);
 //  - all population planes are written by one launch, rows by grid
-//    coordinates (a launch per plane with a 64-bit modulo per cell ran at a
-//    third of the bandwidth);
+//    coordinates (no division per cell);
 //  - labels, areas, statistics and the mass come from one density pass over
 //    32 x 8 tiles that joins the gas cells of each tile in shared memory and
 //    flags the tiles holding gas; the passes after it visit only those.
@@ -59,8 +58,8 @@ __global__ void __launch_bounds__(kThreads) k_density(const FieldParams fp, floa
 // (16-bit words: 8192^2 with 1, 2, 4, 8 rows 2001, 1183, 811, 1060 us, FP32
 // 804, 772, 881, 1175). All planes of 8192^2 take 772 us (FP32, 6.3 TB/s) and
 // 811 us (FP16; 861 without the streaming hint, which costs FP32 nothing and
-// gives it nothing); a launch per plane with a division per cell took 2452 and
-// 2330 us.
+// gives it nothing); a launch per plane with a 64-bit division per cell takes 2452
+// and 2330 us.
 template <int S>
 constexpr int pop_rows() {
   return S == LBM_F32 ? 2 : 4;
@@ -125,7 +124,7 @@ __global__ void __launch_bounds__(kThreads) k_pops_out(const FieldParams fp, int
 }
 
 // --- mask: its rows without their padding, 16 cells per thread ---
-// (A 2-D copy by the copy engine path took 67 us at 8192^2, this 20.)
+// (8192^2 20 us; a 2-D device copy takes 67.)
 __global__ void __launch_bounds__(kThreads) k_mask_out(const uint8_t* __restrict__ mask, int mpitch, int nx, int ny,
                                                        int vec, uint8_t* __restrict__ out) {
   const int x = 16 * (blockIdx.x * kThreads + threadIdx.x);

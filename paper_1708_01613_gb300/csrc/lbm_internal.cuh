@@ -240,7 +240,7 @@ long long tile_cells(int storage, bool tau_one);
 // The boxes of a batch as a kernel argument, with the tiles of the boxes
 // before each (rows of tiles, top to bottom).
 struct BatchBoxes {
-  static constexpr int kMost = 40;  // 4 KB of arguments
+  static constexpr int kMost = 40;  // 4 KB; larger batches read the tables (32 KB of arguments would go)
   int n;
   int first[kMost];
   BatchInst in[kMost];

@@ -29,14 +29,14 @@
 // What bounds them: the label phase by its read of the populations (8192^2 FP32
 // 380 us, 6.4 TB/s; FP16 270 us); the others, over 10 % of the tiles of a box at
 // most, by the chain of dependent loads of each tile. Microseconds of the
-// phases 1 to 4 (the chain of eight launches this replaces, where a label pass
-// wrote densities and every listed tile went through five of them): 160 x 80
-// 5.1 + 4.6 + 8.0 + 2.9 (36 in all); 1024^2 FP16 8.3 + 6.2 + 11 + 3.6 (41);
-// 4096^2 FP32 104 + 9.2 + 37 + 3.3 (212); 8192^2 FP32 384 + 17 + 145 + 4 (705).
-// Walks to roots go side by side, and a cell's own state is loaded with the
-// window (one after the other: scan 6.4 and zone 9.1 us at 160 x 80).
-// A launch of its own for final labels and another for the mask over all listed
-// tiles, as before, cost 5 to 45 us and 4 to 100 us more.
+// phases 1 to 4, and in brackets of the whole with a launch for each of the eight
+// things they do (densities written and read, every listed tile visited by five
+// kernels): 160 x 80 5.1 + 4.6 + 8.0 + 2.9 (36); 1024^2 FP16 8.3 + 6.2 + 11 + 3.6
+// (41); 4096^2 FP32 104 + 9.2 + 37 + 3.3 (212); 8192^2 FP32 384 + 17 + 145 + 4
+// (705). Final labels in a launch of their own cost 5 to 45 us more, the mask over
+// all listed tiles in place of the film tiles 4 to 100 us. Walks to roots go side
+// by side, and a cell's own state is loaded with the window (one after the other:
+// scan 6.4 and zone 9.1 us at 160 x 80).
 #include <algorithm>
 
 #include "bounce.cuh"

@@ -1,6 +1,7 @@
 // Fused time step over tiles of a few rows: k_step_tile (one box) and
-// k_step_tile_batch (many). It serves every box but the largest of 16-bit
-// storage.
+// k_step_tile_batch (many). It serves every box but those that the staged march
+// of step.cu steps faster: above 30 M cells for 16-bit storage at tau = 1, above
+// 1.5 M for FP32 at tau != 1 (Tiles).
 //
 // A CTA takes a few rows of a strip of columns, one warp per row and one for
 // the halo row on either side. Each lane owns 2 P neighbouring cells;
