@@ -23,23 +23,20 @@ __device__ __forceinline__ float rcp_approx(float a) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
   return r;
 }
-// 1 / a for 0 < a < 2^102 by two Newton-Raphson steps r <- r + r (1 - a r) on
-// the hardware's approximation. The residual is exact in a fused operation, so
-// the second step rounds correctly (Markstein, IBM J. Res. Dev. 34, 1990): equal
-// to __frcp_rn for every such a, without its branch. The approximation flushes
-// subnormal arguments, so the steps run on a 2^24; powers of two change no
-// rounding, and the second one stands in for the sign. (Other densities are
-// faults, see report_faults.) The scale's multiplication costs the 16-bit step,
-// which issue bounds, 0.4 to 0.8 %: 8192^2 FP16 with its read-out 5578 -> 5598
-// us, 1024^2 FP16 742 -> 748.
-constexpr float kRecipScale = 16777216.0f;
+// 1 / rho for a density 0 < rho < 2^102, given as b = 2^24 rho, by two
+// Newton-Raphson steps r <- r + r (1 - b r) on the hardware's approximation. The
+// residual is exact in a fused operation, so the second step rounds correctly
+// (Markstein, IBM J. Res. Dev. 34, 1990): equal to __frcp_rn(rho) for every such
+// density, without its branch. The approximation flushes subnormal arguments, and
+// b is none; powers of two change no rounding, and the second one stands in for
+// the sign. (Other densities are faults, see report_faults.)
+constexpr float kRhoScale = 16777216.0f;
 
-__device__ __forceinline__ float recip(float a) {
-  const float b = __fmul_rn(a, kRecipScale);
+__device__ __forceinline__ float recip(float b) {
   float n = rcp_approx(-b);
   n = __fmaf_rn(n, __fmaf_rn(b, n, 1.0f), n);
   n = __fmaf_rn(n, __fmaf_rn(b, n, 1.0f), n);
-  return __fmul_rn(n, -kRecipScale);
+  return __fmul_rn(n, -kRhoScale);
 }
 
 template <typename V>
@@ -52,9 +49,9 @@ struct VOps<float> {
   static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
   static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
   static __device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-  static __device__ __forceinline__ float rcp(float a) { return recip(a); }
+  static __device__ __forceinline__ float rcp(float b) { return recip(b); }
   static __device__ __forceinline__ float ex2(float a) { return exp2_approx(a); }
-  static __device__ __forceinline__ void note(float rho, uint32_t& worst) { worst = __viaddmax_u32(__float_as_uint(rho), 0xffffffffu, worst); }
+  static __device__ __forceinline__ void note(float b, uint32_t& worst) { worst = __viaddmax_u32(__float_as_uint(b), 0xffffffffu, worst); }
 };
 
 // The pair type uses the packed two-wide FP32 instructions of sm_100 and
@@ -67,19 +64,19 @@ struct VOps<float2> {
   static __device__ __forceinline__ float2 sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
   static __device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
   static __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-  static __device__ __forceinline__ float2 rcp(float2 a) {
+  static __device__ __forceinline__ float2 rcp(float2 b) {
     // the negative of the reciprocal throughout: a sign flips no rounding,
-    // and 1 - a r is then one fused operation
-    const float2 one = set(1.f), b = mul(a, set(kRecipScale));
+    // and 1 - b r is then one fused operation
+    const float2 one = set(1.f);
     float2 n = make_float2(rcp_approx(-b.x), rcp_approx(-b.y));
     n = fma(n, fma(b, n, one), n);
     n = fma(n, fma(b, n, one), n);
-    return mul(n, set(-kRecipScale));
+    return mul(n, set(-kRhoScale));
   }
   static __device__ __forceinline__ float2 ex2(float2 a) { return make_float2(exp2_approx(a.x), exp2_approx(a.y)); }
-  static __device__ __forceinline__ void note(float2 rho, uint32_t& worst) {
-    VOps<float>::note(rho.x, worst);
-    VOps<float>::note(rho.y, worst);
+  static __device__ __forceinline__ void note(float2 b, uint32_t& worst) {
+    VOps<float>::note(b.x, worst);
+    VOps<float>::note(b.y, worst);
   }
 };
 
@@ -129,20 +126,24 @@ __device__ __forceinline__ void force_of(const V s[Q], V psi_c, float G, V& Fx, 
 // ones. With DEV the values are deviations from w_i rho_ref: j is unchanged
 // (sum e_i w_i = 0) and the equilibrium deviation is
 // w_i (rho - rho_ref - 1.5 rho u^2 + rho (3 e.u + 4.5 (e.u)^2)).
+// The density enters as b = 2^24 rho (recip); with DEV one fused operation gives
+// it from the summed deviations in place of rho, so the scale costs nothing there.
 template <bool TAU_ONE, bool DEV, typename V>
 __device__ __forceinline__ void collide(V f[Q], V rho_raw, V jx, V jy, V Fx, V Fy, const StepParams& p, uint32_t& worst) {
   using O = VOps<V>;
-  const V rho = full_rho<DEV>(rho_raw, p);
-  const V ir = O::rcp(rho);
+  const V b = DEV ? O::fma(rho_raw, O::set(kRhoScale), O::set(p.rho_ref * kRhoScale)) : O::mul(rho_raw, O::set(kRhoScale));
+  const V ir = O::rcp(b);
   // tau stays a multiplier at tau = 1 too: a packed add of the product gp s
   // (force_of) and j would be contracted to one rounding, unlike the scalar one
   const V tau = O::set(p.tau);
   const V ux = O::mul(O::fma(tau, Fx, jx), ir);
   const V uy = O::mul(O::fma(tau, Fy, jy), ir);
-  O::note(rho, worst);
+  O::note(b, worst);
   const V uu = O::fma(ux, ux, O::mul(uy, uy));
-  const V a = DEV ? O::fma(O::mul(O::set(-1.5f), rho), uu, rho_raw) : O::mul(rho, O::fma(O::set(-1.5f), uu, O::set(1.0f)));
-  const V r3 = O::mul(O::set(3.0f), rho), r45 = O::mul(O::set(4.5f), rho);
+  constexpr float k = DEV ? 1.0f / kRhoScale : 1.0f;
+  const V rho = DEV ? b : rho_raw;  // times k
+  const V a = DEV ? O::fma(O::mul(O::set(-1.5f * k), rho), uu, rho_raw) : O::mul(rho, O::fma(O::set(-1.5f), uu, O::set(1.0f)));
+  const V r3 = O::mul(O::set(3.0f * k), rho), r45 = O::mul(O::set(4.5f * k), rho);
   const V w1 = O::set(kW1), w5 = O::set(kW5);
   V feq[Q];
   feq[0] = O::mul(O::set(kW0), a);
@@ -173,11 +174,11 @@ __device__ __forceinline__ void collide(V f[Q], V rho_raw, V jx, V jy, V Fx, V F
   for (int i = 0; i < Q; ++i) f[i] = TAU_ONE ? feq[i] : O::fma(O::sub(feq[i], f[i]), om, f[i]);
 }
 
-// A step kernel tracks `worst`, the largest bits(rho) - 1 (as unsigned) of the
-// densities it collided: a density that is not in (0, 1e30) - zero, negative,
-// NaN or infinite - has the largest values, at one operation per cell.
+// A step kernel tracks `worst`, the largest bits(b) - 1 (as unsigned) of the
+// scaled densities b it collided: a density that is not in (0, 1e30) - zero,
+// negative, NaN or infinite - has the largest values, at one operation per cell.
 __device__ __forceinline__ void report_faults(uint32_t worst, int* flags) {
-  if (worst >= __float_as_uint(1e30f) - 1u) atomicOr(flags + FLAG_NUMERIC, 1);
+  if (worst >= __float_as_uint(1e30f * kRhoScale) - 1u) atomicOr(flags + FLAG_NUMERIC, 1);
 }
 
 }  // namespace

@@ -20,8 +20,8 @@ __global__ void k_recip(unsigned lo, unsigned hi, unsigned long long* bad) {
   for (unsigned long long b = lo + blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; b < hi;
        b += (unsigned long long)gridDim.x * blockDim.x) {
     const float a = __uint_as_float((unsigned)b), c = __uint_as_float((unsigned)(b ^ 1));  // a neighbour beside it
-    const float2 p = VOps<float2>::rcp(make_float2(a, c));
-    n += __float_as_uint(recip(a)) != __float_as_uint(__frcp_rn(a));
+    const float2 p = VOps<float2>::rcp(make_float2(__fmul_rn(a, kRhoScale), __fmul_rn(c, kRhoScale)));
+    n += __float_as_uint(recip(__fmul_rn(a, kRhoScale))) != __float_as_uint(__frcp_rn(a));
     n += __float_as_uint(p.x) != __float_as_uint(__frcp_rn(a));
     n += c > 0.f && __float_as_uint(p.y) != __float_as_uint(__frcp_rn(c));
   }
