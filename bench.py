@@ -474,7 +474,7 @@ def run_served(args, dev, world, rank, capacity_ups):
 def run_batched(args, dev, world, rank):
     """64 independent boxes of mixed size (sides 256-2048 log-uniform, 5-200
     bubbles, 1k-20k steps each, FP16-deviation storage, barrier on, K = 10):
-    one batch (persistent launch per step, graphs, autotuned tiles) against the
+    one batch (one launch per step, graphs, tuned work items) against the
     same boxes stepped one after another with lbm_step. Both time exactly
     sum_i cells_i * steps_i updates; `step_scale` shrinks all step counts."""
     import torch
